@@ -50,7 +50,7 @@ struct HostCells3 {
 };
 int64_t build_cells_3d(int64_t n, const double *x, const double *R, const double *lo,
                        const double *hi, const int32_t *rowptr, const int32_t *col, HostCells3 &out);
-// Row tiles of the TF32 tensor-core L-apply (tiles.cpp): rows in the spatial order, the
+// Row tiles of the batched L-apply (tiles.cpp): Morton-consecutive rows, the
 // halo (union of their columns) and sliced-ELL record slots.
 struct TileLayout {
     int rows_per_tile = 0;
@@ -68,8 +68,6 @@ struct TileLayout {
 // order[n]: the rows in tile order.  Returns the number of record slots.
 int64_t build_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, const int32_t *order, int rows_per_tile,
                     int width_multiple, TileLayout &out);
-// Spatial order of the points (order.cpp): aligned runs of 2, 4, .. 64 are compact boxes.
-void spatial_order(int64_t n, int dim, const double *x, int32_t *order);
 // Reference rules (quadrature.cpp).
 void gauss_jacobi_newton(int n, double a, double b, double *t, double *w);
 void triangle_rule(int n1d, double *xi /*2*n1d^2*/, double *w);
@@ -191,11 +189,11 @@ struct mlpg_ctx {
     int32_t *rowidx = nullptr;  // [nnz] row of each pattern entry
     double *abc = nullptr;      // [3][n] MS partial products
 
-    // block-Jacobi preconditioner: blocks of kBlockPts points in the spatial order
+    // block-Jacobi preconditioner: Morton-ordered blocks of kBlockPts points
     int64_t nblk = 0;
     int32_t *bmember = nullptr; // [nblk * kBlockPts] point of each block slot (-1: empty)
     int32_t *bof = nullptr;     // [n] block * kBlockPts + slot of each point
-    std::vector<int32_t> h_order;  // [n] points in the spatial order (host)
+    std::vector<int32_t> h_order;  // [n] points in Morton order (host)
 
     // row tiles of the FP32 L-apply (tiles.cpp), used when m % 4 == 0
     int tile_rows = 0, tile_chunk = 0, tile_dpt = 0, tile_xs = 0;  // rows per tile, directions per CTA, per thread, smem row stride

@@ -7,7 +7,7 @@
 // every few Arnoldi steps.  Orthogonalisation is classical Gram-Schmidt
 // applied twice (CGS2) in FP64, or once in the FP32 correction solves (16-byte
 // vectorised passes); block sums are formed in FP64 whatever the vector type.
-// Right preconditioning by the block-Jacobi inverses (blocks of 16 spatially ordered points)
+// Right preconditioning by the block-Jacobi inverses (16-point Morton blocks)
 // of each L_m.
 //
 // The same engine with M = 1 runs the scattering iteration on the

@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(256) k_faces32(int64_t nbr, int m, int tm_log2
 
 // ---------------------------------------------------------------------------
 // Row tiles (m % 4 == 0), shared by the CUDA-core and tensor-core tile
-// kernels.  A tile is TR rows in the spatial order; its halo is the sorted union
+// kernels.  A tile is TR Morton-consecutive rows; its halo is the sorted union
 // of their columns.  One CTA per (row tile, direction chunk) stages the halo
 // rows of X (mc of the m directions) in shared memory once, so a neighbour
 // row shared by several rows of the tile is read from HBM once per tile.  The
@@ -858,7 +858,7 @@ __global__ void k_interp_apply(int64_t n, const int32_t *__restrict__ rowptr, co
 
 
 // ---------------------------------------------------------------------------
-// Block-Jacobi preconditioner.  Points are grouped into spatially ordered blocks
+// Block-Jacobi preconditioner.  Points are grouped into Morton-ordered blocks
 // of B = MLPG_BLOCK_PTS; for every (block, direction) the dense B x B diagonal
 // block of L_m is inverted (Gauss-Jordan with partial pivoting, FP32, one warp;
 // lane l owns column l of the augmented [A | I]).  The inverse is stored
@@ -1336,7 +1336,7 @@ __global__ void k_diff_values(int64_t n, int64_t nnz, double kappa, const int32_
     }
 }
 
-// Inverse of the diagonal block (MLPG_BLOCK_PTS ordered points) of one FP64
+// Inverse of the diagonal block (MLPG_BLOCK_PTS Morton points) of one FP64
 // operator on the pattern: one warp per block, Gauss-Jordan with partial
 // pivoting on [A | I] in shared memory, lane l owning column l.
 __global__ void __launch_bounds__(256) k_block_inv64(int64_t nblk, const int32_t *__restrict__ rowptr,
@@ -2081,17 +2081,32 @@ mlpg_status apply_prec(mlpg_ctx *ctx, T *v, T *z, const double *sc) {
 template mlpg_status apply_prec<double>(mlpg_ctx *, double *, double *, const double *);
 template mlpg_status apply_prec<float>(mlpg_ctx *, float *, float *, const double *);
 
-// Spatial order of the points (order.cpp; host, once per point set) cut into blocks of
+// Morton order of the points (host, once per point set) cut into blocks of
 // MLPG_BLOCK_PTS consecutive points.
 mlpg_status build_blocks(mlpg_ctx *ctx) {
     const int64_t n = ctx->n;
+    const int d = ctx->dim;
+    std::vector<std::pair<uint64_t, int32_t>> key(n);
+    for (int64_t i = 0; i < n; ++i) {
+        uint64_t code = 0;
+        uint32_t qv[3] = {0, 0, 0};
+        for (int a = 0; a < d; ++a) {
+            double t = (ctx->h_x[i * d + a] - ctx->opt.lo[a]) / (ctx->opt.hi[a] - ctx->opt.lo[a]);
+            t = t < 0 ? 0 : (t > 1 ? 1 : t);
+            qv[a] = (uint32_t)(t * 1048575.0);
+        }
+        for (int b = 19; b >= 0; --b)
+            for (int a = d - 1; a >= 0; --a) code = (code << 1) | ((qv[a] >> b) & 1u);
+        key[i] = {code, (int32_t)i};
+    }
+    std::sort(key.begin(), key.end());
     ctx->nblk = (n + kB - 1) / kB;
     std::vector<int32_t> member(ctx->nblk * kB, -1), bof(n);
     ctx->h_order.resize(n);
-    spatial_order(n, ctx->dim, ctx->h_x.data(), ctx->h_order.data());
     for (int64_t r = 0; r < n; ++r) {
-        member[r] = ctx->h_order[r];
-        bof[ctx->h_order[r]] = (int32_t)r;
+        member[r] = key[r].second;
+        bof[key[r].second] = (int32_t)r;
+        ctx->h_order[r] = key[r].second;
     }
     MLPG_TRY(dalloc(ctx, &ctx->bmember, ctx->nblk * kB));
     MLPG_TRY(dalloc(ctx, &ctx->bof, n));

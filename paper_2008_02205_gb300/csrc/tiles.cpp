@@ -1,6 +1,6 @@
 // Row tiles of the batched transport operator apply (host, once per point set).
 //
-// The rows of the overlap pattern are taken in a spatial order (order.cpp) of their
+// The rows of the overlap pattern are taken in the Morton order of their
 // points and cut into tiles of `rows_per_tile` consecutive rows, so that the
 // rows of one tile are close in space and share most of their overlap
 // partners.  For every tile:
