@@ -79,12 +79,13 @@ typedef struct {
                               neighbours, e.g. extent 2.5-3 point spacings); 3D: 0 or 1;
                               default 1 */
     void *stream;          /* cudaStream_t to run on; NULL = a stream owned by the library */
-    int apply_kernel;      /* MLPG_MIXED batched L-apply: 0 = automatic (m % 4 == 0: row tiles with a
-                              staged halo when that takes at most two direction chunks, else row
-                              tiles in gather mode; otherwise row teams), 1 = one team of
+    int apply_kernel;      /* MLPG_MIXED batched L-apply: 0 = automatic (2D: row tiles with a staged halo when
+                              that takes at most two direction chunks, else row tiles in gather mode; 3D:
+                              gather mode; row teams for what these do not take), 1 = one team of
                               direction lanes per row gathering X through L1, 2 = row tiles with the
-                              tile's neighbour rows staged in shared memory (m % 4 == 0), 3 = the
-                              same tiles with the combination of the base arrays on tensor cores
+                              tile's neighbour rows staged in shared memory (m % 4 == 0; the automatic
+                              choice uses them for any m), 3 = row
+                              tiles with the combination of the base arrays on tensor cores
                               (TF32 split in high and low parts: FP32 accuracy; m % 8 == 0),
                               4 = row tiles with only the operator records staged and X read
                               from global memory (L2) per entry: no halo in shared memory, so a
@@ -92,10 +93,11 @@ typedef struct {
                               e.g. 3D, whose halos leave room for few directions per chunk);
                               default 0 */
     int tile_rows;         /* row tiles: rows per tile, 32 or 64 (apply_kernel 2, 3), 4, 8, 16 or
-                              32 (apply_kernel 4); 0 = 64, or in gather mode the most rows that
-                              keep a CTA at or below 320 threads */
-    int tile_dpt;          /* row tiles: directions per thread, 4 or 8 (must divide m); 0 = 8 when
-                              m % 8 == 0 with a staged halo, else 4 */
+                              32 (apply_kernel 4); 0 = by the problem's size (automatic choice), 64, or
+                              in gather mode the most rows that keep a CTA at or below 320 (row,
+                              direction group) tasks */
+    int tile_dpt;          /* row tiles: directions per thread, 4 or 8 (must divide m); 0 = 4, with an
+                              explicit apply_kernel 2 or 3 8 when m % 8 == 0 */
     int outer_precond;     /* outer GMRES on Phi: 0 = none (the paper's), 1 = DSA-like diffusion
                               correction, right preconditioner I + C^-1 Ms with the P1-diffusion
                               operator C = diag(1/(3 sigma_t,i)) sum_a K_aa + kappa M0 + Mt - Ms

@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 SO = os.path.join(HERE, "libmlpg.so")
 SOURCES = ["api.cu", "neighbors.cu", "assemble.cu", "assemble3d.cu", "cells2d.cu", "operators.cu", "krylov.cu", "noalloc.cu", "geometry.cpp",
-           "quadrature.cpp", "tiles.cpp", "cells3d.cu"]
+           "quadrature.cpp", "tiles.cpp", "order.cpp", "cells3d.cu"]
 # per-file flags: the device 3D cell builder rounds like the host builder (no contraction)
 EXTRA = {"cells3d.cu": ["--fmad=false"]}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

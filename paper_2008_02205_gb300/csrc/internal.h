@@ -50,7 +50,7 @@ struct HostCells3 {
 };
 int64_t build_cells_3d(int64_t n, const double *x, const double *R, const double *lo,
                        const double *hi, const int32_t *rowptr, const int32_t *col, HostCells3 &out);
-// Row tiles of the batched L-apply (tiles.cpp): Morton-consecutive rows, the
+// Row tiles of the tensor-core L-apply (tiles.cpp): consecutive rows of the spatial order, the
 // halo (union of their columns) and sliced-ELL record slots.
 struct TileLayout {
     int rows_per_tile = 0;
@@ -68,6 +68,25 @@ struct TileLayout {
 // order[n]: the rows in tile order.  Returns the number of record slots.
 int64_t build_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, const int32_t *order, int rows_per_tile,
                     int width_multiple, TileLayout &out);
+// Spatial order of the points (order.cpp): aligned runs of 2, 4, .. 64 are compact boxes.
+void spatial_order(int64_t n, int dim, const double *x, int32_t *order);
+// Row tiles of row pairs (tiles.cpp): one slot per union column of two rows.
+struct PairTileLayout {
+    int rows_per_tile = 0;
+    int64_t ntile = 0;
+    std::vector<int64_t> base;    // ntile + 1: first slot of each tile
+    std::vector<int32_t> width;   // ntile: slots per pair (longest union of the tile, rounded up)
+    std::vector<int32_t> row;     // ntile * rows_per_tile: row of each row slot, -1 past n
+    std::vector<int32_t> plen;    // ntile * rows_per_tile / 2: union length of each pair
+    std::vector<int64_t> hptr;    // ntile + 1: halo ranges in hcol (empty without a halo)
+    std::vector<int32_t> hcol;    // halo columns, sorted within each tile
+    std::vector<int32_t> perm0, perm1;   // slot -> pattern entry of the pair's first / second row, or -1
+    std::vector<int32_t> lcol;    // slot -> halo index of its column (the column itself without a halo)
+    int64_t max_halo = 0;
+    int32_t max_width = 0;
+};
+int64_t build_pair_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, const int32_t *order,
+                         int rows_per_tile, int width_multiple, bool with_halo, PairTileLayout &out);
 // Reference rules (quadrature.cpp).
 void gauss_jacobi_newton(int n, double a, double b, double *t, double *w);
 void triangle_rule(int n1d, double *xi /*2*n1d^2*/, double *w);
@@ -193,10 +212,11 @@ struct mlpg_ctx {
     int64_t nblk = 0;
     int32_t *bmember = nullptr; // [nblk * kBlockPts] point of each block slot (-1: empty)
     int32_t *bof = nullptr;     // [n] block * kBlockPts + slot of each point
-    std::vector<int32_t> h_order;  // [n] points in Morton order (host)
+    std::vector<int32_t> h_order;  // [n] points in the spatial order of the row tiles (host)
 
-    // row tiles of the FP32 L-apply (tiles.cpp), used when m % 4 == 0
+    // row tiles of the FP32 L-apply (tiles.cpp)
     int tile_rows = 0, tile_chunk = 0, tile_dpt = 0, tile_xs = 0;  // rows per tile, directions per CTA, per thread, smem row stride
+    int tile_ks = 1;            // warp groups that share a tile's slots
     bool tile_mma = false;      // the tensor-core variant of the tiled apply (apply_kernel 3)
     bool tile_gather = false;   // tiles with X read from global memory, no staged halo (apply_kernel 4)
     int64_t ntile = 0, nslot = 0;
@@ -204,10 +224,11 @@ struct mlpg_ctx {
     int tile_xs_f4 = 0;         // float4 words of the staged halo (the record stages follow)
     int64_t tile_max_halo = 0;  // largest halo of a tile
     int *d_tile_err = nullptr;  // set by a tile-kernel wait that gave up (bounded waits)
+    int32_t *t_head = nullptr;   // [ntile][4]: first slot, slots per pair, halo range (row pairs)
     int32_t *t_base = nullptr, *t_width = nullptr, *t_row = nullptr, *t_hptr = nullptr, *t_hcol = nullptr;
-    int32_t *t_perm = nullptr, *t_lcol = nullptr;
+    int32_t *t_perm = nullptr, *t_perm1 = nullptr, *t_lcol = nullptr, *t_plen = nullptr;   // t_perm1, t_plen: row pairs
     int32_t *t_bhalo = nullptr;  // [nb]: halo offset (index x tile_xs) of each boundary-segment entry's column
-    float *t_rec = nullptr;     // [nslot][rec words]: the base-array values of each slot, then its halo index
+    float *t_rec = nullptr;     // the base-array values of each slot and its halo index (per slot, or per stage of slots)
     float *Pinv = nullptr;      // [nblk][kBlockPts][kBlockPts][m] inverse diagonal blocks of L_m
     uint16_t *Pinv16 = nullptr; // same, FP16 bits scaled by Pscale^-1 (mixed mode), or null
     float *Pscale = nullptr;    // [nblk][m] power-of-two decode factor of each FP16 block

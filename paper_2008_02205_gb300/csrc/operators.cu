@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(256) k_faces32(int64_t nbr, int m, int tm_log2
 
 // ---------------------------------------------------------------------------
 // Row tiles (m % 4 == 0), shared by the CUDA-core and tensor-core tile
-// kernels.  A tile is TR Morton-consecutive rows; its halo is the sorted union
+// kernels.  A tile is TR rows in the spatial order; its halo is the sorted union
 // of their columns.  One CTA per (row tile, direction chunk) stages the halo
 // rows of X (mc of the m directions) in shared memory once, so a neighbour
 // row shared by several rows of the tile is read from HBM once per tile.  The
@@ -480,19 +480,13 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-constexpr int kRecK = 4;        // record pipeline: entries (k steps) per stage
-constexpr int kRecKGather = 8;  // ... in gather mode (more entries' loads in flight between barriers)
-__host__ __device__ constexpr int rec_k(bool gather) { return gather ? kRecKGather : kRecK; }
+constexpr int kRecK = 4;        // record pipeline of the tensor-core kernel: entries (k steps) per stage
 constexpr int kRecStages = 4;   // record pipeline: stages in flight
-// direction groups per row: threads per CTA = rows per tile x groups (<= 640)
-// (gather mode: at most 320 threads, so that two CTAs of the 4-direction kernel fit an SM
-// under its register bound; measured 3.32 against 3.96 ms at 40^3 with 272 directions)
+// direction groups per row tile (the chunk): at most 640 threads' worth of (row, group) tasks, 320 with
+// eight directions each or in gather mode; the row-pair kernel runs half as many threads
 __host__ __device__ constexpr int tile_max_groups(int tr, int dpt, bool gather = false) {
     return (gather || dpt == 8 ? 320 : 640) / tr;
 }
-// CTAs per SM that the register allocation is bounded for (0: no bound; an explicit 1
-// measured more registers and fewer CTAs per SM for the staged-halo kernels)
-__host__ __device__ constexpr int tile_min_blocks(int dpt, bool gather) { return gather && dpt == 4 ? 2 : 0; }
 // shared memory of one stage of records (TR rows per tile), in float4
 template <int D, int TR>
 __host__ __device__ constexpr int rec_stage_f4() { return kRecK * TR * (rec_words<D>() / 4); }
@@ -554,191 +548,352 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
     return false;
 }
 
-// Tiled FP32 L-apply, one CTA per (row tile, direction chunk).  Thread 0
-// feeds the CTA's shared memory through bulk copies (the TMA engine), each
-// completing on an mbarrier:
-//   * the halo rows of X (the union of the tile's columns, the chunk's
-//     directions): one copy per row, all on one barrier;
-//   * the tile's record slots, kRecK entries per stage (kRecKGather in gather
-//     mode), kRecStages stages in flight; a stage's buffer is refilled once every
-//     thread is done with it (a proxy fence and the CTA barrier order the reads
-//     before the refill).
-// Thread (s, g) owns row slot s and DPT directions of the chunk (quads g and
-// g + G, G = mc / DPT, so the threads of a row read one contiguous run of the
-// staged row), combines the K base-array values of an entry with its
-// directions' coefficients and accumulates value x X, two directions per
-// packed FP32 FMA; then it adds the outflow-face terms of a boundary row and
-// writes Y = L X or Y = B - L X.  Every decision taken on a wait is
-// block-uniform; a wait that gives up sets *err, lets the copies in flight
-// land (bounded waits) and ends the CTA.
-// GX (gather mode): no halo is staged; a record's index word is the global
-// offset col x m of its column's row, and the thread reads its directions of
-// that row from global memory (L2).  Without the halo in shared memory a
-// chunk holds all directions (up to the thread limit), so the records are
-// streamed once per tile, not once per chunk: the choice for large direction
-// sets, whose halos leave room for only a few directions per chunk.
-template <int D, int DPT, int TR, bool GX>
-__global__ void __launch_bounds__(TR * tile_max_groups(TR, DPT, GX), tile_min_blocks(DPT, GX)) k_spmm32_tile(
-    int m, int mc, int xs, int hx_f4, const int32_t *__restrict__ base, const int32_t *__restrict__ width,
-    const int32_t *__restrict__ trow, const int32_t *__restrict__ hptr, const int32_t *__restrict__ hcol,
+// ---------------------------------------------------------------------------
+// Tiled FP32 L-apply on row pairs, one CTA per (row tile, direction chunk).
+//
+// Thread (s, g) owns rows 2s and 2s + 1 of the tile and DPT directions of the
+// chunk (quads g and g + G, G = chunk / DPT, so the threads of a pair read one
+// contiguous run of an X row).  A slot holds both rows' K base-array values,
+// interleaved, so that one packed FP32 FMA serves the two rows and an X value is
+// fetched once for both; with the pair's union list 14 % of the products multiply
+// a zero.  The combination is the Horner form in Omega (2D: v = a0 + ox (ax +
+// ox axx + oy axy) + oy (ay + oy ayy)): the K - 1 FMAs of the plain sum, but D
+// coefficients per direction in registers instead of K - 1.
+//
+// The slots stream through a ring in shared memory that belongs to one warp: the
+// kPairStages next groups of four slots of the warp's pairs, each group moved by
+// one bulk copy (the TMA engine) that completes on the warp's own mbarrier and is
+// refilled by the warp's lane 0 once all its lanes are done with it.  The reads
+// (generic proxy) are ordered before the refill (async proxy) by a proxy fence in
+// every lane and the warp barrier; without it a refill could overwrite a group
+// still being read.  No warp waits for another after the halo has arrived, and
+// each warp streams only its own longest pair.
+// The halo rows of X (the union of the tile's columns, the chunk's directions)
+// are staged once per CTA: one bulk copy per row, all on one barrier.  UA (m no
+// multiple of four: rows of X do not start on 16-byte boundaries): 4-byte cp.async
+// copies.  GX (gather mode): no halo is staged; the index of a slot is the global
+// offset col x m of its column's row and the thread reads X from global memory (L1
+// / L2).  Without the halo a chunk holds all directions, so the slots are streamed
+// once per tile: the choice for large direction sets.
+// KS > 1: KS groups of warps share a tile's slots and add their sums in shared
+// memory, in group order (small problems, which leave most SMs idle).
+// Every wait is bounded: a warp whose wait gives up sets *err and leaves once its
+// copies in flight have landed (bounded waits again).
+//
+// What bounds it.  2D: the FP32 FMA pipe (a packed FMA issues every second clock:
+// 26 us at 256^2 S8 with the union's zeros) and, beside it, the shared-memory
+// return path (a 16-byte load costs a warp 4 clocks, 2 when the lanes of each
+// even-odd pair share their address; 26 us); about 60 % of the issue slots are taken.
+// 3D: X through the L1 (272 directions: half of the 2 GB that 24^3 reads come from L2).
+// Before (one row per thread, CTA-wide record stages) and after, warm, back to back:
+//   2D  32^2 S4 14.4 -> 10.3 us, 100^2 S8 24.6 -> 20.6, 256^2 S8 80.5 -> 60.8,
+//       128^2 S12 63.8 -> 45.1, 181^2 with 14 directions (row teams before) 47.1 -> 23.9
+//   3D  8^3 S4 65.6 -> 28.8 us, 20^3 S8 154.6 -> 138.6, 24^3 x 272 759 -> 579
+// Tried and not kept: the combination on mma.sync (FP16 parts) with the union of
+// 8 rows, whose legacy tensor path issues one m16n8k16 in about 64 clocks here (93 us at
+// 256^2 S8, 1.5 ms at 24^3 x 272); a producer warp with CTA-wide stages (66 us).
+// ---------------------------------------------------------------------------
+template <int D>
+__host__ __device__ constexpr int pair_f4() { return 2 * NA<D>() / 4; }   // float4 per slot
+static_assert(2 * 6 % 4 == 0 && 2 * 10 % 4 == 0, "whole float4 words per slot");
+// one group: four column indices, then the values of four slots.  208 bytes (2D) and 336 (3D) are
+// 80 mod 128, so the groups of up to eight neighbouring pairs start on different banks.
+template <int D>
+__host__ __device__ constexpr int group_f4() { return 1 + 4 * pair_f4<D>(); }
+
+template <int D>
+__global__ void k_pair_records(int64_t nslot, int64_t nnz, int tp, int xs, const int32_t *__restrict__ perm0,
+                               const int32_t *__restrict__ perm1, const int32_t *__restrict__ lcol,
+                               const float *__restrict__ A32, float4 *__restrict__ rec) {
+    constexpr int K = NA<D>(), F4 = pair_f4<D>(), GF = group_f4<D>();
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;   // slot: [tile][k][pair]
+    if (e >= nslot) return;
+    // tile widths are multiples of four, so groups never straddle tiles: [tile][k / 4][pair][group]
+    const int64_t quad = e / (4 * tp);
+    const int r = (int)(e - quad * (4 * tp)), k = r / tp, s = r - k * tp;
+    const int32_t p0 = perm0[e], p1 = perm1[e];
+    float v[2 * K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+        v[2 * q] = p0 >= 0 ? A32[q * nnz + p0] : 0.0f;
+        v[2 * q + 1] = p1 >= 0 ? A32[q * nnz + p1] : 0.0f;
+    }
+    float4 *g = rec + (quad * tp + s) * GF;
+    reinterpret_cast<int32_t *>(g)[k] = lcol[e] * xs;
+    float4 *o = g + 1 + k * F4;
+#pragma unroll
+    for (int q = 0; q < F4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+
+// Two FP32 values in one 64-bit register pair.  As opaque 64-bit values: with float2 operands the
+// compiler keeps one half of a pair whose halves are equal and rebuilds it by moves at every use (24
+// moves a slot in the 2D kernel, against 28 FMAs).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm volatile("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;\n" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// v = sum_k c_k a_k of one slot and direction for both rows (o: the direction's D components, each in
+// both halves), Horner in Omega; array order 1, Omega_a, Omega_a^2, Omega_a Omega_b (a < b)
+template <int D>
+__device__ __forceinline__ f32x2 pair_combine(const f32x2 *a, const f32x2 *o) {
+    if constexpr (D == 2) {
+        const f32x2 tx = fma2(o[0], a[3], fma2(o[1], a[5], a[1]));
+        const f32x2 ty = fma2(o[1], a[4], a[2]);
+        return fma2(o[1], ty, fma2(o[0], tx, a[0]));
+    } else {
+        const f32x2 tx = fma2(o[0], a[4], fma2(o[1], a[7], fma2(o[2], a[8], a[1])));
+        const f32x2 ty = fma2(o[1], a[5], fma2(o[2], a[9], a[2]));
+        const f32x2 tz = fma2(o[2], a[6], a[3]);
+        return fma2(o[2], tz, fma2(o[1], ty, fma2(o[0], tx, a[0])));
+    }
+}
+
+constexpr int kPairStages = 3;
+constexpr int kPairMaxThreads = 320;
+constexpr int kPairMaxWarps = kPairMaxThreads / 32;
+constexpr int kPairMinTiles = 304;     // tiles wanted: two per SM
+constexpr int kPairWarpsPerSm = 12;    // warps per SM below which warps share the slots of a tile
+__host__ __device__ constexpr int pair_min_blocks(int d, int dpt) { return dpt == 8 ? 1 : (d == 2 ? 3 : 2); }
+// the most pairs that the 32 lanes of one warp of a tile belong to
+static int pairs_per_warp(int TP, int G) {
+    int most = 1;
+    for (int w = 0; w * 32 < TP * G; ++w)
+        most = std::max(most, std::min(TP - 1, (w * 32 + 31) / G) - w * 32 / G + 1);
+    return most;
+}
+
+// tile header: first slot, slots per pair (unused here), halo range
+template <int D, int DPT, bool GX, bool UA>
+__global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_spmm32_pair(
+    int m, int mc, int G, int TP, int KS, int xs, int hx_f4, int ppw, const int4 *__restrict__ head,
+    const int32_t *__restrict__ plen, const int2 *__restrict__ trow, const int32_t *__restrict__ hcol,
     const float4 *__restrict__ rec, const float *__restrict__ coef32, const int32_t *__restrict__ bptr,
     const int32_t *__restrict__ bhalo, const float *__restrict__ bval, int64_t nb, const float *__restrict__ X,
     const float *__restrict__ B, float *__restrict__ Y, int *__restrict__ err) {
-    constexpr int K = NA<D>(), RW4 = rec_words<D>() / 4, NQ = DPT / 4, NS = kRecStages;
-    constexpr int RK = rec_k(GX);            // entries per record stage
-    constexpr int SF4 = RK * TR * RW4;      // float4 per record stage
-    constexpr uint32_t SBYTES = SF4 * 16u;
+    constexpr int K = NA<D>(), F4 = pair_f4<D>(), GF = group_f4<D>(), NQ = DPT / 4, NS = kPairStages;
     extern __shared__ float4 smem_x4[];
-    __shared__ __align__(8) uint64_t bars[NS + 1];   // record stages, then the halo
+    __shared__ __align__(8) uint64_t full[kPairMaxWarps][NS], hbar;
     float *Xs = reinterpret_cast<float *>(smem_x4);
-    float4 *Rs = smem_x4 + hx_f4;
-    const int t = blockIdx.x, m0 = blockIdx.y * mc, mcw = min(mc, m - m0), G = mc / DPT;
-    const int s = threadIdx.x / G, g = threadIdx.x - s * G;
-    const int W = width[t], nst = W / RK;
-    const float4 *rg = rec + (int64_t)base[t] * RW4;
-    const int h0 = hptr[t], hn = hptr[t + 1] - h0;
-    const uint32_t row_bytes = (uint32_t)mcw * 4u;
-    if (threadIdx.x == 0) {
-        for (int b = 0; b <= NS; ++b) mbar_init(&bars[b], 1);
+    const int t = blockIdx.x, m0 = blockIdx.y * mc, mcw = min(mc, m - m0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int4 hd = head[t];
+    // KS warp groups of w1 warps share the tile: group ks takes the slot groups ks, ks + KS, ..
+    const int w1 = (TP * G + 31) >> 5, ks = warp / w1, wk = warp - ks * w1, tk = wk * 32 + lane;
+    // the warp's pairs, its longest union and its ring
+    int s = tk / G;
+    const bool live = s < TP;
+    if (!live) s = TP - 1;
+    const int g = live ? tk - s * G : 0;
+    const int s0 = min(TP - 1, wk * 32 / G), np = min(TP - 1, (wk * 32 + 31) / G) - s0 + 1;
+    const int nq = max(0, ((__reduce_max_sync(0xffffffffu, live ? plen[t * TP + s] : 0) + 3) / 4 - ks + KS - 1) / KS);
+    float4 *ring = smem_x4 + hx_f4 + warp * (NS * ppw * GF);
+    const float4 *src = rec + ((int64_t)hd.x / 4 + (int64_t)ks * TP + s0) * GF;
+    const int64_t qstep = (int64_t)KS * TP * GF;
+    const uint32_t gbytes = (uint32_t)(np * GF) * 16u;
+    if (lane == 0) {
+        for (int b = 0; b < NS; ++b) mbar_init(&full[warp][b], 1);
+        if (tid == 0) mbar_init(&hbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if constexpr (!GX) mbar_expect(&bars[NS], (uint32_t)hn * row_bytes);
-        for (int st = 0; st < NS && st < nst; ++st) {
-            mbar_expect(&bars[st], SBYTES);
-            bulk_g2s(Rs + st * SF4, rg + (int64_t)st * SF4, SBYTES, &bars[st]);
+        fence_proxy_async();
+        for (int b = 0; b < NS && b < nq; ++b) {
+            mbar_expect(&full[warp][b], gbytes);
+            bulk_g2s(ring + b * ppw * GF, src + b * qstep, gbytes, &full[warp][b]);
         }
     }
-    if constexpr (!GX)
-        for (int hh = threadIdx.x; hh < hn; hh += blockDim.x)
-            bulk_g2s(Xs + hh * xs, X + (int64_t)hcol[h0 + hh] * m + m0, row_bytes, &bars[NS]);
-    // GX: X is read from global memory, at the chunk's first direction
-    const float *Xg = X + m0;
-    // the thread's directions and their coefficient pairs
+    __syncthreads();
+    if constexpr (!GX && !UA) {
+        const int hn = hd.w - hd.z;
+        if (tid == 0) mbar_expect(&hbar, (uint32_t)(hn * mcw) * 4u);
+        for (int hh = tid; hh < hn; hh += blockDim.x)
+            bulk_g2s(Xs + hh * xs, X + (int64_t)hcol[hd.z + hh] * m + m0, (uint32_t)mcw * 4u, &hbar);
+    }
+    if constexpr (!GX && UA) {
+        const int hn = hd.w - hd.z;
+        for (int e = tid; e < hn * mcw; e += blockDim.x) {
+            const int hh = e / mcw, k = e - hh * mcw;
+            cp_async4(Xs + hh * xs + k, X + (int64_t)hcol[hd.z + hh] * m + m0 + k);
+        }
+        cp_async_commit();
+    }
+    const int2 rows = live ? trow[t * TP + s] : make_int2(-1, -1);
     int qoff[NQ];
     bool on[NQ];
+    f32x2 o[DPT][D];   // the directions' components, each in both halves
 #pragma unroll
     for (int u = 0; u < NQ; ++u) {
         qoff[u] = 4 * (g + u * G);
-        on[u] = qoff[u] < mcw;
-    }
-    float2 c[K][2 * NQ];   // c[0] unused (the coefficient of the first array is 1)
+        on[u] = live && qoff[u] < mcw;
 #pragma unroll
-    for (int u = 0; u < NQ; ++u)
+        for (int h = 0; h < 4; ++h) {
+            const int d = m0 + min(on[u] ? qoff[u] + h : 0, mcw - 1);   // UA: a last quad may be partial
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int d0 = m0 + (on[u] ? qoff[u] : 0) + 2 * h;
-#pragma unroll
-            for (int k = 1; k < K; ++k) c[k][2 * u + h] = make_float2(coef32[16 * d0 + k], coef32[16 * (d0 + 1) + k]);
-        }
-    float2 acc[2 * NQ];
-#pragma unroll
-    for (int j = 0; j < 2 * NQ; ++j) acc[j] = make_float2(0.0f, 0.0f);
-    bool ok = true;
-    if constexpr (!GX) ok = __syncthreads_and(mbar_wait(&bars[NS], 0));
-    int st = 0;
-    for (; st < nst && ok; ++st) {
-        const int b = st % NS;
-        if (!__syncthreads_and(mbar_wait(&bars[b], (st / NS) & 1))) { ok = false; break; }
-        const float4 *rb = Rs + b * SF4 + s * RW4;
-#pragma unroll
-        for (int kk = 0; kk < RK; ++kk) {
-            float a[4 * RW4];
-#pragma unroll
-            for (int q = 0; q < RW4; ++q) {
-                const float4 v = rb[kk * TR * RW4 + q];
-                a[4 * q] = v.x; a[4 * q + 1] = v.y; a[4 * q + 2] = v.z; a[4 * q + 3] = v.w;
+            for (int c = 0; c < D; ++c) {
+                const float v = coef32[16 * d + 1 + c];
+                o[4 * u + h][c] = pack2(v, v);
             }
-            const float *xr = (GX ? Xg : Xs) + __float_as_int(a[K]);
-            float2 ab[K];   // the entry's values, each in both halves of a pair
+        }
+    }
+    float2 acc[DPT];
 #pragma unroll
-            for (int k2 = 0; k2 < K; ++k2) ab[k2] = make_float2(a[k2], a[k2]);
+    for (int j = 0; j < DPT; ++j) acc[j] = make_float2(0.0f, 0.0f);
+    bool ok = true;
+    if constexpr (!GX && !UA) ok = __all_sync(0xffffffffu, mbar_wait(&hbar, 0));
+    if constexpr (!GX && UA) {
+        cp_async_wait<0>();
+        __syncthreads();
+    }
+    const float *Xb = GX ? X + m0 : Xs;
+    const float4 *gp = ring + (s - s0) * GF;
+    int q = 0, b = 0;
+    uint32_t ph = 0;
+    for (; q < nq && ok; ++q) {
+        ok = __all_sync(0xffffffffu, mbar_wait(&full[warp][b], ph));
+        if (!ok) break;
+        const float4 *gb = gp + b * ppw * GF;
+        const int4 id4 = *reinterpret_cast<const int4 *>(gb);
+        const int id[4] = {id4.x, id4.y, id4.z, id4.w};
+        auto load_x = [&](int kk, float4 *x4) {
+#pragma unroll
+            for (int u = 0; u < NQ; ++u)
+                // GX: a quad past the last chunk's directions is not read (it may lie past X)
+                x4[u] = !GX ? *reinterpret_cast<const float4 *>(Xb + id[kk] + qoff[u])
+                            : (on[u] ? __ldg(reinterpret_cast<const float4 *>(Xb + id[kk] + qoff[u]))
+                                     : make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+        };
+        float4 x4[GX ? 4 : 1][NQ];   // gather mode: the four loads in flight together
+        if constexpr (GX)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) load_x(kk, x4[kk]);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            if constexpr (!GX) load_x(kk, x4[0]);
+            f32x2 a[K];
+#pragma unroll
+            for (int w = 0; w < F4; ++w) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(gb + 1 + kk * F4 + w);
+                a[2 * w] = v.x;
+                a[2 * w + 1] = v.y;
+            }
 #pragma unroll
             for (int u = 0; u < NQ; ++u) {
-                // GX: a quad past the last chunk's directions is not read (it may lie past X)
-                const float4 x4 = !GX ? *reinterpret_cast<const float4 *>(xr + qoff[u])
-                                      : (on[u] ? __ldg(reinterpret_cast<const float4 *>(xr + qoff[u]))
-                                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f));
-                const float2 xp[2] = {make_float2(x4.x, x4.y), make_float2(x4.z, x4.w)};
+                const float4 x = x4[GX ? kk : 0][u];
+                const float xv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float2 v = ab[0];
-#pragma unroll
-                    for (int k2 = 1; k2 < K; ++k2) v = __ffma2_rn(c[k2][2 * u + h], ab[k2], v);
-                    acc[2 * u + h] = __ffma2_rn(v, xp[h], acc[2 * u + h]);
+                for (int h = 0; h < 4; ++h) {
+                    float v0, v1;
+                    unpack2(pair_combine<D>(a, o[4 * u + h]), v0, v1);
+                    // two scalar FMAs: a packed one would first copy x into both halves
+                    acc[4 * u + h].x = fmaf(v0, xv[h], acc[4 * u + h].x);
+                    acc[4 * u + h].y = fmaf(v1, xv[h], acc[4 * u + h].y);
                 }
             }
         }
-        // every thread is done with buffer b: its reads (generic proxy) are ordered before the
-        // bulk copy that refills it (async proxy) by a proxy fence, then the CTA barrier.
-        // Without the fence a refill could overwrite a stage still being read: measured at 40^3
-        // in gather mode, where results moved by 3.5e-3 under a different register allocation.
         fence_proxy_async();
-        __syncthreads();
-        if (threadIdx.x == 0 && st + NS < nst) {
-            mbar_expect(&bars[b], SBYTES);
-            bulk_g2s(Rs + b * SF4, rg + (int64_t)(st + NS) * SF4, SBYTES, &bars[b]);
+        __syncwarp();
+        if (lane == 0 && q + NS < nq) {
+            mbar_expect(&full[warp][b], gbytes);
+            bulk_g2s(ring + b * ppw * GF, src + (q + NS) * qstep, gbytes, &full[warp][b]);
+        }
+        if (++b == NS) {
+            b = 0;
+            ph ^= 1u;
         }
     }
-    if (!ok) {   // (block-uniform) report, let the copies in flight land, leave
-        if (threadIdx.x == 0) {
+    if (!ok) {   // (warp-uniform) report, let the copies in flight land, leave
+        if (lane == 0) {
             atomicOr(err, 1);
-            if constexpr (!GX) mbar_wait(&bars[NS], 0);
-            for (int k = st; k < nst && k < st + NS; ++k) mbar_wait(&bars[k % NS], (k / NS) & 1);
+            if constexpr (!GX && !UA) mbar_wait(&hbar, 0);
+            for (int k = q; k < nq && k < q + NS; ++k) {
+                mbar_wait(&full[warp][b], ph);
+                if (++b == NS) {
+                    b = 0;
+                    ph ^= 1u;
+                }
+            }
         }
-        __syncthreads();
+        __syncwarp();
         return;
     }
-    const int32_t row = trow[(int64_t)t * TR + s];
-    if (row < 0) return;
-    // outflow-face terms of a boundary row: sum_f max(Omega . n_f, 0) (S_f X)_i
-    const int32_t q0 = bptr[row], q1 = bptr[row + 1];
-    if (q1 > q0) {
-        float2 fc[NF<D>()][2 * NQ];
+    if (KS > 1) {   // add the groups' sums, in group order; the rings are free once every warp is here
+        float2 *part = reinterpret_cast<float2 *>(smem_x4 + hx_f4);
+        __syncthreads();
+        if (ks > 0)
 #pragma unroll
-        for (int u = 0; u < NQ; ++u)
+            for (int j = 0; j < DPT; ++j) part[(((ks - 1) * DPT + j) * w1) * 32 + tk] = acc[j];
+        __syncthreads();
+        if (ks > 0) return;
+        for (int k = 0; k < KS - 1; ++k)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int d0 = m0 + (on[u] ? qoff[u] : 0) + 2 * h;
-#pragma unroll
-                for (int f = 0; f < NF<D>(); ++f)
-                    fc[f][2 * u + h] = make_float2(coef32[16 * d0 + face_slot<D>() + f],
-                                                   coef32[16 * (d0 + 1) + face_slot<D>() + f]);
+            for (int j = 0; j < DPT; ++j) {
+                const float2 v = part[((k * DPT + j) * w1) * 32 + tk];
+                acc[j].x += v.x;
+                acc[j].y += v.y;
             }
-        for (int32_t q = q0; q < q1; ++q) {
-            const float *xr = (GX ? Xg : Xs) + bhalo[q];
-            float2 sv[NF<D>()];
+    }
 #pragma unroll
-            for (int f = 0; f < NF<D>(); ++f) {
-                const float v = bval[f * nb + q];
-                sv[f] = make_float2(v, v);
-            }
+    for (int r = 0; r < 2; ++r) {
+        const int32_t row = r == 0 ? rows.x : rows.y;
+        if (row < 0) continue;
+        float res[DPT];
+#pragma unroll
+        for (int j = 0; j < DPT; ++j) res[j] = r == 0 ? acc[j].x : acc[j].y;
+        // outflow-face terms of a boundary row: sum_f max(Omega . n_f, 0) (S_f X)_i
+        const int32_t q1 = bptr[row + 1];
+        for (int32_t p = bptr[row]; p < q1; ++p) {
+            const float *xr = Xb + bhalo[p];
+            float sv[NF<D>()];
+#pragma unroll
+            for (int f = 0; f < NF<D>(); ++f) sv[f] = bval[f * nb + p];
 #pragma unroll
             for (int u = 0; u < NQ; ++u) {
-                const float4 x4 = (GX && !on[u]) ? make_float4(0.0f, 0.0f, 0.0f, 0.0f)
+                const float4 xf = (GX && !on[u]) ? make_float4(0.0f, 0.0f, 0.0f, 0.0f)
                                                  : *reinterpret_cast<const float4 *>(xr + qoff[u]);
-                const float2 xp[2] = {make_float2(x4.x, x4.y), make_float2(x4.z, x4.w)};
+                const float xv[4] = {xf.x, xf.y, xf.z, xf.w};
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float2 v = make_float2(0.0f, 0.0f);
+                for (int h = 0; h < 4; ++h) {
+                    float v = 0.0f;
 #pragma unroll
-                    for (int f = 0; f < NF<D>(); ++f) v = __ffma2_rn(fc[f][2 * u + h], sv[f], v);
-                    acc[2 * u + h] = __ffma2_rn(v, xp[h], acc[2 * u + h]);
+                    for (int c = 0; c < D; ++c) {   // faces -e_c, +e_c
+                        float oc, od;
+                        unpack2(o[4 * u + h][c], oc, od);
+                        v = fmaf(fmaxf(-oc, 0.0f), sv[2 * c], fmaf(fmaxf(oc, 0.0f), sv[2 * c + 1], v));
+                    }
+                    res[4 * u + h] = fmaf(v, xv[h], res[4 * u + h]);
                 }
             }
         }
-    }
 #pragma unroll
-    for (int u = 0; u < NQ; ++u) {
-        if (!on[u]) continue;
-        const int64_t e = (int64_t)row * m + m0 + qoff[u];
-        float4 o = make_float4(acc[2 * u].x, acc[2 * u].y, acc[2 * u + 1].x, acc[2 * u + 1].y);
-        if (B) {
-            const float4 bv = *reinterpret_cast<const float4 *>(B + e);
-            o = make_float4(bv.x - o.x, bv.y - o.y, bv.z - o.z, bv.w - o.w);
+        for (int u = 0; u < NQ; ++u) {
+            if (!on[u]) continue;
+            const int64_t e = (int64_t)row * m + m0 + qoff[u];
+            if constexpr (UA) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    if (qoff[u] + h < mcw) Y[e + h] = B ? B[e + h] - res[4 * u + h] : res[4 * u + h];
+            } else {
+                float4 v = make_float4(res[4 * u], res[4 * u + 1], res[4 * u + 2], res[4 * u + 3]);
+                if (B) {
+                    const float4 bv = *reinterpret_cast<const float4 *>(B + e);
+                    v = make_float4(bv.x - v.x, bv.y - v.y, bv.z - v.z, bv.w - v.w);
+                }
+                *reinterpret_cast<float4 *>(Y + e) = v;
+            }
         }
-        *reinterpret_cast<float4 *>(Y + e) = o;
     }
 }
 
@@ -1475,28 +1630,45 @@ Team pick_team(int m) {
 static int64_t team_grid(int64_t n, const Team &) { return (n * 32 + 255) / 256; }
 static int64_t rowteam_grid(int64_t n, const Team &tm) { return ((n << tm.tm_log2) + 255) / 256; }
 
-// Row tiles of the FP32 L-apply: built once per point set when m % 4 == 0.
-// Tile shape: TR rows per tile and DPT directions per thread, from the options
-// or by default 64 rows and 8 directions (4 when m % 8 != 0) with a staged
-// halo, 4 directions and at most 320 threads per CTA in gather mode; G = chunk
-// / DPT thread groups per row.  The directions are split into chunks (one CTA
-// each) until a tile's staged halo, halo x (chunk + 4) floats, and the record
-// stages fit kTileSmem (staged halo), or until G fits the thread limit
-// (gather).  The automatic choice stages the halo while that takes at most
-// two chunks, and gathers otherwise.
+// Row tiles of the FP32 L-apply: built once per point set.  Tile shape: TR rows
+// per tile and DPT directions per thread, from the options or by the rules of
+// plan_tiles; G = chunk / DPT thread groups per row pair.  The directions are
+// split into chunks (one CTA each) until a tile's staged halo, halo x (chunk + 4)
+// floats, and the record stages fit kTileSmem (staged halo), or until G fits the
+// thread limit (gather).  The automatic choice stages the halo while that takes
+// at most two chunks, and gathers otherwise (m % 4 == 0; row teams serve the
+// rest).
 constexpr size_t kTileSmem = 100 * 1024;
 
-template <int D, int DPT, int TR, bool GX>
-static mlpg_status launch_tile(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
+template <int D, int DPT, bool GX, bool UA>
+static mlpg_status launch_pair(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
     const dim3 tg((unsigned)ctx->ntile, (unsigned)((ctx->m + ctx->tile_chunk - 1) / ctx->tile_chunk));
-    const int threads = TR * (ctx->tile_chunk / DPT);
-    k_spmm32_tile<D, DPT, TR, GX><<<tg, threads, ctx->tile_smem, ctx->stream>>>(
-        ctx->m, ctx->tile_chunk, ctx->tile_xs, ctx->tile_xs_f4, ctx->t_base, ctx->t_width, ctx->t_row, ctx->t_hptr,
-        ctx->t_hcol, reinterpret_cast<const float4 *>(ctx->t_rec), ctx->coef32, ctx->bptr, ctx->t_bhalo, ctx->bval32,
-        ctx->nb, X, B, Y, ctx->d_tile_err);
+    const int TP = ctx->tile_rows / 2, G = ctx->tile_chunk / DPT;
+    k_spmm32_pair<D, DPT, GX, UA><<<tg, (TP * G + 31) / 32 * 32 * ctx->tile_ks, ctx->tile_smem, ctx->stream>>>(
+        ctx->m, ctx->tile_chunk, G, TP, ctx->tile_ks, ctx->tile_xs, ctx->tile_xs_f4, pairs_per_warp(TP, G),
+        reinterpret_cast<const int4 *>(ctx->t_head), ctx->t_plen, reinterpret_cast<const int2 *>(ctx->t_row), ctx->t_hcol,
+        reinterpret_cast<const float4 *>(ctx->t_rec), ctx->coef32, ctx->bptr, ctx->t_bhalo, ctx->bval32, ctx->nb, X, B, Y,
+        ctx->d_tile_err);
     CU_LAUNCH(ctx);
     return MLPG_OK;
 }
+// Warp groups that share the slots of a tile: enough of them to give every SM kPairWarpsPerSm warps,
+// while a group keeps at least two groups of four slots and the CTA its thread limit
+static int pair_split(int64_t ctas, int TP, int G, int width) {
+    const int w1 = (TP * G + 31) / 32;
+    int ks = 1;
+    while (2 * ks * w1 * 32 <= kPairMaxThreads && ctas * w1 * ks < (int64_t)kPairWarpsPerSm * 152 && width / (8 * ks) >= 2)
+        ks *= 2;
+    return ks;
+}
+// shared memory of the warps' rings, or of the partial sums of the split, which reuse it
+template <int D>
+static size_t ring_bytes(int TP, int G, int dpt, int ks) {
+    const size_t w1 = (size_t)(TP * G + 31) / 32;
+    const size_t ring = w1 * ks * kPairStages * pairs_per_warp(TP, G) * group_f4<D>() * sizeof(float4);
+    return std::max(ring, (ks - 1) * w1 * 32 * 2 * dpt * sizeof(float));
+}
+
 template <int D, int TR, int NT>
 static mlpg_status launch_mma(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
     const dim3 tg((unsigned)ctx->ntile, (unsigned)(ctx->m / (8 * NT)));
@@ -1528,41 +1700,29 @@ static mlpg_status run_tile(mlpg_ctx *ctx, const float *X, const float *B, float
         if (ctx->tile_rows == 32) { MMA_NT_SWITCH(D, 32, launch_mma, ctx, X, B, Y) }
         MMA_NT_SWITCH(D, 64, launch_mma, ctx, X, B, Y)
     }
-    const int key = ctx->tile_dpt * 100 + ctx->tile_rows;
-    if (ctx->tile_gather) switch (key) {
-            case 804: return launch_tile<D, 8, 4, true>(ctx, X, B, Y);
-            case 404: return launch_tile<D, 4, 4, true>(ctx, X, B, Y);
-            case 808: return launch_tile<D, 8, 8, true>(ctx, X, B, Y);
-            case 816: return launch_tile<D, 8, 16, true>(ctx, X, B, Y);
-            case 832: return launch_tile<D, 8, 32, true>(ctx, X, B, Y);
-            case 408: return launch_tile<D, 4, 8, true>(ctx, X, B, Y);
-            case 416: return launch_tile<D, 4, 16, true>(ctx, X, B, Y);
-            default: return launch_tile<D, 4, 32, true>(ctx, X, B, Y);
-        }
-    switch (key) {
-        case 832: return launch_tile<D, 8, 32, false>(ctx, X, B, Y);
-        case 864: return launch_tile<D, 8, 64, false>(ctx, X, B, Y);
-        case 432: return launch_tile<D, 4, 32, false>(ctx, X, B, Y);
-        default: return launch_tile<D, 4, 64, false>(ctx, X, B, Y);
-    }
+    if (ctx->tile_gather)
+        return ctx->tile_dpt == 8 ? launch_pair<D, 8, true, false>(ctx, X, B, Y) : launch_pair<D, 4, true, false>(ctx, X, B, Y);
+    if ((ctx->m & 3) != 0) return launch_pair<D, 4, false, true>(ctx, X, B, Y);
+    return ctx->tile_dpt == 8 ? launch_pair<D, 8, false, false>(ctx, X, B, Y) : launch_pair<D, 4, false, false>(ctx, X, B, Y);
 }
-template <int D, int DPT, int TR, bool GX>
-static mlpg_status tile_attr(mlpg_ctx *ctx) {
-    // the kernel's attribute is shared by every context: set to the fixed budget, never lowered
-    // (the record stages of 32-row gather tiles alone reach the 48 KB default)
-    CU(ctx, cudaFuncSetAttribute(k_spmm32_tile<D, DPT, TR, GX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+// the kernel's attribute is shared by every context: set to the fixed budget, never lowered
+template <int D, int DPT, bool GX, bool UA>
+static mlpg_status pair_attr(mlpg_ctx *ctx) {
+    CU(ctx, cudaFuncSetAttribute(k_spmm32_pair<D, DPT, GX, UA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kTileSmem));
     return MLPG_OK;
 }
 
 // One tile layout: rows per tile, directions per thread and per CTA (chunk),
-// staged halo or gather mode, the host-side tiles.  chunk == 0: no layout.
+// staged halo or gather mode, the host-side tiles (row pairs, or single rows for
+// the tensor cores).  chunk == 0: no layout.
 struct TilePlan {
-    int tr = 0, dpt = 0, chunk = 0;
+    int tr = 0, dpt = 0, chunk = 0, ks = 1;
     bool gather = false, mma = false;
     size_t rec_smem = 0;
     TileLayout tl;
-    int64_t nslot = 0;
+    PairTileLayout pl;
+    int64_t nslot = 0, max_halo = 0;
 };
 
 // Plans the tiles of one mode; an explicit request that cannot be met is an
@@ -1574,11 +1734,20 @@ static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P)
     P = TilePlan();
     P.gather = gather;
     P.mma = mma;
-    // gather: four directions per thread measured fastest (more CTAs per SM)
-    const int dpt = ctx->opt.tile_dpt ? ctx->opt.tile_dpt : ((m & 7) == 0 && !gather ? 8 : 4);
-    if (m % dpt != 0) return set_err(ctx, MLPG_ERR_ARG, "tile_dpt must divide the number of directions");
+    // m no multiple of four: staged value by value.  The automatic choice takes four directions per thread:
+    // eight measured slower at every size (256^2 S8: 69.3 against 60.8 us; more registers, fewer warps)
+    const int dpt = (m & 3) != 0 ? 4 : (ctx->opt.tile_dpt ? ctx->opt.tile_dpt : ((m & 7) == 0 && !gather && (ask || mma) ? 8 : 4));
+    if ((m & 3) == 0 && m % dpt != 0) return set_err(ctx, MLPG_ERR_ARG, "tile_dpt must divide the number of directions");
     int tr = ctx->opt.tile_rows;
-    if (gather && tr == 0) {   // the most rows per tile with at most 320 threads per CTA
+    if (tr == 0 && !ask) {
+        // gather: the most rows per tile (X rows shared through the L1) that keep a CTA at or below
+        // kPairMaxThreads; staged: 64 rows (the smallest halo per row), fewer while that leaves SMs without a tile
+        const int G = (m + dpt - 1) / dpt;
+        tr = gather ? 32 : 64;
+        while (tr > 4 && gather && tr / 2 * G > kPairMaxThreads) tr /= 2;
+        while (tr > (gather ? 4 : 8) && (ctx->n + tr - 1) / tr < kPairMinTiles) tr /= 2;
+    }
+    if (gather && tr == 0) {   // the most rows per tile with at most 320 (row, direction group) tasks
         const int G = (m + dpt - 1) / dpt;
         tr = 4;
         for (int c : {32, 16, 8})
@@ -1592,12 +1761,18 @@ static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P)
         return ask ? set_err(ctx, MLPG_ERR_ARG, "apply_kernel 4 takes 4, 8, 16 or 32 rows per tile") : MLPG_OK;
     if (gather && (int64_t)ctx->n * m >= (int64_t(1) << 31))
         return ask ? set_err(ctx, MLPG_ERR_ARG, "apply_kernel 4 needs n x m < 2^31 (32-bit record offsets)") : MLPG_OK;
-    const int rk = rec_k(gather);
-    P.nslot = build_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), ctx->h_order.data(), tr, rk, P.tl);
-    const TileLayout &tl = P.tl;
-    if (P.nslot * (int64_t)(rec_words<D>() / 4) >= (int64_t(1) << 31) || tl.hptr.back() >= (int64_t(1) << 31))
-        return MLPG_OK;   // beyond 32-bit slot indices: the row-team kernel serves
-    P.rec_smem = (size_t)kRecStages * rk * tr * (rec_words<D>() / 4) * sizeof(float4);
+    if (mma) {
+        P.nslot = build_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), ctx->h_order.data(), tr, kRecK, P.tl);
+        P.max_halo = P.tl.max_halo;
+        if (P.nslot * (int64_t)(rec_words<D>() / 4) >= (int64_t(1) << 31) || P.tl.hptr.back() >= (int64_t(1) << 31))
+            return MLPG_OK;   // beyond 32-bit slot indices: the row-team kernel serves
+        P.rec_smem = (size_t)kRecStages * kRecK * tr * (rec_words<D>() / 4) * sizeof(float4);
+    } else {
+        P.nslot = build_pair_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), ctx->h_order.data(), tr, 4, !gather,
+                                   P.pl);
+        P.max_halo = P.pl.max_halo;
+        if (P.nslot >= (int64_t(1) << 31) || P.pl.hptr.back() >= (int64_t(1) << 31)) return MLPG_OK;
+    }
     int chunk = 0;
     if (mma) {
         // tensor-core tiles: chunks of 8 NT directions (NT <= 6) dividing m; shared-memory row stride
@@ -1605,14 +1780,19 @@ static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P)
         if ((m & 7) != 0) return set_err(ctx, MLPG_ERR_ARG, "apply_kernel 3 needs a multiple of 8 directions");
         for (int nt = 6; nt >= 2 && !chunk; --nt) {
             const int mc = 8 * nt, xs = mc + (16 - mc % 32 + 32) % 32;
-            if (m % mc == 0 && (size_t)tl.max_halo * xs * sizeof(float) + P.rec_smem <= kTileSmem) chunk = mc;
+            if (m % mc == 0 && (size_t)P.max_halo * xs * sizeof(float) + P.rec_smem <= kTileSmem) chunk = mc;
         }
         if (!chunk) return set_err(ctx, MLPG_ERR_ARG, "apply_kernel 3: no direction chunk fits shared memory");
     }
-    for (int nchunk = 1; nchunk <= m / 4 && !mma; ++nchunk) {
+    for (int nchunk = 1; nchunk <= (m + 3) / 4 && !mma; ++nchunk) {
         const int G = (m + dpt * nchunk - 1) / (dpt * nchunk);
-        if (G > tile_max_groups(tr, dpt, gather)) continue;
-        if (gather || (size_t)tl.max_halo * (G * dpt + 4) * sizeof(float) + P.rec_smem <= kTileSmem) {
+        if (ask ? G > tile_max_groups(tr, dpt, gather) : tr / 2 * G > kPairMaxThreads) continue;
+        const int64_t nch = (m + G * dpt - 1) / (G * dpt);
+        P.ks = pair_split(P.pl.ntile * nch, tr / 2, G, P.pl.max_width);
+        const size_t halo = gather ? 0 : (size_t)P.max_halo * (G * dpt + 4) * sizeof(float);
+        while (P.ks > 1 && halo + ring_bytes<D>(tr / 2, G, dpt, P.ks) > kTileSmem) P.ks /= 2;
+        P.rec_smem = ring_bytes<D>(tr / 2, G, dpt, P.ks);
+        if (halo + P.rec_smem <= kTileSmem) {
             chunk = G * dpt;
             break;
         }
@@ -1623,111 +1803,110 @@ static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P)
     return MLPG_OK;
 }
 
+template <typename T>
+static mlpg_status to_device(mlpg_ctx *ctx, T **d, const std::vector<T> &h) {
+    MLPG_TRY(dalloc(ctx, d, h.size()));
+    if (!h.empty()) CU(ctx, cudaMemcpyAsync(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
+    return MLPG_OK;
+}
+
 template <int D>
 static mlpg_status init_tiles(mlpg_ctx *ctx) {
     const int m = ctx->m, kind = ctx->opt.apply_kernel;
-    if ((m & 3) != 0 || kind == 1) return MLPG_OK;
+    if (kind == 1) return MLPG_OK;
+    ctx->h_order.resize(ctx->n);
+    spatial_order(ctx->n, D, ctx->h_x.data(), ctx->h_order.data());
     TilePlan P;
-    if (kind != 4) {
+    // automatic choice: 3D halos (some 700 rows for 32) leave room for few directions per chunk, and
+    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit
+    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->n * m < (int64_t(1) << 31);
+    if (kind != 4 && !skip) {
         MLPG_TRY(plan_tiles<D>(ctx, false, kind == 3, P));
-        // automatic choice: staged halos pay while the records are read by few chunks;
-        // past two chunks the gather mode reads them once
+        // staged halos pay while the records are read by few chunks; past two chunks the gather
+        // mode reads them once
         if (kind == 0 && P.chunk && (m + P.chunk - 1) / P.chunk > 2) P.chunk = 0;
     }
-    if (kind == 4 || (kind == 0 && P.chunk == 0)) MLPG_TRY(plan_tiles<D>(ctx, true, false, P));
+    if (kind == 4 || (kind == 0 && P.chunk == 0 && (m & 3) == 0)) MLPG_TRY(plan_tiles<D>(ctx, true, false, P));
     if (P.chunk == 0) return MLPG_OK;
-    const int tr = P.tr, dpt = P.dpt, chunk = P.chunk;
+    const int tr = P.tr, chunk = P.chunk;
     const bool gather = P.gather, mma = P.mma;
-    const size_t rec_smem = P.rec_smem;
     const int64_t nslot = P.nslot;
-    TileLayout &tl = P.tl;
     ctx->tile_rows = tr;
-    ctx->tile_dpt = dpt;
+    ctx->tile_dpt = P.dpt;
+    ctx->tile_ks = P.ks;
     ctx->tile_chunk = chunk;
     ctx->tile_mma = mma;
     ctx->tile_gather = gather;
     // gather: the record index is the column's global offset col x m; otherwise the column's
     // staged row in shared memory, a padded row that spreads halo rows over the banks
     ctx->tile_xs = gather ? m : (mma ? chunk + (16 - chunk % 32 + 32) % 32 : chunk + 4);
-    if (gather) {   // global columns of the slots (zero for padding: a zero record)
-        for (int64_t e = 0; e < nslot; ++e) tl.lcol[e] = tl.perm[e] >= 0 ? ctx->h_col[tl.perm[e]] : 0;
-    }
-    ctx->ntile = tl.ntile;
-    ctx->nslot = nslot;
     cudaStream_t s = ctx->stream;
-    std::vector<int32_t> base32(tl.ntile + 1), hptr32(tl.ntile + 1);
-    for (int64_t t = 0; t <= tl.ntile; ++t) {
-        base32[t] = (int32_t)tl.base[t];
-        hptr32[t] = (int32_t)tl.hptr[t];
-    }
-    MLPG_TRY(dalloc(ctx, &ctx->t_base, tl.ntile + 1));
-    MLPG_TRY(dalloc(ctx, &ctx->t_width, tl.ntile));
-    MLPG_TRY(dalloc(ctx, &ctx->t_row, tl.ntile * tr));
-    MLPG_TRY(dalloc(ctx, &ctx->t_hptr, tl.ntile + 1));
-    MLPG_TRY(dalloc(ctx, &ctx->t_hcol, tl.hcol.size()));
-    MLPG_TRY(dalloc(ctx, &ctx->t_perm, nslot));
-    MLPG_TRY(dalloc(ctx, &ctx->t_lcol, nslot));
-    MLPG_TRY(dalloc(ctx, &ctx->t_rec, nslot * rec_words<D>()));
-    CU(ctx, cudaMemcpyAsync(ctx->t_base, base32.data(), base32.size() * 4, cudaMemcpyHostToDevice, s));
-    CU(ctx, cudaMemcpyAsync(ctx->t_width, tl.width.data(), tl.width.size() * 4, cudaMemcpyHostToDevice, s));
-    CU(ctx, cudaMemcpyAsync(ctx->t_row, tl.row.data(), tl.row.size() * 4, cudaMemcpyHostToDevice, s));
-    CU(ctx, cudaMemcpyAsync(ctx->t_hptr, hptr32.data(), hptr32.size() * 4, cudaMemcpyHostToDevice, s));
-    CU(ctx, cudaMemcpyAsync(ctx->t_hcol, tl.hcol.data(), tl.hcol.size() * 4, cudaMemcpyHostToDevice, s));
-    CU(ctx, cudaMemcpyAsync(ctx->t_perm, tl.perm.data(), nslot * 4, cudaMemcpyHostToDevice, s));
-    CU(ctx, cudaMemcpyAsync(ctx->t_lcol, tl.lcol.data(), nslot * 4, cudaMemcpyHostToDevice, s));
-    // halo offset (index x shared-memory row stride) of every boundary-segment entry's column
-    {
-        std::vector<int32_t> bptr(ctx->n + 1), bcol(std::max<int64_t>(ctx->nb, 1)), bhalo(std::max<int64_t>(ctx->nb, 1), 0);
-        CU(ctx, cudaMemcpyAsync(bptr.data(), ctx->bptr, (ctx->n + 1) * 4, cudaMemcpyDeviceToHost, s));
-        if (ctx->nb > 0) CU(ctx, cudaMemcpyAsync(bcol.data(), ctx->bcol, ctx->nb * 4, cudaMemcpyDeviceToHost, s));
-        CU(ctx, cudaStreamSynchronize(s));
-        for (int64_t r = 0; r < tl.ntile * tr; ++r) {
-            const int32_t i = tl.row[r];
-            if (i < 0) continue;
-            if (gather) {
-                for (int32_t q = bptr[i]; q < bptr[i + 1]; ++q) bhalo[q] = bcol[q] * m;
-                continue;
-            }
-            const int64_t t = r / tr;
-            const int32_t *hb = tl.hcol.data() + tl.hptr[t], *he = tl.hcol.data() + tl.hptr[t + 1];
-            for (int32_t q = bptr[i]; q < bptr[i + 1]; ++q) {
-                const int32_t *hit = std::lower_bound(hb, he, bcol[q]);
-                if (hit == he || *hit != bcol[q]) return set_err(ctx, MLPG_ERR_ARG, "boundary entry outside its tile's halo");
-                bhalo[q] = (int32_t)(hit - hb) * ctx->tile_xs;
-            }
+    const int64_t ntile = mma ? P.tl.ntile : P.pl.ntile;
+    const std::vector<int64_t> &base = mma ? P.tl.base : P.pl.base, &hptr = mma ? P.tl.hptr : P.pl.hptr;
+    const std::vector<int32_t> &row = mma ? P.tl.row : P.pl.row, &hcol = mma ? P.tl.hcol : P.pl.hcol;
+    ctx->ntile = ntile;
+    ctx->nslot = nslot;
+    std::vector<int32_t> base32(base.begin(), base.end()), hptr32(hptr.begin(), hptr.end()), head(4 * ntile);
+    if (mma) {
+        MLPG_TRY(to_device(ctx, &ctx->t_base, base32));
+        MLPG_TRY(to_device(ctx, &ctx->t_hptr, hptr32));
+        MLPG_TRY(to_device(ctx, &ctx->t_width, P.tl.width));
+    } else {   // tile headers: first slot, slots per pair, halo range
+        for (int64_t t = 0; t < ntile; ++t) {
+            head[4 * t] = base32[t];
+            head[4 * t + 1] = P.pl.width[t];
+            head[4 * t + 2] = hptr32[t];
+            head[4 * t + 3] = hptr32[t + 1];
         }
-        MLPG_TRY(dalloc(ctx, &ctx->t_bhalo, bhalo.size()));
-        CU(ctx, cudaMemcpyAsync(ctx->t_bhalo, bhalo.data(), bhalo.size() * 4, cudaMemcpyHostToDevice, s));
-        CU(ctx, cudaStreamSynchronize(s));
+        MLPG_TRY(to_device(ctx, &ctx->t_head, head));
     }
+    MLPG_TRY(to_device(ctx, &ctx->t_hcol, hcol));
+    MLPG_TRY(to_device(ctx, &ctx->t_row, row));
+    MLPG_TRY(to_device(ctx, &ctx->t_lcol, mma ? P.tl.lcol : P.pl.lcol));
+    MLPG_TRY(to_device(ctx, &ctx->t_perm, mma ? P.tl.perm : P.pl.perm0));
+    if (!mma) {
+        MLPG_TRY(to_device(ctx, &ctx->t_perm1, P.pl.perm1));
+        MLPG_TRY(to_device(ctx, &ctx->t_plen, P.pl.plen));
+    }
+    MLPG_TRY(dalloc(ctx, &ctx->t_rec, nslot * (mma ? rec_words<D>() : group_f4<D>())));   // a group: group_f4 float4 for four slots
+    // halo offset (index x shared-memory row stride) of every boundary-segment entry's column
+    std::vector<int32_t> bptr(ctx->n + 1), bcol(std::max<int64_t>(ctx->nb, 1)), bhalo(std::max<int64_t>(ctx->nb, 1), 0);
+    CU(ctx, cudaMemcpyAsync(bptr.data(), ctx->bptr, (ctx->n + 1) * 4, cudaMemcpyDeviceToHost, s));
+    if (ctx->nb > 0) CU(ctx, cudaMemcpyAsync(bcol.data(), ctx->bcol, ctx->nb * 4, cudaMemcpyDeviceToHost, s));
+    CU(ctx, cudaStreamSynchronize(s));
+    for (int64_t r = 0; r < ntile * tr; ++r) {
+        const int32_t i = row[r];
+        if (i < 0) continue;
+        if (gather) {
+            for (int32_t q = bptr[i]; q < bptr[i + 1]; ++q) bhalo[q] = bcol[q] * m;
+            continue;
+        }
+        const int64_t t = r / tr;
+        const int32_t *hb = hcol.data() + hptr[t], *he = hcol.data() + hptr[t + 1];
+        for (int32_t q = bptr[i]; q < bptr[i + 1]; ++q) {
+            const int32_t *hit = std::lower_bound(hb, he, bcol[q]);
+            if (hit == he || *hit != bcol[q]) return set_err(ctx, MLPG_ERR_ARG, "boundary entry outside its tile's halo");
+            bhalo[q] = (int32_t)(hit - hb) * ctx->tile_xs;
+        }
+    }
+    MLPG_TRY(to_device(ctx, &ctx->t_bhalo, bhalo));
     CU(ctx, cudaStreamSynchronize(s));   // the host vectors go out of scope
     if (mma) {
-        mlpg_status st = MLPG_OK;
         auto set = [&]() -> mlpg_status {
             if (tr == 32) { MMA_NT_SWITCH(D, 32, mma_attr, ctx) }
             MMA_NT_SWITCH(D, 64, mma_attr, ctx)
         };
-        st = set();
-        if (st != MLPG_OK) return st;
-    } else if (gather) switch (dpt * 100 + tr) {
-            case 804: MLPG_TRY((tile_attr<D, 8, 4, true>(ctx))); break;
-            case 808: MLPG_TRY((tile_attr<D, 8, 8, true>(ctx))); break;
-            case 816: MLPG_TRY((tile_attr<D, 8, 16, true>(ctx))); break;
-            case 832: MLPG_TRY((tile_attr<D, 8, 32, true>(ctx))); break;
-            case 404: MLPG_TRY((tile_attr<D, 4, 4, true>(ctx))); break;
-            case 408: MLPG_TRY((tile_attr<D, 4, 8, true>(ctx))); break;
-            case 416: MLPG_TRY((tile_attr<D, 4, 16, true>(ctx))); break;
-            default: MLPG_TRY((tile_attr<D, 4, 32, true>(ctx))); break;
-        }
-    else switch (dpt * 100 + tr) {
-            case 832: MLPG_TRY((tile_attr<D, 8, 32, false>(ctx))); break;
-            case 864: MLPG_TRY((tile_attr<D, 8, 64, false>(ctx))); break;
-            case 432: MLPG_TRY((tile_attr<D, 4, 32, false>(ctx))); break;
-            default: MLPG_TRY((tile_attr<D, 4, 64, false>(ctx))); break;
-        }
-    ctx->tile_xs_f4 = gather ? 0 : (int)(tl.max_halo * ctx->tile_xs / 4);
-    ctx->tile_smem = (size_t)ctx->tile_xs_f4 * sizeof(float4) + rec_smem;
-    ctx->tile_max_halo = tl.max_halo;
+        MLPG_TRY(set());
+    } else {
+        MLPG_TRY((pair_attr<D, 8, true, false>(ctx)));
+        MLPG_TRY((pair_attr<D, 4, true, false>(ctx)));
+        MLPG_TRY((pair_attr<D, 8, false, false>(ctx)));
+        MLPG_TRY((pair_attr<D, 4, false, false>(ctx)));
+        MLPG_TRY((pair_attr<D, 4, false, true>(ctx)));
+    }
+    ctx->tile_xs_f4 = gather ? 0 : (int)((P.max_halo * ctx->tile_xs + 3) / 4);
+    ctx->tile_smem = (size_t)ctx->tile_xs_f4 * sizeof(float4) + P.rec_smem;
+    ctx->tile_max_halo = P.max_halo;
     if (!ctx->d_tile_err) {
         MLPG_TRY(dalloc(ctx, &ctx->d_tile_err, 1));
         CU(ctx, cudaMemsetAsync(ctx->d_tile_err, 0, sizeof(int), s));
@@ -1812,8 +1991,14 @@ static mlpg_status form_operators_d(mlpg_ctx *ctx, double kappa) {
                                                     ctx->A64, ctx->A32, ctx->T64, ctx->S64);
     CU_LAUNCH(ctx);
     if (ctx->t_rec) {
-        k_tile_records<D><<<(ctx->nslot + 255) / 256, 256, 0, s>>>(ctx->nslot, nnz, ctx->tile_xs, ctx->t_perm, ctx->t_lcol,
-                                                                   ctx->A32, reinterpret_cast<float4 *>(ctx->t_rec));
+        const int64_t gr = (ctx->nslot + 255) / 256;
+        if (ctx->tile_mma)
+            k_tile_records<D><<<gr, 256, 0, s>>>(ctx->nslot, nnz, ctx->tile_xs, ctx->t_perm, ctx->t_lcol, ctx->A32,
+                                                 reinterpret_cast<float4 *>(ctx->t_rec));
+        else
+            k_pair_records<D><<<gr, 256, 0, s>>>(ctx->nslot, nnz, ctx->tile_rows / 2, ctx->tile_xs, ctx->t_perm,
+                                                 ctx->t_perm1, ctx->t_lcol, ctx->A32,
+                                                 reinterpret_cast<float4 *>(ctx->t_rec));
         CU_LAUNCH(ctx);
     }
     int64_t tot = nnz * m;
@@ -2102,11 +2287,9 @@ mlpg_status build_blocks(mlpg_ctx *ctx) {
     std::sort(key.begin(), key.end());
     ctx->nblk = (n + kB - 1) / kB;
     std::vector<int32_t> member(ctx->nblk * kB, -1), bof(n);
-    ctx->h_order.resize(n);
     for (int64_t r = 0; r < n; ++r) {
         member[r] = key[r].second;
         bof[key[r].second] = (int32_t)r;
-        ctx->h_order[r] = key[r].second;
     }
     MLPG_TRY(dalloc(ctx, &ctx->bmember, ctx->nblk * kB));
     MLPG_TRY(dalloc(ctx, &ctx->bof, n));

@@ -1,7 +1,7 @@
 // Row tiles of the batched transport operator apply (host, once per point set).
 //
-// The rows of the overlap pattern are taken in the Morton order of their
-// points and cut into tiles of `rows_per_tile` consecutive rows, so that the
+// The rows of the overlap pattern are taken in a spatial order of their points
+// (order.cpp) and cut into tiles of `rows_per_tile` consecutive rows, so that the
 // rows of one tile are close in space and share most of their overlap
 // partners.  For every tile:
 //   * the halo: the sorted union of the pattern columns of its rows, whose
@@ -118,6 +118,94 @@ int64_t build_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, const 
                     pe[s] = p;
                     le[s] = pos[col[p]];
                 }
+            }
+        }
+    });
+    return nslot;
+}
+
+// ---------------------------------------------------------------------------
+// Row tiles of row pairs.  Rows 2s and 2s + 1 of a tile form pair s, whose
+// entry list is the sorted union of the two rows' columns: one slot per union
+// column holds both rows' entries (-1 where a row has none), so that the value
+// of X at that column is fetched once for two rows.  Entry k of pair s sits at
+// slot base[t] + k * pairs + s for k < width[t] (the tile's longest union,
+// rounded up to width_multiple); plen[t * pairs + s] is the pair's own length.
+// ---------------------------------------------------------------------------
+int64_t build_pair_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, const int32_t *order,
+                         int rows_per_tile, int width_multiple, bool with_halo, PairTileLayout &out) {
+    const int64_t TR = rows_per_tile, TP = TR / 2;
+    out = PairTileLayout{};
+    out.rows_per_tile = rows_per_tile;
+    out.ntile = (n + TR - 1) / TR;
+    const int64_t ntile = out.ntile;
+    out.base.assign(ntile + 1, 0);
+    out.width.assign(ntile, 0);
+    out.row.assign(ntile * TR, -1);
+    out.plen.assign(ntile * TP, 0);
+    out.hptr.assign(ntile + 1, 0);
+    const int T = tile_threads(n, ntile);
+    auto merge = [rowptr, col](int32_t i, int32_t j, auto &&f) {   // f(entry of i or -1, entry of j or -1, column)
+        int32_t a = i >= 0 ? rowptr[i] : 0, b = j >= 0 ? rowptr[j] : 0;
+        const int32_t ae = i >= 0 ? rowptr[i + 1] : 0, be = j >= 0 ? rowptr[j + 1] : 0;
+        while (a < ae || b < be) {
+            const int32_t ca = a < ae ? col[a] : INT32_MAX, cb = b < be ? col[b] : INT32_MAX;
+            const int32_t c = std::min(ca, cb);
+            f(ca == c ? a : -1, cb == c ? b : -1, c);
+            a += ca == c;
+            b += cb == c;
+        }
+    };
+    std::vector<std::vector<int32_t>> halo(with_halo ? ntile : 0);
+    over_tiles(ntile, T, [&](int64_t t0, int64_t t1, int) {
+        std::vector<int64_t> stamp(with_halo ? n : 0, -1);
+        for (int64_t t = t0; t < t1; ++t) {
+            int32_t w = 0;
+            for (int64_t s = 0; s < TR && t * TR + s < n; ++s) out.row[t * TR + s] = order[t * TR + s];
+            for (int64_t s = 0; s < TP; ++s) {
+                int32_t len = 0;
+                merge(out.row[t * TR + 2 * s], out.row[t * TR + 2 * s + 1], [&](int32_t, int32_t, int32_t c) {
+                    ++len;
+                    if (with_halo && stamp[c] != t) {
+                        stamp[c] = t;
+                        halo[t].push_back(c);
+                    }
+                });
+                out.plen[t * TP + s] = len;
+                w = std::max(w, len);
+            }
+            if (with_halo) std::sort(halo[t].begin(), halo[t].end());
+            out.width[t] = (w + width_multiple - 1) / width_multiple * width_multiple;
+        }
+    });
+    for (int64_t t = 0; t < ntile; ++t) {
+        const int64_t h = with_halo ? (int64_t)halo[t].size() : 0;
+        out.base[t + 1] = out.base[t] + (int64_t)out.width[t] * TP;
+        out.hptr[t + 1] = out.hptr[t] + h;
+        out.max_halo = std::max<int64_t>(out.max_halo, h);
+        out.max_width = std::max<int32_t>(out.max_width, out.width[t]);
+    }
+    out.hcol.resize(out.hptr[ntile]);
+    const int64_t nslot = out.base[ntile];
+    out.perm0.assign(nslot, -1);
+    out.perm1.assign(nslot, -1);
+    out.lcol.assign(nslot, 0);
+    over_tiles(ntile, T, [&](int64_t t0, int64_t t1, int) {
+        std::vector<int32_t> pos(with_halo ? n : 0, 0);
+        for (int64_t t = t0; t < t1; ++t) {
+            if (with_halo) {
+                const std::vector<int32_t> &h = halo[t];
+                std::copy(h.begin(), h.end(), out.hcol.begin() + out.hptr[t]);
+                for (int32_t k = 0; k < (int32_t)h.size(); ++k) pos[h[k]] = k;
+            }
+            for (int64_t s = 0; s < TP; ++s) {
+                int64_t e = out.base[t] + s;
+                merge(out.row[t * TR + 2 * s], out.row[t * TR + 2 * s + 1], [&](int32_t a, int32_t b, int32_t c) {
+                    out.perm0[e] = a;
+                    out.perm1[e] = b;
+                    out.lcol[e] = with_halo ? pos[c] : c;
+                    e += TP;
+                });
             }
         }
     });
