@@ -2,7 +2,8 @@
 // outermost integration of the SUPG transport forms (Sec. 2.2, Sec. 3.2,
 // Alg. 1, Eq. weak-transport), 2D.
 //
-// One CTA integrates one cell i.  The functions that can reach the cell (at
+// The linear functions (the default) have a kernel of their own, k_assemble_2d_lin.
+// Orders 0 and 2: one CTA integrates one cell i.  The functions that can reach the cell (at
 // most MLPG_MAX_CELL_FUNCS, drawn from the overlap row of i) are staged in
 // shared memory.  Quadrature points are generated in the kernel from the cell
 // polygon: fan triangles (x_i, v_k, v_{k+1}) with the conical-product rule
@@ -17,8 +18,10 @@
 // per-cell sums are added into the CSR pattern at the end.
 // Materials are constant over the cell, so sigma-weighted forms are the cell
 // sums times sigma_t(i), sigma_s(i).
+#include <algorithm>
 #include <cmath>
 
+#include "fixed_sum.cuh"
 #include "internal.h"
 
 namespace mlpg {
@@ -27,7 +30,6 @@ namespace {
 
 constexpr int kMaxS = MLPG_MAX_CELL_FUNCS;
 constexpr int kThreads = 512;
-constexpr int kChunk = 64;                                       // points per RK chunk
 constexpr int kMaxTri = 64;   // reference triangle rule size cap
 constexpr int kMaxLine = 16;
 
@@ -123,93 +125,13 @@ __device__ bool rk_point(double px, double py, double s, int S, const double *fx
     return true;
 }
 
-// RK functions at (px, py) for the assembly kernel, writing into the shared
-// table (U, Ux, Uy at [a * stride]).  The first pass stores W and its
-// gradient in the table slots so that the second pass does not repeat the
-// square roots; support tests compare squared distances.  Returns the
-// support mask (bit a set when function a is supported), or 0 when the
-// moment matrix is not positive definite.
-__device__ uint64_t rk_point_tab(double px, double py, double s, int S, const double *fx, const double *fy,
-                                 const double *fR2, const double *finvh, const double *fV, double *U, double *Ux,
-                                 double *Uy, int stride) {
-    // M, Dx, Dy are symmetric: their six distinct entries (0,0) (0,1) (0,2) (1,1) (1,2) (2,2)
-    constexpr int EI[6] = {0, 0, 0, 1, 1, 2}, EJ[6] = {0, 1, 2, 1, 2, 2};
-    double m[6] = {0}, mx[6] = {0}, my[6] = {0};
-    const double is = 1.0 / s;
-    uint64_t mask = 0;
-    for (int a = 0; a < S; ++a) {
-        const double dx = px - fx[a], dy = py - fy[a];
-        const double r2 = dx * dx + dy * dy;
-        if (!(r2 < fR2[a])) {
-            U[a * stride] = 0.0;
-            Ux[a * stride] = 0.0;
-            Uy[a * stride] = 0.0;
-            continue;
-        }
-        mask |= uint64_t(1) << a;
-        const double ir = r2 > 0.0 ? rsqrt(r2) : 0.0;
-        const double chi = r2 * ir * finvh[a];
-        const double W = spline_w(chi);
-        const double g = spline_dw(chi) * finvh[a] * ir;
-        const double Wx = g * dx, Wy = g * dy, v = fV[a];
-        U[a * stride] = W;
-        Ux[a * stride] = Wx;
-        Uy[a * stride] = Wy;
-        const double P[3] = {1.0, dx * is, dy * is};
-        const double vW = v * W, vWx = v * Wx, vWy = v * Wy;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-            const int i = EI[e], j = EJ[e];
-            const double pp = P[i] * P[j];
-            const double ex = ((i == 1) * P[j] + (j == 1) * P[i]) * is;
-            const double ey = ((i == 2) * P[j] + (j == 2) * P[i]) * is;
-            m[e] += vW * pp;
-            mx[e] += ex * vW + pp * vWx;
-            my[e] += ey * vW + pp * vWy;
-        }
-    }
-    // M = L L^T; the triangular solves multiply by the reciprocal pivots
-    double L00 = m[0];
-    if (!(L00 > 0.0)) return 0;
-    L00 = sqrt(L00);
-    const double r00 = 1.0 / L00;
-    const double L10 = m[1] * r00, L20 = m[2] * r00;
-    const double d1 = m[3] - L10 * L10;
-    if (!(d1 > 1e-14 * m[3])) return 0;
-    const double L11 = sqrt(d1), r11 = 1.0 / L11;
-    const double L21 = (m[4] - L20 * L10) * r11;
-    const double d2 = m[5] - L20 * L20 - L21 * L21;
-    if (!(d2 > 1e-14 * m[5])) return 0;
-    const double r22 = 1.0 / sqrt(d2);
-    auto solve = [&](double b0, double b1, double b2, double *o) {
-        double y0 = b0 * r00, y1 = (b1 - L10 * y0) * r11, y2 = (b2 - L20 * y0 - L21 * y1) * r22;
-        o[2] = y2 * r22;
-        o[1] = (y1 - L21 * o[2]) * r11;
-        o[0] = (y0 - L10 * o[1] - L20 * o[2]) * r00;
-    };
-    double C[3], Cx[3], Cy[3];
-    solve(1.0, 0.0, 0.0, C);
-    solve(-(mx[0] * C[0] + mx[1] * C[1] + mx[2] * C[2]), -(mx[1] * C[0] + mx[3] * C[1] + mx[4] * C[2]),
-          -(mx[2] * C[0] + mx[4] * C[1] + mx[5] * C[2]), Cx);
-    solve(-(my[0] * C[0] + my[1] * C[1] + my[2] * C[2]), -(my[1] * C[0] + my[3] * C[1] + my[4] * C[2]),
-          -(my[2] * C[0] + my[4] * C[1] + my[5] * C[2]), Cy);
-    for (uint64_t bits = mask; bits; bits &= bits - 1) {
-        const int a = __ffsll((long long)bits) - 1;
-        const double W = U[a * stride], Wx = Ux[a * stride], Wy = Uy[a * stride];
-        const double P1 = (px - fx[a]) * is, P2 = (py - fy[a]) * is;
-        const double PC = C[0] + P1 * C[1] + P2 * C[2];
-        U[a * stride] = W * PC;
-        Ux[a * stride] = W * (C[1] * is + Cx[0] + P1 * Cx[1] + P2 * Cx[2]) + PC * Wx;
-        Uy[a * stride] = W * (C[2] * is + Cy[0] + P1 * Cy[1] + P2 * Cy[2]) + PC * Wy;
-    }
-    return mask;
-}
-
-// RK functions of order ORD (0 or 2; order 1 is rk_point_tab) at (px, py):
-// the basis is every monomial of xi = (p - x_j)/s up to degree ORD, ordered
-// 1, xi_x, xi_y, xi_x^2, xi_x xi_y, xi_y^2.  Same table layout, first-pass use
-// of the table and return value (support mask, 0 when the moment matrix is
-// not positive definite) as rk_point_tab.
+// RK functions of order ORD (0 or 2; the linear ones are in k_assemble_2d_lin) at
+// (px, py), into the shared table (U, Ux, Uy at [a * stride]): the basis is every
+// monomial of xi = (p - x_j)/s up to degree ORD, ordered 1, xi_x, xi_y, xi_x^2,
+// xi_x xi_y, xi_y^2.  The first pass stores W and its gradient in the table slots so
+// that the second does not repeat the square roots; support tests compare squared
+// distances.  Returns the support mask (bit a set when function a is supported), or 0
+// when the moment matrix is not positive definite.
 template <int ORD>
 __device__ uint64_t rk_point_gen(double px, double py, double s, int S, const double *fx, const double *fy,
                                  const double *fR2, const double *finvh, const double *fV, double *U, double *Ux,
@@ -358,8 +280,8 @@ struct AsmArgs {
 };
 
 // mats layout: 0 M0, 1 Mt, 2 Ms, 3-4 G, 5-6 Gt, 7-8 Gs, 9-12 K (xx, xy, yx, yy), 13-16 S_f
-// ORD: RK order; MAXS: functions reaching one cell (<= 64, one mask word);
-// CHUNK: quadrature points per RK pass.  The linear path is <1, 40, 64>.
+// ORD: RK order (0 or 2); MAXS: functions reaching one cell (<= 64, one mask word);
+// CHUNK: quadrature points per RK pass.
 template <int ORD, int MAXS, int CHUNK>
 __global__ void __launch_bounds__(kThreads, 1) k_assemble_2d(AsmArgs A) {
     // unordered pairs a <= b of the staged functions: M0, K^xx, K^yy and the face forms are
@@ -482,12 +404,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_assemble_2d(AsmArgs A) {
                 int f = -A.labels[c0 + e] - 1;
                 fslot = (f == face_slot[0]) ? 0 : 1;
             }
-            uint64_t mk;
-            if constexpr (ORD == 1)
-                mk = rk_point_tab(px, py, scale, nS, fx, fy, fR2, finvh, fV, tU + tid, tUx + tid, tUy + tid, kChunk);
-            else
-                mk = rk_point_gen<ORD>(px, py, scale, nS, fx, fy, fR2, finvh, fV, tU + tid, tUx + tid, tUy + tid,
-                                       kChunk);
+            const uint64_t mk = rk_point_gen<ORD>(px, py, scale, nS, fx, fy, fR2, finvh, fV, tU + tid, tUx + tid,
+                                                  tUy + tid, kChunk);
             if (!mk) atomicOr(A.flag, 1);
             tMask[tid] = mk;
             tW[tid] = wq;
@@ -592,6 +510,443 @@ __global__ void __launch_bounds__(kThreads, 1) k_assemble_2d(AsmArgs A) {
         if (vqy != 0.0) atomicAdd(&A.vecs[2 * n + a], qi * vqy);
         if (face_slot[0] >= 0 && vb0 != 0.0) atomicAdd(&A.vecs[(3 + face_slot[0]) * n + a], vb0);
         if (face_slot[1] >= 0 && vb1 != 0.0) atomicAdd(&A.vecs[(3 + face_slot[1]) * n + a], vb1);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Volume and surface forms with the linear RK functions (the default): one CTA per
+// cell, its points in chunks of at most 64 (one mask word per function).  Per chunk:
+//   1. each function's point mask and each point's function list (distances in
+//      FP32 from the generator, FP64 where that could decide wrongly);
+//   2. RK functions, two lanes per point over the point's own list (about 13 of the
+//      35 functions that reach the cell); the derivative moments are the third-order
+//      moments of the kernel's radial derivative (9 sums instead of 12);
+//   3. the table sqrt(w) (U, U_x, U_y) in fixed point, 54 bits below the chunk's
+//      largest U and largest derivative;
+//   4. every unordered pair a <= b sums the nine products over the points both
+//      support, in 64-bit integers (fixed_sum.cuh), and adds them to the pattern's
+//      upper entry; G(b, a) goes to six buffers of its own, and k_mirror_2d fills the lower
+//      entries (M0, K and S are each other's transposes) and applies the volumes V_b.
+// Points on box edges follow in chunks of their own, in FP64 (S_f and B_f only).
+//
+// What bounds it: the FP64 units (1.6 operations per clock and SM), in the RK
+// functions; before, every warp of a cell ran twelve FP64 operations for each point
+// at which any of its 32 pairs was supported, and the RK functions one point per thread
+// on 64 of 512 threads.  128^2 points: 40.4 -> 9.9 ms (FP64 pipe 78 % busy).
+// ---------------------------------------------------------------------------
+constexpr int kLinThreads = 128, kLinPts = 64;
+constexpr int kLinEntries = 2048;   // table entries (points x functions) of 24 bytes: four CTAs per SM
+
+__global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, double *__restrict__ gt) {
+    __shared__ double fx[kMaxS], fy[kMaxS], fR2[kMaxS], finvh[kMaxS], fV[kMaxS];
+    __shared__ float ffx[kMaxS], ffy[kMaxS], ffR2[kMaxS], fslack[kMaxS], qfx[kLinPts], qfy[kLinPts];
+    __shared__ double qx[kLinPts], qy[kLinPts], qsw[kLinPts];
+    __shared__ int qfs[kLinPts], pcnt[kLinPts];
+    __shared__ int32_t fidx[kMaxS];
+    __shared__ uint64_t fmask[kMaxS];
+    __shared__ uint8_t plist[kLinPts][kMaxS];
+    __shared__ int wcnt[kLinThreads / 32];
+    __shared__ int S_sh;
+    __shared__ unsigned top[2];
+    extern __shared__ __align__(16) double lin_tab[];
+    const int64_t i = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double xi = A.x[2 * i], yi = A.x[2 * i + 1];
+    const int32_t c0 = A.cptr[i], nv = A.cptr[i + 1] - c0;
+    const double *vt = A.verts + 2 * (int64_t)c0;
+    // radius of the cell around its generator, the boundary edges and the faces it touches (every thread)
+    double rc2 = 0.0;
+    int nbe = 0, nf = 0, face_slot[2] = {-1, -1};
+    for (int k = 0; k < nv; ++k) {
+        const int32_t L = A.labels[c0 + k];
+        if (L < 0 && L != kLabelExtent) {
+            const int f = -L - 1;
+            ++nbe;
+            if (face_slot[0] != f && face_slot[1] != f) {
+                if (nf == 0) face_slot[0] = f;
+                else if (nf == 1) face_slot[1] = f;
+                ++nf;
+            }
+        }
+    }
+    for (int k = lane; k < nv; k += 32) {
+        const double dx = vt[2 * k] - xi, dy = vt[2 * k + 1] - yi;
+        rc2 = fmax(rc2, dx * dx + dy * dy);
+    }
+    for (int o = 16; o > 0; o >>= 1) rc2 = fmax(rc2, __shfl_xor_sync(0xffffffffu, rc2, o));
+    const double rc = sqrt(rc2);
+    if (tid == 0) {
+        S_sh = 0;
+        if (nf > 2) atomicOr(A.flag, 4);
+    }
+    __syncthreads();
+    // the functions that can reach the cell, in overlap-row order (ascending)
+    const int32_t r0 = A.rowptr[i], rl = A.rowptr[i + 1] - r0;
+    for (int base = 0; base < rl; base += kLinThreads) {
+        const int c = base + tid;
+        bool in = false;
+        int32_t j = 0;
+        double xj = 0.0, yj = 0.0, Rj = 0.0;
+        if (c < rl) {
+            j = A.col[r0 + c];
+            xj = A.x[2 * (int64_t)j];
+            yj = A.x[2 * (int64_t)j + 1];
+            Rj = A.R[j];
+            const double dx = xj - xi, dy = yj - yi;
+            in = sqrt(dx * dx + dy * dy) < Rj + rc * (1.0 + 1e-12);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) wcnt[warp] = __popc(bal);
+        __syncthreads();
+        int off = S_sh;
+        for (int w = 0; w < warp; ++w) off += wcnt[w];
+        const int slot = off + __popc(bal & ((1u << lane) - 1u));
+        if (in && slot < kMaxS) {
+            fidx[slot] = j;
+            fx[slot] = xj;
+            fy[slot] = yj;
+            fR2[slot] = Rj * Rj;
+            finvh[slot] = 2.0 / Rj;
+            fV[slot] = A.V[j];
+            const float dx = (float)(xj - xi), dy = (float)(yj - yi), r2 = (float)Rj * (float)Rj;
+            ffx[slot] = dx;
+            ffy[slot] = dy;
+            ffR2[slot] = r2;
+            // coordinates rounded to 2^-24 of at most a few R: 1e-4 is far outside
+            fslack[slot] = 1e-4f * (dx * dx + dy * dy + r2);
+        }
+        __syncthreads();
+        if (tid == 0)
+            for (int w = 0; w < kLinThreads / 32; ++w) S_sh += wcnt[w];
+        __syncthreads();
+    }
+    const int S = S_sh;
+    if (S > kMaxS) {   // (block-uniform) too many functions reach the cell
+        if (tid == 0) atomicOr(A.flag, 2);
+        return;
+    }
+    const double s = 0.5 * A.R[i], is = 1.0 / s;
+    const int nP = S * (S + 1) / 2;
+    const int nvol = nv * A.ntri, ntot = nvol + nbe * A.nline;
+    const int cap = min(kLinPts, kLinEntries / S);
+    const int nvc = (nvol + cap - 1) / cap, vstep = (nvol + nvc - 1) / nvc;   // even volume chunks
+    double vq0 = 0.0, vqx = 0.0, vqy = 0.0, vb0 = 0.0, vb1 = 0.0;   // vectors of function tid
+    const double st = A.sig_t[i], ss = A.sig_s[i];
+    const int64_t nnz = A.nnz, n = A.n;
+    for (int base = 0; base < ntot;) {
+        const bool vol = base < nvol;
+        const int P = vol ? min(vstep, nvol - base) : min(cap, ntot - base);
+        double *tabu = lin_tab;                                            // [P][S] u
+        double2 *tabd = reinterpret_cast<double2 *>(lin_tab + ((P * S + 1) & ~1));   // [P][S] (u_x, u_y)
+        if (tid < P) {
+            const int k = base + tid;
+            double dx, dy, wq;   // relative to the generator
+            int fs = -1;
+            if (vol) {
+                const int e = k / A.ntri, r = k - e * A.ntri, e1 = e + 1 == nv ? 0 : e + 1;
+                const double ax = vt[2 * e] - xi, ay = vt[2 * e + 1] - yi, bx = vt[2 * e1] - xi, by = vt[2 * e1 + 1] - yi;
+                dx = ax * c_tri_xi[2 * r] + bx * c_tri_xi[2 * r + 1];
+                dy = ay * c_tri_xi[2 * r] + by * c_tri_xi[2 * r + 1];
+                wq = c_tri_w[r] * fabs(ax * by - ay * bx);
+                qx[tid] = xi + dx;
+                qy[tid] = yi + dy;
+            } else {
+                const int kb = k - nvol, eb = kb / A.nline, r = kb - eb * A.nline;
+                int e = -1, c = -1;   // eb-th boundary edge of the cell
+                for (int t = 0; t < nv; ++t) {
+                    const int32_t L = A.labels[c0 + t];
+                    if (L < 0 && L != kLabelExtent && ++c == eb) { e = t; break; }
+                }
+                const int e1 = e + 1 == nv ? 0 : e + 1;
+                const double p0x = vt[2 * e], p0y = vt[2 * e + 1], ex = vt[2 * e1] - p0x, ey = vt[2 * e1 + 1] - p0y;
+                const double s01 = 0.5 * (c_line_t[r] + 1.0);
+                qx[tid] = p0x + ex * s01;
+                qy[tid] = p0y + ey * s01;
+                wq = c_line_w[r] * 0.5 * sqrt(ex * ex + ey * ey);
+                dx = qx[tid] - xi;
+                dy = qy[tid] - yi;
+                fs = -A.labels[c0 + e] - 1 == face_slot[0] ? 0 : 1;
+            }
+            qfx[tid] = (float)dx;
+            qfy[tid] = (float)dy;
+            qsw[tid] = sqrt(wq);
+            qfs[tid] = fs;
+        }
+        if (tid == 0) top[0] = top[1] = 0;
+        for (int k = tid; k < P * S; k += kLinThreads) {
+            tabu[k] = 0.0;
+            tabd[k] = make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+        // 1. masks: four lanes per function
+        for (int f0 = 0; f0 < S; f0 += kLinThreads / 4) {
+            const int a = f0 + (tid >> 2);
+            unsigned lo = 0, hi = 0;
+            if (a < S) {
+                const float ax = ffx[a], ay = ffy[a], R2 = ffR2[a], slack = fslack[a];
+                for (int p = tid & 3; p < P; p += 4) {
+                    const float dx = qfx[p] - ax, dy = qfy[p] - ay, r2 = dx * dx + dy * dy;
+                    bool sup = r2 < R2;
+                    if (fabsf(r2 - R2) <= slack) {
+                        const double ex = qx[p] - fx[a], ey = qy[p] - fy[a];
+                        sup = ex * ex + ey * ey < fR2[a];
+                    }
+                    if (p < 32) lo |= (unsigned)sup << p;
+                    else hi |= (unsigned)sup << (p - 32);
+                }
+            }
+            lo |= __shfl_xor_sync(0xffffffffu, lo, 1);
+            hi |= __shfl_xor_sync(0xffffffffu, hi, 1);
+            lo |= __shfl_xor_sync(0xffffffffu, lo, 2);
+            hi |= __shfl_xor_sync(0xffffffffu, hi, 2);
+            if (a < S && (tid & 3) == 0) fmask[a] = (uint64_t)hi << 32 | lo;
+        }
+        __syncthreads();
+        if (tid < P) {
+            int c = 0;
+            for (int a = 0; a < S; ++a)
+                if ((fmask[a] >> tid) & 1) plist[tid][c++] = (uint8_t)a;
+            pcnt[tid] = c;
+        }
+        __syncthreads();
+        // 2. RK functions: two lanes per point, 16 points per warp
+        unsigned mx0 = 0, mx1 = 0;   // high words of the largest |sqrt(w) u|, |sqrt(w) du|
+        for (int p0 = warp * 16; p0 < P; p0 += kLinThreads / 2) {
+            const int p = min(p0 + (lane >> 1), P - 1), l2 = lane & 1;   // spare lanes repeat the last point
+            const bool mine = p0 + (lane >> 1) < P;
+            const int cnt = pcnt[p];
+            const double px = qx[p], py = qy[p];
+            double m[6], t[9];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) m[k] = 0.0;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) t[k] = 0.0;
+            for (int k = l2; k < cnt; k += 2) {
+                const int a = plist[p][k];
+                const double dx = px - fx[a], dy = py - fy[a], r2 = dx * dx + dy * dy;
+                const double ir = r2 > 0.0 ? rsqrt(r2) : 0.0, ih = finvh[a], chi = r2 * ir * ih;
+                const double W = spline_w(chi), g = spline_dw(chi) * ih * ir, v = fV[a];
+                if (mine) tabd[p * S + a] = make_double2(W, g);
+                const double aw = v * W, bw = v * g * s, X = dx * is, Y = dy * is;
+                const double ax = aw * X, ay = aw * Y;
+                m[0] += aw; m[1] += ax; m[2] += ay;
+                m[3] += ax * X; m[4] += ax * Y; m[5] += ay * Y;
+                const double bx = bw * X, by = bw * Y, bxx = bx * X, bxy = bx * Y, byy = by * Y;
+                t[0] += bx; t[1] += by; t[2] += bxx; t[3] += bxy; t[4] += byy;
+                t[5] += bxx * X; t[6] += bxx * Y; t[7] += bxy * Y; t[8] += byy * Y;
+            }
+#pragma unroll
+            for (int k = 0; k < 6; ++k) m[k] += __shfl_xor_sync(0xffffffffu, m[k], 1);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], 1);
+            // M = L L^T with reciprocal pivots
+            bool ok = m[0] > 0.0;
+            const double i0 = rsqrt(m[0]), L10 = m[1] * i0, L20 = m[2] * i0;
+            const double d1 = m[3] - L10 * L10;
+            ok = ok && d1 > 1e-14 * m[3];
+            const double i1 = rsqrt(d1), L21 = (m[4] - L20 * L10) * i1;
+            const double d2 = m[5] - L20 * L20 - L21 * L21;
+            ok = ok && d2 > 1e-14 * m[5];
+            const double i2 = rsqrt(d2);
+            auto solve = [&](double b0, double b1, double b2, double *r) {
+                const double y0 = b0 * i0, y1 = (b1 - L10 * y0) * i1, y2 = (b2 - L20 * y0 - L21 * y1) * i2;
+                r[2] = y2 * i2;
+                r[1] = (y1 - L21 * r[2]) * i1;
+                r[0] = (y0 - L10 * r[1] - L20 * r[2]) * i0;
+            };
+            double C[3], Cx[3], Cy[3];
+            solve(1.0, 0.0, 0.0, C);
+            // C_c = -M^-1 D_c C, D_c C [i] = ((i == c) + m_i C_c) / s + sum_j T_c[i][j] C_j (M C = e_1 takes the
+            // first term's sum); T_c[i][j] the third-order moments
+            solve(-(m[0] * C[1] * is + t[0] * C[0] + t[2] * C[1] + t[3] * C[2]),
+                  -((1.0 + m[1] * C[1]) * is + t[2] * C[0] + t[5] * C[1] + t[6] * C[2]),
+                  -(m[2] * C[1] * is + t[3] * C[0] + t[6] * C[1] + t[7] * C[2]), Cx);
+            solve(-(m[0] * C[2] * is + t[1] * C[0] + t[3] * C[1] + t[4] * C[2]),
+                  -(m[1] * C[2] * is + t[3] * C[0] + t[6] * C[1] + t[7] * C[2]),
+                  -((1.0 + m[2] * C[2]) * is + t[4] * C[0] + t[7] * C[1] + t[8] * C[2]), Cy);
+            if (!ok && mine && l2 == 0) atomicOr(A.flag, 1);
+            const double sw = qsw[p], gx = C[1] * is + Cx[0], gy = C[2] * is + Cy[0];
+            for (int k = l2; k < cnt && mine; k += 2) {
+                const int a = plist[p][k];
+                const double dx = px - fx[a], dy = py - fy[a], X = dx * is, Y = dy * is;
+                const double2 wg = tabd[p * S + a];
+                const double W = wg.x * sw, PC = C[0] + X * C[1] + Y * C[2], h = PC * (wg.y * sw);
+                const double u = W * PC;
+                const double ux = W * (gx + X * Cx[1] + Y * Cx[2]) + h * dx, uy = W * (gy + X * Cy[1] + Y * Cy[2]) + h * dy;
+                tabu[p * S + a] = ok ? u : 0.0;
+                tabd[p * S + a] = ok ? make_double2(ux, uy) : make_double2(0.0, 0.0);
+                if (ok) {
+                    mx0 = max(mx0, (unsigned)__double2hiint(u) & 0x7fffffffu);
+                    mx1 = max(mx1, max((unsigned)__double2hiint(ux) & 0x7fffffffu, (unsigned)__double2hiint(uy) & 0x7fffffffu));
+                }
+            }
+        }
+        mx0 = __reduce_max_sync(0xffffffffu, mx0);
+        mx1 = __reduce_max_sync(0xffffffffu, mx1);
+        if (lane == 0) {
+            atomicMax(&top[0], mx0);
+            atomicMax(&top[1], mx1);
+        }
+        __syncthreads();
+        if (tid < S)   // vectors, before the table changes to fixed point
+            for (uint64_t bits = fmask[tid]; bits; bits &= bits - 1) {
+                const int p = __ffsll((long long)bits) - 1;
+                const double sw = qsw[p], u = sw * tabu[p * S + tid];
+                if (vol) {
+                    const double2 d = tabd[p * S + tid];
+                    vq0 += u;
+                    vqx += sw * d.x;
+                    vqy += sw * d.y;
+                } else if (qfs[p] == 0) {
+                    vb0 += u;
+                } else {
+                    vb1 += u;
+                }
+            }
+        // 3. fixed point, in place
+        const int x0 = top_exp(top[0]), x1 = top_exp(top[1]);
+        int2 *iu = reinterpret_cast<int2 *>(tabu);
+        int4 *id = reinterpret_cast<int4 *>(tabd);
+        if (vol) {
+            __syncthreads();
+            const double sc0 = ldexp(1.0, 54 - x0), sc1 = ldexp(1.0, 54 - x1);   // 64 products of 2^108 fit 64 bits
+            for (int k = tid; k < P * S; k += kLinThreads) {
+                const int p = k / S, a = k - p * S;
+                if (!((fmask[a] >> p) & 1)) continue;   // zero already
+                const double u = tabu[k];
+                const double2 d = tabd[k];
+                iu[k] = fixed_parts(u, sc0);
+                const int2 ix = fixed_parts(d.x, sc1), iy = fixed_parts(d.y, sc1);
+                id[k] = make_int4(ix.x, ix.y, iy.x, iy.y);
+            }
+            __syncthreads();
+        }
+        // 4. pairs.  value = 2^(e_a + e_b) 2^-108 (A 2^56 + B 2^28) = 2^(e_a + e_b - 56) (16 A + B / 2^24)
+        const double f00 = ldexp(1.0, 2 * x0 - 56), f01 = ldexp(1.0, x0 + x1 - 56), f11 = ldexp(1.0, 2 * x1 - 56);
+        for (int pb = warp * 32; pb < nP; pb += kLinThreads) {   // whole warps: the reductions name every lane
+            const int pr = pb + lane;
+            int a = 0, b = 0;
+            uint64_t mask = 0;
+            if (pr < nP) {   // row a of the upper triangle: a S - a (a - 1) / 2 <= pr
+                a = (int)(((float)(2 * S + 1) - sqrtf((float)((2 * S + 1) * (2 * S + 1) - 8 * pr))) * 0.5f);
+                a = max(0, min(a, S - 1));
+                while (a > 0 && a * S - a * (a - 1) / 2 > pr) --a;
+                while ((a + 1) * S - (a + 1) * a / 2 <= pr) ++a;
+                b = a + pr - (a * S - a * (a - 1) / 2);
+                mask = fmask[a] & fmask[b];
+            }
+            const uint64_t any = (uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)mask) |
+                                 ((uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)(mask >> 32)) << 32);
+            if (!any) continue;
+            int pos = -1;
+            if (mask) {
+                pos = find_col(A.col, A.rowptr[fidx[a]], A.rowptr[fidx[a] + 1], fidx[b]);
+                if (pos < 0) atomicOr(A.flag, 8);
+            }
+            if (!vol) {
+                double f[2] = {0.0, 0.0};
+                for (uint64_t bits = mask; bits; bits &= bits - 1) {
+                    const int p = __ffsll((long long)bits) - 1;
+                    const double w = tabu[p * S + a] * tabu[p * S + b];
+                    if (qfs[p] == 0) f[0] += w;
+                    else f[1] += w;
+                }
+                if (pos < 0) continue;
+                if (f[0] != 0.0) atomicAdd(&A.mats[(13 + face_slot[0]) * nnz + pos], f[0]);
+                if (f[1] != 0.0) atomicAdd(&A.mats[(13 + face_slot[1]) * nnz + pos], f[1]);
+                continue;
+            }
+            long long hh[9], hl[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) hh[k] = hl[k] = 0;
+            for (uint64_t bits = any; bits; bits &= bits - 1) {
+                const int p = __ffsll((long long)bits) - 1;
+                const int2 ua = iu[p * S + a], ub = iu[p * S + b];
+                const int4 da = id[p * S + a], db = id[p * S + b];
+                const int ah[3] = {ua.x, da.x, da.z}, al[3] = {ua.y, da.y, da.w};
+                const int bh[3] = {ub.x, db.x, db.z}, bl[3] = {ub.y, db.y, db.w};
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        hh[3 * q + r] = mad_wide(ah[q], bh[r], hh[3 * q + r]);
+                        hl[3 * q + r] = mad_wide(ah[q], bl[r], hl[3 * q + r]);
+                        hl[3 * q + r] = mad_wide(al[q], bh[r], hl[3 * q + r]);
+                    }
+            }
+            if (pos < 0) continue;
+            double v[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k)
+                v[k] = (double)(hh[k] * 16 + (hl[k] >> 24)) * (k == 0 ? f00 : (k < 3 || k % 3 == 0 ? f01 : f11));
+            atomicAdd(&A.mats[pos], v[0]);
+            atomicAdd(&A.mats[nnz + pos], st * v[0]);
+            atomicAdd(&A.mats[2 * nnz + pos], ss * v[0]);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const double gab = v[3 * (1 + c)], gba = v[1 + c];   // d_c u_a u_b, u_a d_c u_b
+                atomicAdd(&A.mats[(3 + c) * nnz + pos], gab);
+                atomicAdd(&A.mats[(5 + c) * nnz + pos], st * gab);
+                atomicAdd(&A.mats[(7 + c) * nnz + pos], ss * gab);
+                atomicAdd(&gt[c * nnz + pos], gba);
+                atomicAdd(&gt[(2 + c) * nnz + pos], st * gba);
+                atomicAdd(&gt[(4 + c) * nnz + pos], ss * gba);
+#pragma unroll
+                for (int d = 0; d < 2; ++d) atomicAdd(&A.mats[(9 + 2 * c + d) * nnz + pos], v[3 * (1 + c) + 1 + d]);
+            }
+        }
+        __syncthreads();
+        base += P;
+    }
+    if (tid < S) {
+        const int32_t a = fidx[tid];
+        const double qi = A.q[i];
+        if (vq0 != 0.0) atomicAdd(&A.vecs[a], qi * vq0);
+        if (vqx != 0.0) atomicAdd(&A.vecs[n + a], qi * vqx);
+        if (vqy != 0.0) atomicAdd(&A.vecs[2 * n + a], qi * vqy);
+        if (face_slot[0] >= 0 && vb0 != 0.0) atomicAdd(&A.vecs[(3 + face_slot[0]) * n + a], vb0);
+        if (face_slot[1] >= 0 && vb1 != 0.0) atomicAdd(&A.vecs[(3 + face_slot[1]) * n + a], vb1);
+    }
+}
+
+// Lower entries from the upper ones of k_assemble_2d_lin, and the trial volumes: entry (i, j), i < j, holds the
+// sums without V_j; gt holds G(j, i).  Eight lanes per row.
+__global__ void k_mirror_2d(int64_t n, int64_t nnz, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                            const double *__restrict__ V, const double *__restrict__ gt, double *__restrict__ mats,
+                            int *__restrict__ flag) {
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    if (i >= n) return;
+    const double vi = V[i];
+    for (int32_t p = rowptr[i] + (threadIdx.x & 7); p < rowptr[i + 1]; p += 8) {
+        const int32_t j = col[p];
+        if (j < i) continue;
+        const double vj = V[j];
+        int q = p;
+        if (j != i) {
+            q = find_col(col, rowptr[j], rowptr[j + 1], (int32_t)i);
+            if (q < 0) { atomicOr(flag, 8); continue; }
+        }
+        auto both = [&](int f, double up, double low) {
+            mats[f * nnz + p] = up * vj;
+            if (q != p) mats[f * nnz + q] = low * vi;
+        };
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+            const double v = mats[f * nnz + p];
+            both(f, v, v);
+        }
+#pragma unroll
+        for (int f = 0; f < 6; ++f) both(3 + f, mats[(3 + f) * nnz + p], gt[f * nnz + p]);
+        double k[4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) k[f] = mats[(9 + f) * nnz + p];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) both(9 + f, k[f], k[2 * (f % 2) + f / 2]);
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const double v = mats[(13 + f) * nnz + p];
+            if (v != 0.0) both(13 + f, v, v);
+        }
     }
 }
 
@@ -710,9 +1065,33 @@ mlpg_status run_assemble(mlpg_ctx *ctx) {
         CU_LAUNCH(ctx);
         return MLPG_OK;
     };
-    if (ctx->opt.rk_order == 0) MLPG_TRY(run(k_assemble_2d<0, 48, 32>, 48, 32));
-    else if (ctx->opt.rk_order == 2) MLPG_TRY(run(k_assemble_2d<2, 48, 32>, 48, 32));
-    else MLPG_TRY(run(k_assemble_2d<1, kMaxS, kChunk>, kMaxS, kChunk));
+    if (ctx->opt.rk_order == 0) {
+        MLPG_TRY(run(k_assemble_2d<0, 48, 32>, 48, 32));
+    } else if (ctx->opt.rk_order == 2) {
+        MLPG_TRY(run(k_assemble_2d<2, 48, 32>, 48, 32));
+    } else {
+        struct Scratch {   // G of the lower entries, freed on every return (cudaFree waits for the device)
+            double *p = nullptr;
+            ~Scratch() {
+                if (p) cudaFree(p);
+            }
+        } gt;
+        if (cudaMalloc(&gt.p, sizeof(double) * 6 * std::max<int64_t>(ctx->nnz, 1)) != cudaSuccess) {
+            cudaGetLastError();
+            gt.p = nullptr;
+            return set_err(ctx, MLPG_ERR_OOM, "cudaMalloc failed: assembly buffers");
+        }
+        CU(ctx, cudaMemsetAsync(gt.p, 0, sizeof(double) * 6 * ctx->nnz, ctx->stream));
+        // u and (u_x, u_y) of kLinEntries entries, the first rounded to a 16-byte boundary
+        const size_t smem = sizeof(double) * (3 * (size_t)kLinEntries + 2);
+        CU(ctx, cudaFuncSetAttribute(k_assemble_2d_lin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_assemble_2d_lin<<<(unsigned)ctx->n, kLinThreads, smem, ctx->stream>>>(a, gt.p);
+        CU_LAUNCH(ctx);
+        k_mirror_2d<<<(unsigned)((ctx->n * 8 + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->nnz, ctx->rowptr, ctx->col,
+                                                                                   ctx->V, gt.p, ctx->mats, ctx->d_flag);
+        CU_LAUNCH(ctx);
+        return check_flag(ctx, "assembly");
+    }
     return check_flag(ctx, "assembly");
 }
 

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "fixed_sum.cuh"
 #include "internal.h"
 
 namespace mlpg {
@@ -476,20 +477,6 @@ __device__ __forceinline__ double quad_sum(double v) {   // over the four lanes 
     v += __shfl_xor_sync(0xffffffffu, v, 2);
     return v;
 }
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
-    long long d;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
-// v scaled to 56 bits: two signed parts, v = hi 2^28 + lo, |hi|, |lo| <= 2^27
-__device__ __forceinline__ int2 fixed_parts(double v, double scale) {
-    const long long x = __double2ll_rn(v * scale);
-    const int lo = (int)((unsigned)x << 4) >> 4;
-    return make_int2((int)((x - lo) >> 28), lo);
-}
-// 2^(55 - e) for the largest high word seen (|v| < 2^e); 1 for all zeros
-__device__ __forceinline__ int top_exp(unsigned hiword) { return hiword ? (int)(hiword >> 20) - 1022 : 0; }
-
 template <int NP>
 __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, const int2 *__restrict__ grp,
                                                                     double *__restrict__ gt,   // [9][nnz]: G, Gt, Gs of (b, a)
@@ -773,7 +760,7 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
     __syncthreads();
     // 3. fixed point, in place: (hi, lo) of u, u_x | u_y, u_z
     const int x0 = top_exp(top[0]), x1 = top_exp(top[1]);
-    const double sc0 = ldexp(1.0, 55 - x0), sc1 = ldexp(1.0, 55 - x1);
+    const double sc0 = ldexp(1.0, 55 - x0), sc1 = ldexp(1.0, 55 - x1);   // 48 products of 2^110 fit 64 bits
     int4 *itab = reinterpret_cast<int4 *>(smem_tab);
     for (int k = tid; k < P * S; k += kGrpThreads) {
         const int p = k / S, a = k - p * S;
