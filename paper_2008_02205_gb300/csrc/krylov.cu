@@ -491,19 +491,26 @@ __global__ void k_scale(int64_t n, int M, T *__restrict__ w, const double *__res
     w[e] = (T)((A)w[e] * ssc[m]);
 }
 
-// y = R^{-1} g per system (upper triangular part of the rotated Hessenberg);
-// also a float copy for FP32 vectors
+// y = R^{-1} g per system (upper triangular part of the rotated Hessenberg); also a float copy for FP32
+// vectors.  One warp per system, lane r the right-hand side of row r: each solved unknown is taken out
+// of all rows at once (one thread per system ran the whole triangle through memory, 19 to 39 us).
 __global__ void k_backsolve(int M, int R, const double *__restrict__ H, const double *__restrict__ g,
                             const int *__restrict__ kcol, double *__restrict__ y, float *__restrict__ y32) {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (m >= M) return;
-    int k = kcol[m];
+    const int k = kcol[m];   // at most 32 columns
     const double *Hm = H + (int64_t)m * (R + 1) * R;
-    for (int r = k - 1; r >= 0; --r) {
-        double s = g[m * (R + 1) + r];
-        for (int c = r + 1; c < k; ++c) s -= Hm[r * R + c] * y[c * M + m];
-        y[r * M + m] = Hm[r * R + r] != 0.0 ? s / Hm[r * R + r] : 0.0;
-        y32[r * M + m] = (float)y[r * M + m];
+    double s = lane < k ? g[m * (R + 1) + lane] : 0.0, mine = 0.0;
+    const double d = lane < k ? Hm[lane * R + lane] : 1.0, inv = d != 0.0 ? 1.0 / d : 0.0;
+    for (int c = k - 1; c >= 0; --c) {
+        const double h = lane < c ? Hm[lane * R + c] : 0.0;
+        const double yc = __shfl_sync(0xffffffffu, s * inv, c);
+        if (lane == c) mine = yc;
+        s -= h * yc;
+    }
+    if (lane < k) {
+        y[lane * M + m] = mine;
+        y32[lane * M + m] = (float)mine;
     }
 }
 
@@ -570,19 +577,21 @@ __global__ void k_axpy1(int64_t N, const T *__restrict__ u, T *__restrict__ x) {
     if (e < N) x[e] += u[e];
 }
 
-// out[i] = sum_m w[m] x[i][m]  (angular reduction D, Sec. 4.2)
+// out[i] = sum_m w[m] x[i][m]  (angular reduction D, Sec. 4.2), eight lanes per point: three FP64
+// additions of the lanes' parts per four points (a warp per point took five for each: 34 us at 256^2 S8,
+// all of it in the FP64 units)
 template <typename T>
 __global__ void k_Dreduce(int64_t n, int M, const double *__restrict__ w, const T *__restrict__ x,
                           double *__restrict__ out) {
     using A = typename Arith<T>::type;
-    int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (i >= n) return;
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    const int lane = threadIdx.x & 7;
     A sl = 0;
-    for (int m = lane; m < M; m += 32) sl += (A)w[m] * (A)x[i * M + m];
+    if (i < n)
+        for (int m = lane; m < M; m += 8) sl += (A)w[m] * (A)x[i * M + m];
     double s = (double)sl;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[i] = s;
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (i < n && lane == 0) out[i] = s;
 }
 
 template <typename Ti, typename To>
@@ -827,7 +836,7 @@ static mlpg_status gmres_solve(mlpg_ctx *ctx, Gmres<T> &G, const ApplyFn<T> &A, 
             z = precond(w, G.Zf ? G.Zf + (int64_t)(j + 1) * N : G.Z, G.beta);
             if (!z) return MLPG_ERR_CUDA;
         }
-        k_backsolve<<<(M + 127) / 128, 128, 0, s>>>(M, R, G.H, G.g, G.kcol, G.y, G.y32);
+        k_backsolve<<<wblk, kBlock, 0, s>>>(M, R, G.H, G.g, G.kcol, G.y, G.y32);
         CU_LAUNCH(ctx);
         if (on_cycle) MLPG_TRY(on_cycle(G.y, G.y32, G.kcol, jlast + 1));
         const T *u = G.W;
@@ -974,7 +983,7 @@ static mlpg_status nested_solve(mlpg_ctx *ctx, const double *f, double *Psi_out,
     CU_LAUNCH(ctx);
     // first flight b_psi = L^{-1} f, b_phi = D b_psi
     MLPG_TRY(inner_solve<T>(ctx, rhs, bpsi, inner_tol));
-    k_Dreduce<T><<<nblk(n * 32), kBlock, 0, s>>>(n, ctx->m, ctx->w, bpsi, bphi);
+    k_Dreduce<T><<<nblk(n * 8), kBlock, 0, s>>>(n, ctx->m, ctx->w, bpsi, bphi);
     CU_LAUNCH(ctx);
     MLPG_TRY(shard_sum_dev(ctx, bphi, n));
     // scattering GMRES: (I - D L^{-1} MS) Phi = b_phi
@@ -994,7 +1003,7 @@ static mlpg_status nested_solve(mlpg_ctx *ctx, const double *f, double *Psi_out,
         for (int k = 0;; ++k) {
             MLPG_TRY(apply_MS<T>(ctx, phi, rhs));
             MLPG_TRY(inner_solve<T>(ctx, rhs, x, inner_tol));
-            k_Dreduce<T><<<nblk(n * 32), kBlock, 0, s>>>(n, ctx->m, ctx->w, x, d);
+            k_Dreduce<T><<<nblk(n * 8), kBlock, 0, s>>>(n, ctx->m, ctx->w, x, d);
             CU_LAUNCH(ctx);
             MLPG_TRY(shard_sum_dev(ctx, d, n));
             k_si_update<<<nblk(n), kBlock, 0, s>>>(n, bphi, d, phi, e);
@@ -1028,7 +1037,7 @@ static mlpg_status nested_solve(mlpg_ctx *ctx, const double *f, double *Psi_out,
         T *xt = slot >= 0 ? bank + (int64_t)slot * N : (slot == -1 ? xacc : x);
         MLPG_TRY(apply_MS<T>(ctx, X, rhs));
         MLPG_TRY(inner_solve<T>(ctx, rhs, xt, ctx->cur_inner_tol));
-        k_Dreduce<T><<<nblk(n * 32), kBlock, 0, s>>>(n, ctx->m, ctx->w, xt, d);
+        k_Dreduce<T><<<nblk(n * 8), kBlock, 0, s>>>(n, ctx->m, ctx->w, xt, d);
         CU_LAUNCH(ctx);
         MLPG_TRY(shard_sum_dev(ctx, d, n));
         k_outer_combine<<<nblk(n), kBlock, 0, s>>>(n, X, d, B, Y);
@@ -1137,7 +1146,7 @@ mlpg_status step_fp64(mlpg_ctx *ctx, double dt) {
     MLPG_TRY(rhs_T(ctx, ctx->Psi, ctx->f64));
     MLPG_TRY(nested_solve<double>(ctx, ctx->f64, ctx->tmp64, ctx->Phi, ctx->opt.inner_tol, ctx->opt.outer_tol));
     CU(ctx, cudaMemcpyAsync(ctx->Psi, ctx->tmp64, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
-    k_Dreduce<double><<<nblk(n * 32), kBlock, 0, s>>>(n, ctx->m, ctx->w, ctx->Psi, ctx->Phi);
+    k_Dreduce<double><<<nblk(n * 8), kBlock, 0, s>>>(n, ctx->m, ctx->w, ctx->Psi, ctx->Phi);
     CU_LAUNCH(ctx);
     MLPG_TRY(shard_sum_dev(ctx, ctx->Phi, n));
     // report the FP64 step residual
@@ -1182,7 +1191,7 @@ mlpg_status step_mixed(mlpg_ctx *ctx, double dt) {
     int k = 0;
     double rel = 0.0;
     for (;; ++k) {
-        k_Dreduce<double><<<nblk(n * 32), kBlock, 0, s>>>(n, ctx->m, ctx->w, ctx->Psi, phi_c);
+        k_Dreduce<double><<<nblk(n * 8), kBlock, 0, s>>>(n, ctx->m, ctx->w, ctx->Psi, phi_c);
         CU_LAUNCH(ctx);
         MLPG_TRY(shard_sum_dev(ctx, phi_c, n));
         MLPG_TRY(apply_L64_res(ctx, ctx->Psi, ctx->f64, ctx->res64));
@@ -1204,7 +1213,7 @@ mlpg_status step_mixed(mlpg_ctx *ctx, double dt) {
         k_add<double, double><<<nblk(N), kBlock, 0, s>>>(N, ctx->Psi, ctx->tmp64, ctx->Psi);
         CU_LAUNCH(ctx);
     }
-    k_Dreduce<double><<<nblk(n * 32), kBlock, 0, s>>>(n, ctx->m, ctx->w, ctx->Psi, ctx->Phi);
+    k_Dreduce<double><<<nblk(n * 8), kBlock, 0, s>>>(n, ctx->m, ctx->w, ctx->Psi, ctx->Phi);
     CU_LAUNCH(ctx);
     MLPG_TRY(shard_sum_dev(ctx, ctx->Phi, n));
     ctx->st.last_refinements = k;

@@ -232,65 +232,40 @@ __global__ void k_scan1(int64_t n, const int *__restrict__ in, int32_t *__restri
 // batched L-apply.  A team of TM lanes (power of two) works on one row; lane l
 // owns directions m = l + TM t, t < DPL.  Y = L X, or Y = B - L X when B != 0.
 // ---------------------------------------------------------------------------
-// Warp-per-row layout of the FP64 apply: the 32 lanes of a warp are S
-// entry slots x TM direction lanes (S * TM = 32); lane (s, l) takes the row
-// entries p0 + s, p0 + s + S, ... and the directions l, l + TM, ... (DPL of
-// them).  The S partial sums of each direction are combined with shuffles.
-template <typename T, int DPL>
-__device__ __forceinline__ void slot_reduce(T (&acc)[DPL], int TM) {
-#pragma unroll
-    for (int t = 0; t < DPL; ++t)
-        for (int o = TM; o < 32; o <<= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
-}
-
-template <int DPL>
-__global__ void __launch_bounds__(256) k_spmm64(int64_t n, int m, int tm_log2,
-                                                const int32_t *__restrict__ rowptr,
-                                                const int32_t *__restrict__ col,
-                                                const double *__restrict__ L64,
+// FP64 apply: one thread per (row, direction), a row's threads reading one
+// contiguous run of L64 and of X per entry.  The bound is the FP64 units: 1.6
+// multiply-adds per clock and SM (measured), 36 us at 96^2 S8 against 21 us of
+// memory.  Lanes that split a row's entries and add their parts by shuffles spent
+// a seventh of that time on the additions (54.7 us); here every lane's operation is
+// a product of the sum.
+__global__ void __launch_bounds__(256) k_spmm64(int64_t total, int m, const int32_t *__restrict__ rowptr,
+                                                const int32_t *__restrict__ col, const double *__restrict__ L64,
                                                 const double *__restrict__ X, const double *__restrict__ B,
                                                 double *__restrict__ Y) {
-    const int TM = 1 << tm_log2, S = 32 >> tm_log2;
-    const int lane = threadIdx.x & (TM - 1), slot = (threadIdx.x & 31) >> tm_log2;
-    const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (row >= n) return;
-    double acc[DPL];
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int64_t row = e / m;
+    const int k = (int)(e - row * m);
+    const int32_t p0 = rowptr[row], p1 = rowptr[row + 1];
+    const double *L = L64 + (int64_t)p0 * m + k, *Xk = X + k;
+    double acc0 = 0.0, acc1 = 0.0;
+    int32_t p = p0;
+    for (; p + 8 <= p1; p += 8, L += 8 * (int64_t)m) {   // eight entries' loads in flight
+        double l[8], x[8];
 #pragma unroll
-    for (int t = 0; t < DPL; ++t) acc[t] = 0.0;
-    const int32_t p1 = rowptr[row + 1];
-    int32_t p = rowptr[row] + slot;
-    for (; p + S < p1; p += 2 * S) {  // two entries per lane in flight
-        const int64_t j0 = col[p], j1 = col[p + S];
+        for (int q = 0; q < 8; ++q) {
+            l[q] = __ldg(L + q * (int64_t)m);
+            x[q] = __ldg(Xk + (int64_t)__ldg(col + p + q) * m);
+        }
 #pragma unroll
-        for (int t = 0; t < DPL; ++t) {
-            int k = lane + t * TM;
-            if (k < m) {
-                double l0 = L64[(int64_t)p * m + k], l1 = L64[(int64_t)(p + S) * m + k];
-                double x0 = X[j0 * m + k], x1 = X[j1 * m + k];
-                acc[t] = fma(l0, x0, acc[t]);
-                acc[t] = fma(l1, x1, acc[t]);
-            }
+        for (int q = 0; q < 8; q += 2) {
+            acc0 = fma(l[q], x[q], acc0);
+            acc1 = fma(l[q + 1], x[q + 1], acc1);
         }
     }
-    if (p < p1) {
-        const int64_t j = col[p];
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) {
-            int k = lane + t * TM;
-            if (k < m) acc[t] = fma(L64[(int64_t)p * m + k], X[j * m + k], acc[t]);
-        }
-    }
-    slot_reduce<double, DPL>(acc, TM);
-    if (slot == 0) {
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) {
-            int k = lane + t * TM;
-            if (k < m) {
-                int64_t e = row * m + k;
-                Y[e] = B ? B[e] - acc[t] : acc[t];
-            }
-        }
-    }
+    for (; p < p1; ++p, L += m) acc0 = fma(__ldg(L), __ldg(Xk + (int64_t)__ldg(col + p) * m), acc0);
+    const double acc = acc0 + acc1;
+    Y[e] = B ? B[e] - acc : acc;
 }
 
 // FP32 batched L-apply: a team of TM lanes per row (4 rows per warp for
@@ -949,56 +924,61 @@ __global__ void __launch_bounds__(256) k_rhs64(int64_t n, int m, int tm_log2, in
     }
 }
 
-// abc[0] = Ms Phi, abc[1 + a] = tau Gs^a Phi (1 + D SpMVs on one vector)
+// abc[0] = Ms Phi, abc[1 + a] = tau Gs^a Phi (1 + D SpMVs on one vector), eight lanes
+// per row: a row's entries are read in runs (one thread per row read 76 MB at 256^2 in
+// 43 us, each lane its own lines).  abc32 (or null): float copies divided by 4 pi.
 template <int D>
 __global__ void k_ms_spmv(int64_t n, int64_t nnz, const int32_t *__restrict__ rowptr,
                           const int32_t *__restrict__ col, const double *__restrict__ S64,
-                          const double *__restrict__ phi, double *__restrict__ abc) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+                          const double *__restrict__ phi, double *__restrict__ abc, float *__restrict__ abc32) {
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
+    const int lane = threadIdx.x & 7;
     double acc[NT<D>()];
 #pragma unroll
     for (int a = 0; a < NT<D>(); ++a) acc[a] = 0.0;
-    for (int32_t p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-        double v = phi[col[p]];
+    if (i < n)
+        for (int32_t p = rowptr[i] + lane; p < rowptr[i + 1]; p += 8) {
+            const double v = phi[col[p]];
 #pragma unroll
-        for (int a = 0; a < NT<D>(); ++a) acc[a] = fma(S64[a * nnz + p], v, acc[a]);
-    }
+            for (int a = 0; a < NT<D>(); ++a) acc[a] = fma(S64[a * nnz + p], v, acc[a]);
+        }
 #pragma unroll
-    for (int a = 0; a < NT<D>(); ++a) abc[a * n + i] = acc[a];
+    for (int a = 0; a < NT<D>(); ++a)
+        for (int o = 4; o > 0; o >>= 1) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], o);
+    if (i < n && lane == 0)
+#pragma unroll
+        for (int a = 0; a < NT<D>(); ++a) {
+            abc[a * n + i] = acc[a];
+            if (abc32) abc32[a * n + i] = (float)(acc[a] * (1.0 / kFourPi));
+        }
 }
 
+// thread per (point, direction)
 template <typename T, int D>
-__global__ void k_ms_expand(int64_t n, int m, const double *__restrict__ abc,
+__global__ void k_ms_expand(int64_t total, int m, int64_t n, const double *__restrict__ abc,
                             const double *__restrict__ coef, T *__restrict__ out) {
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n * m) return;
+    if (e >= total) return;
     int64_t i = e / m;
     int k = (int)(e - i * m);
     double v = abc[i];
 #pragma unroll
     for (int a = 0; a < D; ++a) v = v + coef[kCS * k + 1 + a] * abc[(1 + a) * n + i];
-    out[e] = (T)(v / kFourPi);
+    out[e] = (T)(v * (1.0 / kFourPi));
 }
 
 // FP32 variant: the per-point products arrive pre-scaled by 1/(4 pi) in float
 template <int D>
-__global__ void k_ms_expand32(int64_t n, int m, const float *__restrict__ abc32,
+__global__ void k_ms_expand32(int64_t total, int m, int64_t n, const float *__restrict__ abc32,
                               const float *__restrict__ coef32, float *__restrict__ out) {
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n * m) return;
+    if (e >= total) return;
     int64_t i = e / m;
     int k = (int)(e - i * m);
     float v = abc32[i];
 #pragma unroll
     for (int a = 0; a < D; ++a) v = fmaf(coef32[16 * k + 1 + a], abc32[(1 + a) * n + i], v);
     out[e] = v;
-}
-
-__global__ void k_abc32(int64_t cnt, const double *__restrict__ abc, float *__restrict__ abc32) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= cnt) return;
-    abc32[i] = (float)(abc[i] / kFourPi);
 }
 
 __global__ void k_interp_apply(int64_t n, const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
@@ -1115,6 +1095,21 @@ __global__ void __launch_bounds__(256) k_block_inv(int64_t nblk, int m, const in
 // Requires m % 4 == 0 (the caller falls back to k_bjacobi_scalar otherwise).
 // With sc != null the input rows are first scaled by sc[direction] and the
 // scaled rows written back to v (the GMRES basis normalisation, fused here).
+// An FP32 value (its bits) in the vector's type, divided by widen_factor.  For FP64 the bits move to their
+// places in a double whose exponent lacks the difference of the biases, 2^-896 (exact, zeros and
+// subnormals included): integer moves, because the conversion runs on the FP64 units, at 1.9
+// per clock and SM, and would cost as much as the multiply-add (96^2 S8: 28.9 us with it).
+template <typename T>
+__device__ __forceinline__ T widen(uint32_t b) {
+    if constexpr (sizeof(T) == 4) return __uint_as_float(b);
+    else return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3)), (int)(b << 29));
+}
+template <typename T>
+__device__ __forceinline__ T widen_factor() {
+    if constexpr (sizeof(T) == 4) return 1.0f;
+    else return __hiloint2double((1023 + 896) << 20, 0);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const int32_t *__restrict__ bmember,
                                                      const float *__restrict__ Pinv, T *__restrict__ v,
@@ -1142,7 +1137,7 @@ __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const 
         vs[q] = val;
     }
     __syncthreads();
-    const float4 *P4 = reinterpret_cast<const float4 *>(Pinv + blk * (int64_t)kB * kB * m);
+    const uint4 *P4 = reinterpret_cast<const uint4 *>(Pinv + blk * (int64_t)kB * kB * m);
     for (int t = threadIdx.x; t < kB * mc; t += blockDim.x) {
         const int a = t / mc, c = t - a * mc;
         const int32_t i = mem[a];
@@ -1150,15 +1145,16 @@ __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const 
         T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
 #pragma unroll 4
         for (int b = 0; b < kB; ++b) {
-            const float4 p = P4[((int64_t)a * kB + b) * mc + c];
+            const uint4 p = P4[((int64_t)a * kB + b) * mc + c];
             const T *vb = vs + b * m + 4 * c;
-            acc0 += (T)p.x * vb[0];
-            acc1 += (T)p.y * vb[1];
-            acc2 += (T)p.z * vb[2];
-            acc3 += (T)p.w * vb[3];
+            acc0 += widen<T>(p.x) * vb[0];
+            acc1 += widen<T>(p.y) * vb[1];
+            acc2 += widen<T>(p.z) * vb[2];
+            acc3 += widen<T>(p.w) * vb[3];
         }
         T *zo = z + (int64_t)i * m + 4 * c;
-        zo[0] = acc0; zo[1] = acc1; zo[2] = acc2; zo[3] = acc3;
+        const T f = widen_factor<T>();
+        zo[0] = acc0 * f; zo[1] = acc1 * f; zo[2] = acc2 * f; zo[3] = acc3 * f;
     }
 }
 
@@ -1614,17 +1610,6 @@ Team pick_team(int m) {
 }
 
 }  // namespace
-
-#define DISPATCH_DPL(dpl, KERNEL, ...)                                   \
-    switch (dpl) {                                                       \
-        case 1: KERNEL<1><<<grid, 256, 0, s>>>(__VA_ARGS__); break;      \
-        case 2: KERNEL<2><<<grid, 256, 0, s>>>(__VA_ARGS__); break;      \
-        case 3: KERNEL<3><<<grid, 256, 0, s>>>(__VA_ARGS__); break;      \
-        case 4: KERNEL<4><<<grid, 256, 0, s>>>(__VA_ARGS__); break;      \
-        case 5: case 6: KERNEL<6><<<grid, 256, 0, s>>>(__VA_ARGS__); break; \
-        case 7: case 8: KERNEL<8><<<grid, 256, 0, s>>>(__VA_ARGS__); break; \
-        default: KERNEL<16><<<grid, 256, 0, s>>>(__VA_ARGS__); break;    \
-    }
 
 // one warp per row (slot layout) / one team of TM lanes per row
 static int64_t team_grid(int64_t n, const Team &) { return (n * 32 + 255) / 256; }
@@ -2097,11 +2082,10 @@ static void timing_end(mlpg_ctx *ctx) {
 }
 
 mlpg_status apply_L64_res(mlpg_ctx *ctx, const double *X, const double *B, double *Y) {
-    Team tm = pick_team(ctx->m);
-    int64_t grid = team_grid(ctx->n, tm);
-    cudaStream_t s = ctx->stream;
+    const int64_t total = ctx->n * ctx->m;
     timing_begin(ctx);
-    DISPATCH_DPL(tm.dpl, k_spmm64, ctx->n, ctx->m, tm.tm_log2, ctx->rowptr, ctx->col, ctx->L64, X, B, Y);
+    k_spmm64<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col, ctx->L64, X, B,
+                                                                      Y);
     timing_end(ctx);
     CU_LAUNCH(ctx);
     return MLPG_OK;
@@ -2113,7 +2097,6 @@ static mlpg_status apply_faces32(mlpg_ctx *ctx, const Team &tm, const float *X, 
 template <int DIM>
 static mlpg_status apply_L32_res_d(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
     Team tm = pick_team(ctx->m);
-    int64_t grid = team_grid(ctx->n, tm);
     cudaStream_t s = ctx->stream;
     timing_begin(ctx);
     if (ctx->t_rec) {   // the face terms are added inside the tile kernel
@@ -2213,17 +2196,15 @@ template <typename T, int D>
 static mlpg_status apply_MS_d(mlpg_ctx *ctx, const double *phi, T *out) {
     const int64_t n = ctx->n;
     cudaStream_t s = ctx->stream;
-    k_ms_spmv<D><<<(n + 255) / 256, 256, 0, s>>>(n, ctx->nnz, ctx->rowptr, ctx->col, ctx->S64, phi, ctx->abc);
+    float *abc32 = sizeof(T) == 4 ? (float *)(ctx->abc + NT<D>() * n) : nullptr;
+    k_ms_spmv<D><<<(unsigned)((n * 8 + 255) / 256), 256, 0, s>>>(n, ctx->nnz, ctx->rowptr, ctx->col, ctx->S64, phi, ctx->abc,
+                                                                abc32);
     CU_LAUNCH(ctx);
     int64_t nm = n * ctx->m;
-    if constexpr (sizeof(T) == 4) {
-        float *abc32 = (float *)(ctx->abc + NT<D>() * n);
-        k_abc32<<<(NT<D>() * n + 255) / 256, 256, 0, s>>>(NT<D>() * n, ctx->abc, abc32);
-        CU_LAUNCH(ctx);
-        k_ms_expand32<D><<<(nm + 255) / 256, 256, 0, s>>>(n, ctx->m, abc32, ctx->coef32, (float *)out);
-    } else {
-        k_ms_expand<T, D><<<(nm + 255) / 256, 256, 0, s>>>(n, ctx->m, ctx->abc, ctx->coef, out);
-    }
+    if constexpr (sizeof(T) == 4)
+        k_ms_expand32<D><<<(nm + 255) / 256, 256, 0, s>>>(nm, ctx->m, n, abc32, ctx->coef32, (float *)out);
+    else
+        k_ms_expand<T, D><<<(nm + 255) / 256, 256, 0, s>>>(nm, ctx->m, n, ctx->abc, ctx->coef, out);
     CU_LAUNCH(ctx);
     return MLPG_OK;
 }
