@@ -397,6 +397,16 @@ mlpg_status mlpg_step_batch(mlpg_ctx *const *ctxs, const double *dt, int count, 
     if (count == 0) return MLPG_OK;
     std::vector<mlpg_status> st(count, MLPG_OK);
     std::vector<std::thread> th;
+    struct Peers {   // how many problems share the device, for the kernels' choice; 1 again on every return
+        mlpg_ctx *const *c;
+        int k;
+        Peers(mlpg_ctx *const *ctxs_, int count_) : c(ctxs_), k(count_) { set(count_); }
+        ~Peers() { set(1); }
+        void set(int v) {
+            for (int i = 0; i < k; ++i) c[i]->peers = v;
+        }
+    };
+    const Peers peers(ctxs, count);
     int next = 1;   // contexts [next, count) still to run on the caller's thread
     try {
         th.reserve(count - 1);

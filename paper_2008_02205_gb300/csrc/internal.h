@@ -119,6 +119,8 @@ struct Gmres {
     int *d_active_count = nullptr;
     bool reorth = true;        // CGS2 (true) or a single classical Gram-Schmidt pass
     int its_slot = 0;          // iteration counter of the step this solve adds to (0 inner, 1 outer, 2 diffusion)
+    int gs_cluster = 0;        // CTAs per cluster of the one-launch Arnoldi step (0: separate passes)
+    int gs_kind = -1;          // the value of reorth it was set up for
     T *Zf = nullptr;           // R * n * M: preconditioned basis vectors (flexible GMRES), or null
 };
 
@@ -242,6 +244,8 @@ struct mlpg_ctx {
     mlpg_reduce_fn reduce_fn = nullptr;
     void *reduce_user = nullptr;
     double *reduce_host = nullptr;   // n + 8 doubles
+
+    int peers = 1;                   // contexts that the current mlpg_step_batch runs at once
 
     // stats
     mlpg_stats st{};

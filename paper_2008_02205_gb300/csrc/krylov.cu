@@ -22,6 +22,8 @@
 #include <functional>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "internal.h"
 
 namespace mlpg {
@@ -416,32 +418,22 @@ __global__ void k_start(int M, int R, const double *__restrict__ nrm2, double *_
     if (act) atomicAdd(count, 1);
 }
 
-// Column j of the Hessenberg matrix, Givens rotations, residual estimate.
-// One warp per system: the warp first sums the G norm partials of ||w||^2.
-__global__ void k_givens(int M, int R, int j, int G, const double *__restrict__ partial,
-                         const double *__restrict__ h1, const double *__restrict__ h2, double *__restrict__ H,
-                         double *__restrict__ cs, double *__restrict__ sn, double *__restrict__ g,
-                         double *__restrict__ sc, int *__restrict__ active, int *__restrict__ kcol,
-                         int *__restrict__ its, double *__restrict__ resid, const double *__restrict__ bnorm,
-                         double tol, int *__restrict__ count) {
-    const int m = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (m >= M) return;
-    if (!active[m]) {
-        if (lane == 0) sc[m] = 0.0;
-        return;
-    }
-    const double nrm2 = warp_sum_partials(partial + (int64_t)m * G, G, lane);
+// Column j of the Hessenberg matrix, Givens rotations and residual estimate of system m, by one warp.
+// lane l holds entry l of the new column (hl, l <= j < R <= 32); nrm2 = ||w||^2.  Every lane runs the
+// same rotation chain down the column in registers and keeps its own entry.
+__device__ __forceinline__ void givens_column(int m, int lane, int R, int j, double nrm2, double hl,
+                                              double *__restrict__ H, double *__restrict__ cs, double *__restrict__ sn,
+                                              double *__restrict__ g, double *__restrict__ sc, int *__restrict__ active,
+                                              int *__restrict__ kcol, int *__restrict__ its, double *__restrict__ resid,
+                                              const double *__restrict__ bnorm, double tol, int *__restrict__ count) {
     const double hn = sqrt(nrm2);
     double *Hm = H + (int64_t)m * (R + 1) * R;  // Hm[row * R + col]
-    // lane l holds entry l of the new column (l <= j < R <= 32) and the earlier rotation l (l < j);
-    // every lane runs the same rotation chain down the column in registers and keeps its own entry
-    double hl = 0.0, cl = 1.0, sl = 0.0;
-    if (lane <= j) hl = h1[lane * M + m] + (h2 ? h2[lane * M + m] : 0.0);
+    double cl = 1.0, sl = 0.0;
     if (lane < j) {
         cl = cs[m * R + lane];
         sl = sn[m * R + lane];
     }
+    const double gj = g[m * (R + 1) + j], bn = bnorm[m];
     double carry = __shfl_sync(0xffffffffu, hl, 0), mine = 0.0;
     for (int l = 0; l < j; ++l) {
         const double c = __shfl_sync(0xffffffffu, cl, l), sv = __shfl_sync(0xffffffffu, sl, l);
@@ -461,14 +453,13 @@ __global__ void k_givens(int M, int R, int j, int G, const double *__restrict__ 
     sn[m * R + j] = sv;
     Hm[j * R + j] = den;
     Hm[(j + 1) * R + j] = 0.0;
-    double gj = g[m * (R + 1) + j];
     g[m * (R + 1) + j] = c * gj;
     g[m * (R + 1) + j + 1] = -sv * gj;
     its[m] += 1;
     kcol[m] = j + 1;
     double res = fabs(sv * gj);
     resid[m] = res;
-    bool done = res <= tol * bnorm[m] || !(hn > 0.0) || j + 1 == R;
+    bool done = res <= tol * bn || !(hn > 0.0) || j + 1 == R;
     if (done) {
         active[m] = 0;
         sc[m] = 0.0;
@@ -476,6 +467,248 @@ __global__ void k_givens(int M, int R, int j, int G, const double *__restrict__ 
         sc[m] = 1.0 / hn;
         atomicAdd(count, 1);
     }
+}
+
+// One warp per system: the warp first sums the G norm partials of ||w||^2.
+__global__ void k_givens(int M, int R, int j, int G, const double *__restrict__ partial,
+                         const double *__restrict__ h1, const double *__restrict__ h2, double *__restrict__ H,
+                         double *__restrict__ cs, double *__restrict__ sn, double *__restrict__ g,
+                         double *__restrict__ sc, int *__restrict__ active, int *__restrict__ kcol,
+                         int *__restrict__ its, double *__restrict__ resid, const double *__restrict__ bnorm,
+                         double tol, int *__restrict__ count) {
+    const int m = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (m >= M) return;
+    if (!active[m]) {
+        if (lane == 0) sc[m] = 0.0;
+        return;
+    }
+    const double nrm2 = warp_sum_partials(partial + (int64_t)m * G, G, lane);
+    const double hl = lane <= j ? h1[lane * M + m] + (h2 ? h2[lane * M + m] : 0.0) : 0.0;
+    givens_column(m, lane, R, j, nrm2, hl, H, cs, sn, g, sc, active, kcol, its, resid, bnorm, tol, count);
+}
+
+// ---------------------------------------------------------------------------
+// The whole Arnoldi step after the operator in one launch: classical Gram-Schmidt
+// (once, or twice with REORTH) of w against V_0 .. V_{nl-1}, its norm, and the Givens
+// update.  The systems are independent, so a cluster of CTAs takes DV of them (32 bytes of
+// each row: one sector): every CTA keeps its rows of w in shared memory for the whole
+// step, streams its rows of the basis, and the cluster adds the CTAs' sums through
+// distributed shared memory, in rank order.
+//
+// Why: as separate passes (dots, reduction, update, norm, Givens; six launches with
+// REORTH) a small problem's step is launch and reduction latency: 38 us at 32^2 S4,
+// 26 us here.  A large one is better off with the separate passes, which use every SM
+// and move 32-byte sectors of whole rows.  The line: points (times the problems that
+// mlpg_step_batch runs at once, which fill the chip themselves) up to kGsRows32 in FP32,
+// kGsRows64 in FP64, whose sums keep the few FP64 units of a cluster's SMs busy.  Whole
+// steps, separate -> one launch (ms): FP32 32^2 S4 11.4 -> 7.9, 75^2 S6 22.9 -> 18.4,
+// 128^2 S8 25.7 -> 21.8, 180^2 S8 37.7 -> 38.5; 3D 20^3 S8 92.5 -> 86.9; FP64 32^2 S4
+// 28.8 -> 21.2, 64^2 S8 172 -> 167, 96^2 S8 324 -> 362.  Eight problems of 1k to 16k points
+// at once: 57.0 with separate passes, 60.8 in one launch.
+// ---------------------------------------------------------------------------
+constexpr int64_t kGsRows32 = 16384, kGsRows64 = 4096;
+constexpr int kGsGroup = 8;   // basis vectors per accumulator group
+constexpr int kGsMaxCluster = 16;
+constexpr size_t kGsSmem = 200 * 1024;
+template <typename T, int DV>
+struct GsShape {
+    // FP64: every thread's partial sums cost FP64 additions, so few threads; FP32: more loads in flight
+    static constexpr int threads = sizeof(T) == 8 ? 128 : 256;
+    static constexpr int VEC = 16 / (int)sizeof(T);   // values per 16-byte load
+    static constexpr int TPR = DV / VEC;              // threads per row
+    static constexpr int NV = kGsGroup * VEC;         // sums of a thread
+    // bytes besides w: the warps' sums, the CTA's sums and the cluster's (twice MAX_RESTART and the norm),
+    // coefficients of an update
+    static constexpr size_t fixed = (size_t)(threads / 32) * TPR * NV * 8 +
+                                    (size_t)(2 * MLPG_MAX_RESTART + 1) * DV * 8 * 2 + (size_t)MLPG_MAX_RESTART * DV * 8;
+};
+
+// Sums of v[NV] over the lanes of a warp that differ in the bits from TPR up, halving the values at each
+// step (a lane keeps one half and passes the other on): NV - NV / n additions instead of NV log2 n.
+// Afterwards v[0 .. NV TPR / 32) hold the sums of the values from the returned index on.
+template <int HALF, int O, int NV, typename A>
+__device__ __forceinline__ int lanes_sum_from(A (&v)[NV], int lane) {
+    if constexpr (O < 32) {
+        const bool up = lane & O;
+#pragma unroll
+        for (int i = 0; i < HALF; ++i) {
+            const A lo = v[i], hi = v[i + HALF];
+            v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
+        }
+        return (up ? HALF : 0) + lanes_sum_from<HALF / 2, O * 2, NV, A>(v, lane);
+    } else {
+        return 0;
+    }
+}
+template <int NV, int TPR, typename A>
+__device__ __forceinline__ int lanes_sum(A (&v)[NV], int lane) {
+    return lanes_sum_from<NV / 2, TPR, NV, A>(v, lane);
+}
+
+template <typename T, int DV, bool REORTH>
+__global__ void __launch_bounds__(GsShape<T, DV>::threads) k_gs_step(int64_t n, int M, int rpc, int nl, const T *__restrict__ V,
+                                                        int64_t vs, T *__restrict__ w, int R, double *__restrict__ H,
+                                                        double *__restrict__ cs, double *__restrict__ sn,
+                                                        double *__restrict__ g, double *__restrict__ sc,
+                                                        int *__restrict__ active, int *__restrict__ kcol,
+                                                        int *__restrict__ its, double *__restrict__ resid,
+                                                        const double *__restrict__ bnorm, double tol,
+                                                        int *__restrict__ count, int *__restrict__ count_next) {
+    namespace cg = cooperative_groups;
+    using A = typename Arith<T>::type;
+    using V16 = typename Vec16<T>::type;
+    using Sh = GsShape<T, DV>;
+    constexpr int NT = Sh::threads, VEC = Sh::VEC, TPR = Sh::TPR, NV = Sh::NV, RPI = NT / TPR;   // RPI: rows per sweep
+    constexpr int NL = MLPG_MAX_RESTART, NWARP = NT / 32;
+    static_assert(NV * TPR % 32 == 0, "whole sums per lane");
+    extern __shared__ __align__(16) unsigned char gs_smem[];
+    double *red = reinterpret_cast<double *>(gs_smem);                             // [warp][TPR][NV]
+    double *part = red + NWARP * TPR * NV;                                         // [2 NL + 1][DV]
+    double *tot = part + (2 * NL + 1) * DV;                                        // [2 NL + 1][DV]: the cluster's sums
+    A *hc = reinterpret_cast<A *>(tot + (2 * NL + 1) * DV);                        // [NL][DV]: coefficients of an update
+    T *ws = reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(hc) + (size_t)NL * DV * 8);   // [rpc][DV]
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), C = (int)cluster.num_blocks();
+    const int tid = threadIdx.x, d0 = blockIdx.y * DV, q = tid % TPR, r0 = tid / TPR;
+    const int64_t i0 = (int64_t)rank * rpc;
+    const int rows = (int)max((int64_t)0, min((int64_t)rpc, n - i0));
+    const T *Vb = V + i0 * M + d0 + q * VEC;
+    T *wb = w + i0 * M + d0 + q * VEC;
+    if (tid == 0 && rank == 0 && blockIdx.y == 0) *count_next = 0;   // the next step's counter
+    for (int r = r0; r < rows; r += RPI)
+        *reinterpret_cast<V16 *>(ws + (r * TPR + q) * VEC) = *reinterpret_cast<const V16 *>(wb + (int64_t)r * M);
+    // (each thread only touches its own rows of ws: no barrier)
+    const int lane = tid & 31, warp = tid >> 5;
+    auto block_sum = [&](A (&v)[NV], int na, double *out) {   // out[a][d] = sums over the CTA's threads
+        const int first = lanes_sum<NV, TPR, A>(v, lane);
+#pragma unroll
+        for (int i = 0; i < NV * TPR / 32; ++i) red[(warp * TPR + q) * NV + first + i] = (double)v[i];
+        __syncthreads();
+        for (int o = tid; o < na * DV; o += NT) {
+            const int a = o / DV, d = o - a * DV, qq = d / VEC, c = d - qq * VEC;
+            double s = 0.0;
+#pragma unroll
+            for (int w2 = 0; w2 < NWARP; ++w2) s += red[(w2 * TPR + qq) * NV + a * VEC + c];
+            out[o] = s;
+        }
+        __syncthreads();
+    };
+    auto dots = [&](double *out) {   // out[l][d] = this CTA's part of V_l . w
+        for (int l0 = 0; l0 < nl; l0 += kGsGroup) {
+            const int ng = min(kGsGroup, nl - l0);
+            A acc[NV];
+#pragma unroll
+            for (int a = 0; a < NV; ++a) acc[a] = 0;
+            // FP32: sums of four rows, then their sum; FP64 keeps one sum (an addition costs as much as a product)
+            constexpr int CH = sizeof(T) == 4 ? 4 : 1 << 30;
+            for (int rb = r0; rb < rows;) {
+                A pt[sizeof(T) == 4 ? NV : 1];
+                if constexpr (sizeof(T) == 4)
+#pragma unroll
+                    for (int a = 0; a < NV; ++a) pt[a] = 0;
+                for (int c4 = 0; c4 < CH && rb < rows; ++c4, rb += RPI) {
+                    T wv[VEC];
+                    unpack(*reinterpret_cast<const V16 *>(ws + (rb * TPR + q) * VEC), wv);
+                    const T *vr = Vb + (int64_t)rb * M + l0 * vs;
+                    V16 v[kGsGroup];
+#pragma unroll
+                    for (int a = 0; a < kGsGroup; ++a)
+                        if (a < ng) v[a] = __ldg(reinterpret_cast<const V16 *>(vr + a * vs));
+#pragma unroll
+                    for (int a = 0; a < kGsGroup; ++a)
+                        if (a < ng) {
+                            T x[VEC];
+                            unpack(v[a], x);
+#pragma unroll
+                            for (int c = 0; c < VEC; ++c) {
+                                if constexpr (sizeof(T) == 4) pt[a * VEC + c] += (A)x[c] * (A)wv[c];
+                                else acc[a * VEC + c] += (A)x[c] * (A)wv[c];
+                            }
+                        }
+                }
+                if constexpr (sizeof(T) == 4)
+#pragma unroll
+                    for (int a = 0; a < NV; ++a) acc[a] += pt[a];
+            }
+            block_sum(acc, ng, out + l0 * DV);
+        }
+    };
+    auto cluster_sum = [&](int first, int cnt) {   // tot[first ..] = sums of part[first ..] over the cluster
+        cluster.sync();
+        for (int o = tid; o < cnt; o += NT) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int c = 0; c < C; ++c) s += cluster.map_shared_rank(part, c)[first + o];
+            tot[first + o] = s;
+        }
+        __syncthreads();
+    };
+    auto update = [&](const double *h, bool last, A (&nrm)[NV]) {   // w -= sum_l h_l V_l; last: ||w||^2, to global
+        for (int o = tid; o < nl * DV; o += NT) hc[o] = (A)h[o];
+        __syncthreads();
+        for (int r = r0; r < rows; r += RPI) {
+            T wt[VEC];
+            V16 *wp = reinterpret_cast<V16 *>(ws + (r * TPR + q) * VEC);
+            unpack(*wp, wt);
+            A wv[VEC];
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) wv[c] = (A)wt[c];
+            const T *vr = Vb + (int64_t)r * M;
+            for (int l0 = 0; l0 < nl; l0 += kGsGroup) {
+                V16 v[kGsGroup];
+#pragma unroll
+                for (int a = 0; a < kGsGroup; ++a)
+                    if (l0 + a < nl) v[a] = __ldg(reinterpret_cast<const V16 *>(vr + (l0 + a) * vs));
+#pragma unroll
+                for (int a = 0; a < kGsGroup; ++a)
+                    if (l0 + a < nl) {
+                        T x[VEC];
+                        unpack(v[a], x);
+                        const A *hl = hc + (l0 + a) * DV + q * VEC;
+#pragma unroll
+                        for (int c = 0; c < VEC; ++c) wv[c] -= hl[c] * (A)x[c];
+                    }
+            }
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) {
+                wt[c] = (T)wv[c];
+                if (last) nrm[c] += (A)wt[c] * (A)wt[c];
+            }
+            const V16 o = pack<T>(wt);
+            *wp = o;
+            if (last) *reinterpret_cast<V16 *>(wb + (int64_t)r * M) = o;
+        }
+        __syncthreads();
+    };
+    A nrm[NV];   // [0 .. VEC): the norm
+#pragma unroll
+    for (int c = 0; c < NV; ++c) nrm[c] = 0;
+    dots(part);
+    cluster_sum(0, nl * DV);
+    update(tot, !REORTH, nrm);
+    if constexpr (REORTH) {
+        dots(part + NL * DV);
+        cluster_sum(NL * DV, nl * DV);
+        update(tot + NL * DV, true, nrm);
+    }
+    block_sum(nrm, 1, part + 2 * NL * DV);
+    cluster.sync();
+    if (rank == 0) {   // Givens: a warp per system
+        for (int d = warp; d < DV; d += NWARP) {
+            const int m = d0 + d;
+            if (!active[m]) {
+                if (lane == 0) sc[m] = 0.0;
+                continue;
+            }
+            double nrm2 = 0.0;
+            for (int c = 0; c < C; ++c) nrm2 += cluster.map_shared_rank(part, c)[2 * NL * DV + d];
+            double hl = 0.0;
+            if (lane < nl) hl = tot[lane * DV + d] + (REORTH ? tot[(NL + lane) * DV + d] : 0.0);
+            givens_column(m, lane, R, nl - 1, nrm2, hl, H, cs, sn, g, sc, active, kcol, its, resid, bnorm, tol, count);
+        }
+    }
+    cluster.sync();   // no CTA leaves while rank 0 may still read its sums
 }
 
 // w = w * sc[m]  (in the vector's own precision)
@@ -684,13 +917,71 @@ static mlpg_status gmres_alloc(mlpg_ctx *ctx, Gmres<T> &G, int64_t n, int M, int
     // the fused Gram-Schmidt passes write G * nl * M partials with G <= row_blocks(), nl <= R + 1
     G.partial_cap = (int64_t)row_blocks() * (R + 1) * M;
     MLPG_TRY(dalloc(ctx, &G.partial, G.partial_cap));
-    MLPG_TRY(dalloc(ctx, &G.d_active_count, 1));
+    MLPG_TRY(dalloc(ctx, &G.d_active_count, 2));
     if (flexible) MLPG_TRY(dalloc(ctx, &G.Zf, (size_t)R * n * M));
     CU(ctx, cudaFuncSetAttribute(k_cgsv_upd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdSmem));
     void *hp = nullptr;
     CU(ctx, cudaHostAlloc(&hp, sizeof(int) * 4, cudaHostAllocDefault));
     ctx->host_allocs.push_back(hp);
     G.h_active = (int *)hp;
+    G.gs_kind = -1;   // the one-launch Arnoldi step is set up at the first solve
+    return MLPG_OK;
+}
+
+// Cluster size of the one-launch Arnoldi step for M systems of n values, 0 when it does not fit: M a
+// multiple of the cluster's systems (32 bytes of a row; FP32 also 16, for sets that are no multiple of
+// eight), a CTA's rows of w in shared memory.
+template <typename T>
+static int gs_systems(int M) {
+    if (sizeof(T) == 8) return M % 4 == 0 ? 4 : 0;
+    return M % 8 == 0 ? 8 : (M % 4 == 0 ? 4 : 0);
+}
+template <typename T, int DV, bool REORTH>
+static mlpg_status launch_gs(mlpg_ctx *ctx, Gmres<T> &G, int j, double tol, int *count, int *count_next) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    const int rpc = (int)((G.n + G.gs_cluster - 1) / G.gs_cluster);
+    cfg.gridDim = dim3((unsigned)G.gs_cluster, (unsigned)(G.M / DV));
+    cfg.blockDim = dim3(GsShape<T, DV>::threads);
+    cfg.dynamicSmemBytes = GsShape<T, DV>::fixed + (size_t)rpc * DV * sizeof(T);
+    cfg.stream = ctx->stream;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)G.gs_cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    CU(ctx, cudaLaunchKernelEx(&cfg, k_gs_step<T, DV, REORTH>, G.n, G.M, rpc, j + 1, (const T *)G.V, G.n * (int64_t)G.M,
+                               G.V + (int64_t)(j + 1) * G.n * G.M, G.R, G.H, G.cs, G.sn, G.g, G.beta, G.active, G.kcol,
+                               G.its, G.resid, (const double *)G.bnorm, tol, count, count_next));
+    CU_LAUNCH(ctx);
+    return MLPG_OK;
+}
+template <typename T, int DV, bool REORTH>
+static mlpg_status init_gs(mlpg_ctx *ctx, Gmres<T> &G) {
+    G.gs_cluster = 0;
+    const void *f = (const void *)k_gs_step<T, DV, REORTH>;
+    CU(ctx, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsSmem));
+    CU(ctx, cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    for (int C = kGsMaxCluster; C >= 8; C /= 2) {
+        const size_t smem = GsShape<T, DV>::fixed + (size_t)((G.n + C - 1) / C) * DV * sizeof(T);
+        if (smem > kGsSmem) return MLPG_OK;   // smaller clusters need more
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        cfg.gridDim = dim3((unsigned)C, (unsigned)(G.M / DV));
+        cfg.blockDim = dim3(GsShape<T, DV>::threads);
+        cfg.dynamicSmemBytes = smem;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int nc = 0;
+        if (cudaOccupancyMaxActiveClusters(&nc, f, &cfg) == cudaSuccess && nc > 0) {
+            G.gs_cluster = C;
+            return MLPG_OK;
+        }
+        cudaGetLastError();   // no room for a cluster of this size
+    }
     return MLPG_OK;
 }
 
@@ -721,6 +1012,19 @@ static mlpg_status gmres_solve(mlpg_ctx *ctx, Gmres<T> &G, const ApplyFn<T> &A, 
     const bool vec_ok = M % VEC == 0 && M / VEC <= kBlock;
     const int64_t vrows = vec_ok ? (n + kBlock / (M / VEC) - 1) / (kBlock / (M / VEC)) : 1;   // row iterations
     CU(ctx, cudaMemsetAsync(G.its, 0, sizeof(int) * M, s));
+    if (G.gs_kind != (int)G.reorth) {
+        const int dv = gs_systems<T>(M);
+        G.gs_cluster = 0;
+        if constexpr (sizeof(T) == 8) {
+            if (dv) MLPG_TRY((G.reorth ? init_gs<T, 4, true>(ctx, G) : init_gs<T, 4, false>(ctx, G)));
+        } else if (dv == 8) {
+            MLPG_TRY((G.reorth ? init_gs<T, 8, true>(ctx, G) : init_gs<T, 8, false>(ctx, G)));
+        } else if (dv == 4) {
+            MLPG_TRY((G.reorth ? init_gs<T, 4, true>(ctx, G) : init_gs<T, 4, false>(ctx, G)));
+        }
+        G.gs_kind = (int)G.reorth;
+    }
+    const bool one_launch = G.gs_cluster && n * ctx->peers <= (sizeof(T) == 8 ? kGsRows64 : kGsRows32);
     auto norm2 = [&](const T *v) -> mlpg_status {   // G.nrm2[m] = ||v_m||^2
         int g1 = grid_rows(n, mp, 1);
         k_dots<T><<<dim3(g1, mp.mchunks, 1), kBlock, 0, s>>>(n, M, mp.MB, mp.RB, v, 0, v, G.partial);
@@ -756,7 +1060,7 @@ static mlpg_status gmres_solve(mlpg_ctx *ctx, Gmres<T> &G, const ApplyFn<T> &A, 
             MLPG_TRY(A(x, b, G.V));  // r = b - A x -> V_0
         }
         MLPG_TRY(norm2(G.V));
-        CU(ctx, cudaMemsetAsync(G.d_active_count, 0, sizeof(int), s));
+        CU(ctx, cudaMemsetAsync(G.d_active_count, 0, 2 * sizeof(int), s));
         k_start<<<(M + 127) / 128, 128, 0, s>>>(M, R, G.nrm2, G.bnorm, G.g, G.beta, G.active, G.kcol, G.resid, tol,
                                                 first_zero ? 1 : 0, G.d_active_count);
         CU_LAUNCH(ctx);
@@ -781,7 +1085,22 @@ static mlpg_status gmres_solve(mlpg_ctx *ctx, Gmres<T> &G, const ApplyFn<T> &A, 
             MLPG_TRY(A(z, nullptr, w));
             int gnorm = 0;
             const int nl = j + 1;
-            if (vec_ok && !G.reorth && (size_t)nl * M * sizeof(Ar) <= kUpdSmem) {
+            // counters of the systems still iterating: step j adds to slot (j + 1) % 2 and clears the other
+            int *cnt = G.d_active_count;
+            if (one_launch) {
+                cnt = G.d_active_count + ((j + 1) & 1);
+                int *next = G.d_active_count + (j & 1);
+                if constexpr (sizeof(T) == 8) {
+                    MLPG_TRY((G.reorth ? launch_gs<T, 4, true>(ctx, G, j, tol, cnt, next)
+                                       : launch_gs<T, 4, false>(ctx, G, j, tol, cnt, next)));
+                } else if (gs_systems<T>(M) == 8) {
+                    MLPG_TRY((G.reorth ? launch_gs<T, 8, true>(ctx, G, j, tol, cnt, next)
+                                       : launch_gs<T, 8, false>(ctx, G, j, tol, cnt, next)));
+                } else {
+                    MLPG_TRY((G.reorth ? launch_gs<T, 4, true>(ctx, G, j, tol, cnt, next)
+                                       : launch_gs<T, 4, false>(ctx, G, j, tol, cnt, next)));
+                }
+            } else if (vec_ok && !G.reorth && (size_t)nl * M * sizeof(Ar) <= kUpdSmem) {
                 // single classical pass, 16-byte vectors: dots (groups of kDotGroup
                 // basis vectors per grid row), reduce, update + norm partials
                 const int ng = (nl + kDotGroup - 1) / kDotGroup;
@@ -821,14 +1140,17 @@ static mlpg_status gmres_solve(mlpg_ctx *ctx, Gmres<T> &G, const ApplyFn<T> &A, 
                 CU_LAUNCH(ctx);
                 gnorm = g1;   // the norm partials are reduced inside k_givens
             }
-            CU(ctx, cudaMemsetAsync(G.d_active_count, 0, sizeof(int), s));
-            k_givens<<<wblk, kBlock, 0, s>>>(M, R, j, gnorm, G.partial, G.h, G.reorth ? G.h2 : nullptr, G.H, G.cs, G.sn, G.g, G.beta,
-                                             G.active, G.kcol, G.its, G.resid, G.bnorm, tol, G.d_active_count);
-            CU_LAUNCH(ctx);
+            if (!one_launch) {
+                CU(ctx, cudaMemsetAsync(G.d_active_count, 0, sizeof(int), s));
+                k_givens<<<wblk, kBlock, 0, s>>>(M, R, j, gnorm, G.partial, G.h, G.reorth ? G.h2 : nullptr, G.H, G.cs, G.sn,
+                                                 G.g, G.beta, G.active, G.kcol, G.its, G.resid, G.bnorm, tol,
+                                                 G.d_active_count);
+                CU_LAUNCH(ctx);
+            }
             jlast = j;
             bool check = (j + 1) % check_every == 0 || j + 1 == R;
             if (check) {
-                CU(ctx, cudaMemcpyAsync(G.h_active, G.d_active_count, sizeof(int), cudaMemcpyDeviceToHost, s));
+                CU(ctx, cudaMemcpyAsync(G.h_active, cnt, sizeof(int), cudaMemcpyDeviceToHost, s));
                 CU(ctx, cudaStreamSynchronize(s));
                 if (*G.h_active == 0) break;
             }

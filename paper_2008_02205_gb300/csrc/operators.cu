@@ -237,16 +237,24 @@ __global__ void k_scan1(int64_t n, const int *__restrict__ in, int32_t *__restri
 // multiply-adds per clock and SM (measured), 36 us at 96^2 S8 against 21 us of
 // memory.  Lanes that split a row's entries and add their parts by shuffles spent
 // a seventh of that time on the additions (54.7 us); here every lane's operation is
-// a product of the sum.
+// a product of the sum.  SPLIT > 1: that many lanes share a row's entries, for problems
+// too small to fill the chip, where the chain of loads decides.
+template <int SPLIT>
 __global__ void __launch_bounds__(256) k_spmm64(int64_t total, int m, const int32_t *__restrict__ rowptr,
                                                 const int32_t *__restrict__ col, const double *__restrict__ L64,
                                                 const double *__restrict__ X, const double *__restrict__ B,
                                                 double *__restrict__ Y) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    const int64_t row = e / m;
-    const int k = (int)(e - row * m);
-    const int32_t p0 = rowptr[row], p1 = rowptr[row + 1];
+    // SPLIT lanes of one (row, direction) are 32 / SPLIT apart, so that a run of lanes still reads a run of directions
+    const int64_t th = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    constexpr int PW = 32 / SPLIT;   // (row, direction) pairs per warp
+    const int64_t e = SPLIT == 1 ? th : (th >> 5) * PW + (th & (PW - 1));
+    const int part = SPLIT == 1 ? 0 : (int)((th & 31) / PW);
+    const bool live = e < total;
+    if (SPLIT == 1 && !live) return;
+    const int64_t row = live ? e / m : 0;
+    const int k = live ? (int)(e - row * m) : 0;
+    const int32_t r0 = rowptr[row], r1 = live ? rowptr[row + 1] : r0, len = r1 - r0;
+    const int32_t p0 = r0 + len * part / SPLIT, p1 = r0 + len * (part + 1) / SPLIT;
     const double *L = L64 + (int64_t)p0 * m + k, *Xk = X + k;
     double acc0 = 0.0, acc1 = 0.0;
     int32_t p = p0;
@@ -263,9 +271,12 @@ __global__ void __launch_bounds__(256) k_spmm64(int64_t total, int m, const int3
             acc1 = fma(l[q + 1], x[q + 1], acc1);
         }
     }
+#pragma unroll 4
     for (; p < p1; ++p, L += m) acc0 = fma(__ldg(L), __ldg(Xk + (int64_t)__ldg(col + p) * m), acc0);
-    const double acc = acc0 + acc1;
-    Y[e] = B ? B[e] - acc : acc;
+    double acc = acc0 + acc1;
+#pragma unroll
+    for (int o = PW; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (live && part == 0) Y[e] = B ? B[e] - acc : acc;
 }
 
 // FP32 batched L-apply: a team of TM lanes per row (4 rows per warp for
@@ -1118,13 +1129,22 @@ __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const 
     T *vs = reinterpret_cast<T *>(smem_raw);   // [kB][m], then m scale factors
     T *ssc = vs + kB * m;
     const int64_t blk = blockIdx.x;
-    const int mc = m >> 2;                      // float4 chunks per row
+    const int mc = m >> 2, ntask = kB * mc;     // float4 chunks per row
     const int32_t *mem = bmember + blk * kB;
+    const uint4 *P4 = reinterpret_cast<const uint4 *>(Pinv + blk * (int64_t)kB * kB * m);
+    // the first task's inverse entries do not depend on v: their loads overlap the staging
+    int t = threadIdx.x;
+    uint4 q[kB];
+    if (t < ntask) {
+        const int a = t / mc, c = t - a * mc;
+#pragma unroll
+        for (int b = 0; b < kB; ++b) q[b] = __ldg(P4 + ((int64_t)a * kB + b) * mc + c);
+    }
     if (sc)
         for (int k = threadIdx.x; k < m; k += blockDim.x) ssc[k] = (T)sc[k];
     __syncthreads();
-    for (int q = threadIdx.x; q < kB * m; q += blockDim.x) {
-        int b = q / m, k = q - b * m;
+    for (int e = threadIdx.x; e < kB * m; e += blockDim.x) {
+        int b = e / m, k = e - b * m;
         int32_t j = mem[b];
         T val = (T)0;
         if (j >= 0) {
@@ -1134,23 +1154,25 @@ __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const 
                 v[(int64_t)j * m + k] = val;
             }
         }
-        vs[q] = val;
+        vs[e] = val;
     }
     __syncthreads();
-    const uint4 *P4 = reinterpret_cast<const uint4 *>(Pinv + blk * (int64_t)kB * kB * m);
-    for (int t = threadIdx.x; t < kB * mc; t += blockDim.x) {
+    for (bool first = true; t < ntask; t += blockDim.x, first = false) {
         const int a = t / mc, c = t - a * mc;
+        if (!first) {
+#pragma unroll
+            for (int b = 0; b < kB; ++b) q[b] = __ldg(P4 + ((int64_t)a * kB + b) * mc + c);
+        }
         const int32_t i = mem[a];
         if (i < 0) continue;
         T acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
-#pragma unroll 4
+#pragma unroll
         for (int b = 0; b < kB; ++b) {
-            const uint4 p = P4[((int64_t)a * kB + b) * mc + c];
             const T *vb = vs + b * m + 4 * c;
-            acc0 += widen<T>(p.x) * vb[0];
-            acc1 += widen<T>(p.y) * vb[1];
-            acc2 += widen<T>(p.z) * vb[2];
-            acc3 += widen<T>(p.w) * vb[3];
+            acc0 += widen<T>(q[b].x) * vb[0];
+            acc1 += widen<T>(q[b].y) * vb[1];
+            acc2 += widen<T>(q[b].z) * vb[2];
+            acc3 += widen<T>(q[b].w) * vb[3];
         }
         T *zo = z + (int64_t)i * m + 4 * c;
         const T f = widen_factor<T>();
@@ -2081,11 +2103,17 @@ static void timing_end(mlpg_ctx *ctx) {
     ctx->ev_used++;
 }
 
+// values below which four lanes share a row: one thread per value leaves fewer than 16 warps per SM
+constexpr int64_t kSpmm64Split = 152 * 512;
 mlpg_status apply_L64_res(mlpg_ctx *ctx, const double *X, const double *B, double *Y) {
     const int64_t total = ctx->n * ctx->m;
     timing_begin(ctx);
-    k_spmm64<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col, ctx->L64, X, B,
-                                                                      Y);
+    if (total < kSpmm64Split)
+        k_spmm64<4><<<(unsigned)((total * 4 + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col,
+                                                                                 ctx->L64, X, B, Y);
+    else
+        k_spmm64<1><<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col,
+                                                                             ctx->L64, X, B, Y);
     timing_end(ctx);
     CU_LAUNCH(ctx);
     return MLPG_OK;
@@ -2236,8 +2264,8 @@ mlpg_status apply_prec(mlpg_ctx *ctx, T *v, T *z, const double *sc) {
         }
     }
     if ((ctx->m & 3) == 0)
-        k_bjacobi_blk<T><<<(unsigned)ctx->nblk, 256, smem, ctx->stream>>>(ctx->nblk, ctx->m, ctx->bmember, ctx->Pinv, v,
-                                                                           sc, z);
+        k_bjacobi_blk<T><<<(unsigned)ctx->nblk, std::min(256, (kB * (ctx->m >> 2) + 31) / 32 * 32), smem, ctx->stream>>>(
+            ctx->nblk, ctx->m, ctx->bmember, ctx->Pinv, v, sc, z);
     else
         k_bjacobi_scalar<T><<<(unsigned)ctx->nblk, 256, smem, ctx->stream>>>(ctx->nblk, ctx->m, ctx->bmember, ctx->Pinv,
                                                                               v, sc, z);
