@@ -24,6 +24,7 @@
 #include <cuda_fp16.h>
 
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace mlpg {
 
@@ -675,6 +676,7 @@ __global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_sp
     extern __shared__ float4 smem_x4[];
     __shared__ __align__(8) uint64_t full[kPairMaxWarps][NS], hbar;
     float *Xs = reinterpret_cast<float *>(smem_x4);
+    if (gridDim.x <= kPairMinTiles) pdl_trigger();   // one wave at most: the successor finds room at once
     const int t = blockIdx.x, m0 = blockIdx.y * mc, mcw = min(mc, m - m0);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int4 hd = head[t];
@@ -702,6 +704,10 @@ __global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_sp
         }
     }
     __syncthreads();
+    // X, B and Y from here on; the first record groups are on their way
+    pdl_wait();
+    X = after_wait(X);
+    B = after_wait(B);
     if constexpr (!GX && !UA) {
         const int hn = hd.w - hd.z;
         if (tid == 0) mbar_expect(&hbar, (uint32_t)(hn * mcw) * 4u);
@@ -1651,11 +1657,12 @@ template <int D, int DPT, bool GX, bool UA>
 static mlpg_status launch_pair(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
     const dim3 tg((unsigned)ctx->ntile, (unsigned)((ctx->m + ctx->tile_chunk - 1) / ctx->tile_chunk));
     const int TP = ctx->tile_rows / 2, G = ctx->tile_chunk / DPT;
-    k_spmm32_pair<D, DPT, GX, UA><<<tg, (TP * G + 31) / 32 * 32 * ctx->tile_ks, ctx->tile_smem, ctx->stream>>>(
-        ctx->m, ctx->tile_chunk, G, TP, ctx->tile_ks, ctx->tile_xs, ctx->tile_xs_f4, pairs_per_warp(TP, G),
-        reinterpret_cast<const int4 *>(ctx->t_head), ctx->t_plen, reinterpret_cast<const int2 *>(ctx->t_row), ctx->t_hcol,
-        reinterpret_cast<const float4 *>(ctx->t_rec), ctx->coef32, ctx->bptr, ctx->t_bhalo, ctx->bval32, ctx->nb, X, B, Y,
-        ctx->d_tile_err);
+    CU(ctx, launch_pdl(k_spmm32_pair<D, DPT, GX, UA>, tg, dim3((unsigned)((TP * G + 31) / 32 * 32 * ctx->tile_ks)),
+                       ctx->tile_smem, ctx->stream, ctx->m, ctx->tile_chunk, G, TP, ctx->tile_ks, ctx->tile_xs,
+                       ctx->tile_xs_f4, pairs_per_warp(TP, G), reinterpret_cast<const int4 *>(ctx->t_head), ctx->t_plen,
+                       reinterpret_cast<const int2 *>(ctx->t_row), ctx->t_hcol,
+                       reinterpret_cast<const float4 *>(ctx->t_rec), ctx->coef32, ctx->bptr, ctx->t_bhalo, ctx->bval32,
+                       ctx->nb, X, B, Y, ctx->d_tile_err));
     CU_LAUNCH(ctx);
     return MLPG_OK;
 }
