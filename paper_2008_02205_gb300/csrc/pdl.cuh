@@ -11,8 +11,8 @@
 //
 // Applies back to back at 32^2 S4: 4.0 -> 3.0 us.  Tried on every kernel of the Krylov loops
 // and not kept there: blocks that wait hold registers and shared memory that the
-// running kernel's successors need (256^2 S8 mixed step 42.5 -> 51.2 ms, eight batched
-// problems 37.5 -> 40.5, 32^2 S4 FP64 step 20.5 -> 24.3).
+// running kernel's successors need (eight batched problems 37.5 -> 40.5 ms, 32^2 S4 FP64
+// step 20.5 -> 24.3).
 #pragma once
 
 #include <cuda_runtime.h>
