@@ -38,7 +38,8 @@ def _flags():
 def _compile(src):
     obj = os.path.join(BUILD, os.path.basename(src) + ".o")
     path = os.path.join(CSRC, src)
-    deps = [path, os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "fixed_sum.cuh"), os.path.join(CSRC, "pdl.cuh"), os.path.join(ROOT, "include", "mlpg.h")]
+    heads = [os.path.join(CSRC, h) for h in sorted(os.listdir(CSRC)) if h.endswith((".h", ".cuh"))]
+    deps = [path, os.path.join(ROOT, "include", "mlpg.h")] + heads
     if os.path.exists(obj) and all(os.path.getmtime(obj) >= os.path.getmtime(d) for d in deps):
         return obj
     lang = ["-x", "cu"] if src.endswith(".cu") else []

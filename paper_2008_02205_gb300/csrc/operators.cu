@@ -25,6 +25,7 @@
 
 #include "internal.h"
 #include "pdl.cuh"
+#include "widen.cuh"
 
 namespace mlpg {
 
@@ -1105,6 +1106,18 @@ __global__ void __launch_bounds__(256) k_block_inv(int64_t nblk, int m, const in
     if (lane == 0) Pscale[k * (int64_t)m + dir] = amax > 0.0f ? ldexpf(1.0f, ex - 14) : 1.0f;
 }
 
+// An FP32 value (its bits) in the vector's type; for FP64 by integer moves (widen.cuh), because the kernel is
+// bound by the FP64 units (96^2 S8: 28.9 us with the conversion).
+template <typename T>
+__device__ __forceinline__ T widen(uint32_t b) {
+    if constexpr (sizeof(T) == 4) return __uint_as_float(b);
+    else {
+        uint32_t hi, lo;
+        widen_words(b, hi, lo);
+        return __hiloint2double((int)hi, (int)lo);
+    }
+}
+
 // z = P^{-1} v, one CTA per block of kB points.  The kB input rows v[member]
 // (kB x m values) are staged in shared memory once; the block's inverse
 // (kB x kB x m floats, contiguous) is streamed with 16-byte loads.  Thread
@@ -1112,21 +1125,6 @@ __global__ void __launch_bounds__(256) k_block_inv(int64_t nblk, int m, const in
 // Requires m % 4 == 0 (the caller falls back to k_bjacobi_scalar otherwise).
 // With sc != null the input rows are first scaled by sc[direction] and the
 // scaled rows written back to v (the GMRES basis normalisation, fused here).
-// An FP32 value (its bits) in the vector's type, divided by widen_factor.  For FP64 the bits move to their
-// places in a double whose exponent lacks the difference of the biases, 2^-896 (exact, zeros and
-// subnormals included): integer moves, because the conversion runs on the FP64 units, at 1.9
-// per clock and SM, and would cost as much as the multiply-add (96^2 S8: 28.9 us with it).
-template <typename T>
-__device__ __forceinline__ T widen(uint32_t b) {
-    if constexpr (sizeof(T) == 4) return __uint_as_float(b);
-    else return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3)), (int)(b << 29));
-}
-template <typename T>
-__device__ __forceinline__ T widen_factor() {
-    if constexpr (sizeof(T) == 4) return 1.0f;
-    else return __hiloint2double((1023 + 896) << 20, 0);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const int32_t *__restrict__ bmember,
                                                      const float *__restrict__ Pinv, T *__restrict__ v,
@@ -1181,8 +1179,7 @@ __global__ void __launch_bounds__(256) k_bjacobi_blk(int64_t nblk, int m, const 
             acc3 += widen<T>(q[b].w) * vb[3];
         }
         T *zo = z + (int64_t)i * m + 4 * c;
-        const T f = widen_factor<T>();
-        zo[0] = acc0 * f; zo[1] = acc1 * f; zo[2] = acc2 * f; zo[3] = acc3 * f;
+        zo[0] = acc0; zo[1] = acc1; zo[2] = acc2; zo[3] = acc3;
     }
 }
 
