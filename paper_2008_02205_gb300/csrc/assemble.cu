@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
                 for (int p = tid & 3; p < P; p += 4) {
                     const float dx = qfx[p] - ax, dy = qfy[p] - ay, r2 = dx * dx + dy * dy;
                     bool sup = r2 < R2;
-                    if (fabsf(r2 - R2) <= slack) {
+                    if (!(fabsf(r2 - R2) > slack)) {   // close, or beyond FP32's range
                         const double ex = qx[p] - fx[a], ey = qy[p] - fy[a];
                         sup = ex * ex + ey * ey < fR2[a];
                     }

@@ -551,14 +551,14 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
             const float fxr = (float)(xj[0] - g[0]), fyr = (float)(xj[1] - g[1]), fzr = (float)(xj[2] - g[2]);
             const float Rf = (float)Rj, R2f = Rf * Rf;
             const float cx = fxr - red_f[0], cy = fyr - red_f[1], cz = fzr - red_f[2], reach = (Rf + red_f[3]) * 1.0001f;
-            if (cx * cx + cy * cy + cz * cz < reach * reach) {
+            if (!(cx * cx + cy * cy + cz * cz > reach * reach)) {   // (squares beyond FP32's range: all functions)
                 // the coordinates are rounded to 2^-24 of the largest, at most a few R: 1e-4 is far outside
                 const float len2 = fxr * fxr + fyr * fyr + fzr * fzr + R2f, slack = 1e-4f * len2;
                 for (int q = 0; q < P; ++q) {
                     const float dx = qf[3 * q] - fxr, dy = qf[3 * q + 1] - fyr, dz = qf[3 * q + 2] - fzr;
                     const float r2 = dx * dx + dy * dy + dz * dz;
                     bool sup = r2 < R2f;
-                    if (fabsf(r2 - R2f) <= slack) {
+                    if (!(fabsf(r2 - R2f) > slack)) {   // close, or beyond FP32's range
                         const double ex = qx[3 * q] - xj[0], ey = qx[3 * q + 1] - xj[1], ez = qx[3 * q + 2] - xj[2];
                         sup = ex * ex + ey * ey + ez * ez < R2;
                     }

@@ -27,3 +27,21 @@ def test_fp64_step_scales_with_its_source(scale):
             tp.integrate().assemble().step(prob.dt)
             out.append(tp.state() / s)
     assert _rel(out[1], out[0]) < 1e-10
+
+
+@pytest.mark.parametrize("dim,side,scale", [(2, 10, 1e22), (2, 10, 1e-25), (3, 5, 1e22), (3, 5, 1e-25)])
+def test_forms_scale_with_the_lengths(dim, side, scale):
+    """Which functions reach a point is decided in FP32 where that is certain; lengths whose squares leave
+    FP32's range are decided in FP64.  M0_ij = V_j int u_i u_j, K_ij = V_j int du_i du_j with u of order 1 / V:
+    powers 0 and -2 of the unit."""
+    forms = []
+    for s in (1.0, scale):
+        p = mi.small_2d(side, sn=4, seed=4) if dim == 2 else mi.lognormal_3d(side, sn=4, seed=4)
+        with pkg.TransportProblem(p.x * s, p.R * s, p.omega, p.w, p.sigma_t, p.sigma_s, p.q, lo=[0.0] * dim,
+                                  hi=[s] * dim) as tp:
+            tp.integrate().assemble()
+            forms.append((tp.neighbors()[1], tp.forms()[0]))
+    (col, a), (col1, b) = forms
+    assert np.array_equal(col, col1)
+    for k, power in ((0, 0), (3 + 3 * dim, -2)):   # M0, K_xx
+        assert np.abs(b[k] / scale**power - a[k]).max() < 1e-11 * np.abs(a[k]).max()
