@@ -665,13 +665,27 @@ static int pairs_per_warp(int TP, int G) {
     return most;
 }
 
+// (L_d X)_row over the row's own entries, without its face terms
+template <int D>
+__device__ __noinline__ float own_row_sum(const int32_t *rowptr, const int32_t *col, const float *A32, int64_t nnz,
+                                          const float *c, const float *X, int m, int32_t row, int d) {
+    float sum = 0.0f;
+    for (int32_t p = rowptr[row]; p < rowptr[row + 1]; ++p) {
+        float v = A32[p];
+        for (int q = 1; q < NA<D>(); ++q) v = fmaf(c[16 * d + q], A32[q * nnz + p], v);
+        sum = fmaf(v, X[(int64_t)col[p] * m + d], sum);
+    }
+    return sum;
+}
+
 // tile header: first slot, slots per pair (unused here), halo range
 template <int D, int DPT, bool GX, bool UA>
 __global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_spmm32_pair(
     int m, int mc, int G, int TP, int KS, int xs, int hx_f4, int ppw, const int4 *__restrict__ head,
     const int32_t *__restrict__ plen, const int2 *__restrict__ trow, const int32_t *__restrict__ hcol,
     const float4 *__restrict__ rec, const float *__restrict__ coef32, const int32_t *__restrict__ bptr,
-    const int32_t *__restrict__ bhalo, const float *__restrict__ bval, int64_t nb, const float *__restrict__ X,
+    const int32_t *__restrict__ bhalo, const float *__restrict__ bval, int64_t nb, const int32_t *rowptr,
+    const int32_t *col, const float *A32, int64_t nnz, const float *__restrict__ X,
     const float *__restrict__ B, float *__restrict__ Y, int *__restrict__ err) {
     constexpr int K = NA<D>(), F4 = pair_f4<D>(), GF = group_f4<D>(), NQ = DPT / 4, NS = kPairStages;
     extern __shared__ float4 smem_x4[];
@@ -845,6 +859,19 @@ __global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_sp
         float res[DPT];
 #pragma unroll
         for (int j = 0; j < DPT; ++j) res[j] = r == 0 ? acc[j].x : acc[j].y;
+        // slots of the other row's columns and padding slots add a zero times X: nothing for a finite X.  A sum
+        // that is not finite is taken again over the row's own entries, so that an infinity or a NaN in X
+        // reaches the rows whose pattern holds its point and no others.
+        float nf = 0.0f;
+#pragma unroll
+        for (int j = 0; j < DPT; ++j) nf = fmaf(res[j], 0.0f, nf);
+        if (nf != nf)
+#pragma unroll
+            for (int j = 0; j < DPT; ++j) {
+                const int k = qoff[j / 4] + j % 4;
+                if (on[j / 4] && k < mcw && !isfinite(res[j]))
+                    res[j] = own_row_sum<D>(rowptr, col, A32, nnz, coef32, X, m, row, m0 + k);
+            }
         // outflow-face terms of a boundary row: sum_f max(Omega . n_f, 0) (S_f X)_i
         const int32_t q1 = bptr[row + 1];
         for (int32_t p = bptr[row]; p < q1; ++p) {
@@ -1659,7 +1686,7 @@ static mlpg_status launch_pair(mlpg_ctx *ctx, const float *X, const float *B, fl
                        ctx->tile_xs_f4, pairs_per_warp(TP, G), reinterpret_cast<const int4 *>(ctx->t_head), ctx->t_plen,
                        reinterpret_cast<const int2 *>(ctx->t_row), ctx->t_hcol,
                        reinterpret_cast<const float4 *>(ctx->t_rec), ctx->coef32, ctx->bptr, ctx->t_bhalo, ctx->bval32,
-                       ctx->nb, X, B, Y, ctx->d_tile_err));
+                       ctx->nb, ctx->rowptr, ctx->col, ctx->A32, ctx->nnz, X, B, Y, ctx->d_tile_err));
     CU_LAUNCH(ctx);
     return MLPG_OK;
 }
