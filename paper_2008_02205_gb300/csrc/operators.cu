@@ -1856,8 +1856,9 @@ static mlpg_status init_tiles(mlpg_ctx *ctx) {
     spatial_order(ctx->n, D, ctx->h_x.data(), ctx->h_order.data());
     TilePlan P;
     // automatic choice: 3D halos (some 700 rows for 32) leave room for few directions per chunk, and
-    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit
-    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->n * m < (int64_t(1) << 31);
+    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit.  A
+    // request for 64 rows, which gather mode does not take, still goes to the staged tiles.
+    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->opt.tile_rows != 64 && ctx->n * m < (int64_t(1) << 31);
     if (kind != 4 && !skip) {
         MLPG_TRY(plan_tiles<D>(ctx, false, kind == 3, P));
         // staged halos pay while the records are read by few chunks; past two chunks the gather

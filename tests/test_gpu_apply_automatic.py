@@ -47,6 +47,8 @@ CASES = [
     (3, 5, 8, 27, 0, 2, False),     # staged tiles in 3D
     (3, 6, 4, 23, 0, 2, False),
     (3, 6, 4, 24, 0, 4, False),     # gather mode
+    (3, 6, 4, 24, 32, 4, False),
+    (3, 6, 4, 24, 64, 2, False),    # gather mode takes at most 32 rows: staged tiles
 ]
 
 
