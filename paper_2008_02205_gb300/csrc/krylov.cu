@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 
 #include "internal.h"
+#include "pair_sum.cuh"
 
 namespace mlpg {
 
@@ -508,7 +509,8 @@ __global__ void k_givens(int M, int R, int j, int G, const double *__restrict__ 
 // update.  The systems are independent, so a cluster of CTAs takes DV of them (32 bytes of
 // each row: one sector): every CTA keeps its rows of w in shared memory for the whole
 // step, streams its rows of the basis, and the cluster adds the CTAs' sums through
-// distributed shared memory, in rank order.
+// distributed shared memory, in rank order.  FP32 products are summed in pairs of floats up to
+// the warp's sums (pair_sum.cuh), in FP64 from there.
 //
 // Why: as separate passes (dots, reduction, update, norm, Givens; six launches with
 // REORTH) a small problem's step is launch and reduction latency: 38 us at 32^2 S4,
@@ -541,23 +543,30 @@ struct GsShape {
 // Sums of v[NV] over the lanes of a warp that differ in the bits from TPR up, halving the values at each
 // step (a lane keeps one half and passes the other on): NV - NV / n additions instead of NV log2 n.
 // Afterwards v[0 .. NV TPR / 32) hold the sums of the values from the returned index on.
-template <int HALF, int O, int NV, typename A>
-__device__ __forceinline__ int lanes_sum_from(A (&v)[NV], int lane) {
+__device__ __forceinline__ Sum<double> shfl_xor(const Sum<double> &s, int o) {
+    return {__shfl_xor_sync(0xffffffffu, s.v, o)};
+}
+__device__ __forceinline__ Sum<float> shfl_xor(const Sum<float> &s, int o) {
+    return {__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
+}
+template <int HALF, int O, int NV, typename T>
+__device__ __forceinline__ int lanes_sum_from(Sum<T> (&v)[NV], int lane) {
     if constexpr (O < 32) {
         const bool up = lane & O;
 #pragma unroll
         for (int i = 0; i < HALF; ++i) {
-            const A lo = v[i], hi = v[i + HALF];
-            v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, O);
+            const Sum<T> lo = v[i], hi = v[i + HALF];
+            v[i] = up ? hi : lo;
+            v[i].add(shfl_xor(up ? lo : hi, O));
         }
-        return (up ? HALF : 0) + lanes_sum_from<HALF / 2, O * 2, NV, A>(v, lane);
+        return (up ? HALF : 0) + lanes_sum_from<HALF / 2, O * 2, NV, T>(v, lane);
     } else {
         return 0;
     }
 }
-template <int NV, int TPR, typename A>
-__device__ __forceinline__ int lanes_sum(A (&v)[NV], int lane) {
-    return lanes_sum_from<NV / 2, TPR, NV, A>(v, lane);
+template <int NV, int TPR, typename T>
+__device__ __forceinline__ int lanes_sum(Sum<T> (&v)[NV], int lane) {
+    return lanes_sum_from<NV / 2, TPR, NV, T>(v, lane);
 }
 
 template <typename T, int DV, bool REORTH>
@@ -594,10 +603,10 @@ __global__ void __launch_bounds__(GsShape<T, DV>::threads) k_gs_step(int64_t n, 
         *reinterpret_cast<V16 *>(ws + (r * TPR + q) * VEC) = *reinterpret_cast<const V16 *>(wb + (int64_t)r * M);
     // (each thread only touches its own rows of ws: no barrier)
     const int lane = tid & 31, warp = tid >> 5;
-    auto block_sum = [&](A (&v)[NV], int na, double *out) {   // out[a][d] = sums over the CTA's threads
-        const int first = lanes_sum<NV, TPR, A>(v, lane);
+    auto block_sum = [&](Sum<T> (&v)[NV], int na, double *out) {   // out[a][d] = sums over the CTA's threads
+        const int first = lanes_sum<NV, TPR, T>(v, lane);
 #pragma unroll
-        for (int i = 0; i < NV * TPR / 32; ++i) red[(warp * TPR + q) * NV + first + i] = (double)v[i];
+        for (int i = 0; i < NV * TPR / 32; ++i) red[(warp * TPR + q) * NV + first + i] = v[i].value();
         __syncthreads();
         for (int o = tid; o < na * DV; o += NT) {
             const int a = o / DV, d = o - a * DV, qq = d / VEC, c = d - qq * VEC;
@@ -611,39 +620,25 @@ __global__ void __launch_bounds__(GsShape<T, DV>::threads) k_gs_step(int64_t n, 
     auto dots = [&](double *out) {   // out[l][d] = this CTA's part of V_l . w
         for (int l0 = 0; l0 < nl; l0 += kGsGroup) {
             const int ng = min(kGsGroup, nl - l0);
-            A acc[NV];
+            Sum<T> acc[NV];
 #pragma unroll
-            for (int a = 0; a < NV; ++a) acc[a] = 0;
-            // FP32: sums of four rows, then their sum; FP64 keeps one sum (an addition costs as much as a product)
-            constexpr int CH = sizeof(T) == 4 ? 4 : 1 << 30;
-            for (int rb = r0; rb < rows;) {
-                A pt[sizeof(T) == 4 ? NV : 1];
-                if constexpr (sizeof(T) == 4)
+            for (int a = 0; a < NV; ++a) acc[a].clear();
+            for (int rb = r0; rb < rows; rb += RPI) {
+                T wv[VEC];
+                unpack(*reinterpret_cast<const V16 *>(ws + (rb * TPR + q) * VEC), wv);
+                const T *vr = Vb + (int64_t)rb * M + l0 * vs;
+                V16 v[kGsGroup];
 #pragma unroll
-                    for (int a = 0; a < NV; ++a) pt[a] = 0;
-                for (int c4 = 0; c4 < CH && rb < rows; ++c4, rb += RPI) {
-                    T wv[VEC];
-                    unpack(*reinterpret_cast<const V16 *>(ws + (rb * TPR + q) * VEC), wv);
-                    const T *vr = Vb + (int64_t)rb * M + l0 * vs;
-                    V16 v[kGsGroup];
+                for (int a = 0; a < kGsGroup; ++a)
+                    if (a < ng) v[a] = __ldg(reinterpret_cast<const V16 *>(vr + a * vs));
 #pragma unroll
-                    for (int a = 0; a < kGsGroup; ++a)
-                        if (a < ng) v[a] = __ldg(reinterpret_cast<const V16 *>(vr + a * vs));
+                for (int a = 0; a < kGsGroup; ++a)
+                    if (a < ng) {
+                        T x[VEC];
+                        unpack(v[a], x);
 #pragma unroll
-                    for (int a = 0; a < kGsGroup; ++a)
-                        if (a < ng) {
-                            T x[VEC];
-                            unpack(v[a], x);
-#pragma unroll
-                            for (int c = 0; c < VEC; ++c) {
-                                if constexpr (sizeof(T) == 4) pt[a * VEC + c] += (A)x[c] * (A)wv[c];
-                                else acc[a * VEC + c] += (A)x[c] * (A)wv[c];
-                            }
-                        }
-                }
-                if constexpr (sizeof(T) == 4)
-#pragma unroll
-                    for (int a = 0; a < NV; ++a) acc[a] += pt[a];
+                        for (int c = 0; c < VEC; ++c) acc[a * VEC + c].add_product(x[c], wv[c]);
+                    }
             }
             block_sum(acc, ng, out + l0 * DV);
         }
@@ -658,7 +653,7 @@ __global__ void __launch_bounds__(GsShape<T, DV>::threads) k_gs_step(int64_t n, 
         }
         __syncthreads();
     };
-    auto update = [&](const double *h, bool last, A (&nrm)[NV]) {   // w -= sum_l h_l V_l; last: ||w||^2, to global
+    auto update = [&](const double *h, bool last, Sum<T> (&nrm)[NV]) {   // w -= sum_l h_l V_l; last: ||w||^2, to global
         for (int o = tid; o < nl * DV; o += NT) hc[o] = (A)h[o];
         __syncthreads();
         for (int r = r0; r < rows; r += RPI) {
@@ -687,7 +682,7 @@ __global__ void __launch_bounds__(GsShape<T, DV>::threads) k_gs_step(int64_t n, 
 #pragma unroll
             for (int c = 0; c < VEC; ++c) {
                 wt[c] = (T)wv[c];
-                if (last) nrm[c] += (A)wt[c] * (A)wt[c];
+                if (last) nrm[c].add_product(wt[c], wt[c]);
             }
             const V16 o = pack<T>(wt);
             *wp = o;
@@ -695,9 +690,9 @@ __global__ void __launch_bounds__(GsShape<T, DV>::threads) k_gs_step(int64_t n, 
         }
         __syncthreads();
     };
-    A nrm[NV];   // [0 .. VEC): the norm
+    Sum<T> nrm[NV];   // [0 .. VEC): the norm
 #pragma unroll
-    for (int c = 0; c < NV; ++c) nrm[c] = 0;
+    for (int c = 0; c < NV; ++c) nrm[c].clear();
     dots(part);
     cluster_sum(0, nl * DV);
     update(tot, !REORTH, nrm);
