@@ -7,7 +7,7 @@
 // every few Arnoldi steps.  Orthogonalisation is classical Gram-Schmidt
 // applied twice (CGS2) in FP64, or once in the FP32 correction solves (16-byte
 // vectorised passes); sums over a block are formed in FP64, or from FP32 values in
-// pairs of floats, and sums over blocks in FP64 whatever the vector type.
+// three floats, and sums over blocks in FP64 whatever the vector type.
 // Right preconditioning by the block-Jacobi inverses (16-point Morton blocks)
 // of each L_m.
 //
@@ -313,19 +313,14 @@ __device__ __forceinline__ void block_sums(const T (*acc)[VEC], int nacc, int l0
         __syncthreads();
         for (int o = t; o < na * M; o += kBlock) {
             const int a = o / M, m = o - a * M;
-            double sum;
+            double sum = 0.0;
             if constexpr (sizeof(T) == 4) {
-                // an unevaluated sum of two floats (two-sum: hi + lo exact), 48 bits: a conversion and an
-                // FP64 addition per value took 18 of the dots' 29 us at 256^2 S8
-                float hi = 0.0f, lo = 0.0f;
-                for (int k = 0; k < RB; ++k) {
-                    const float x = sh[a * RM + k * M + m], s = __fadd_rn(hi, x), bb = __fsub_rn(s, hi);
-                    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
-                    hi = s;
-                }
-                sum = (double)hi + (double)lo;
+                // three floats (72 bits): a conversion and an FP64 addition per value, both in the FP64 units,
+                // took 18 of the dots' 29 us at 256^2 S8 (26.5 us with the conversion by integer moves)
+                TripleSum ts;
+                for (int k = 0; k < RB; ++k) ts.add(sh[a * RM + k * M + m]);
+                sum = ts.value();
             } else {
-                sum = 0.0;
                 for (int k = 0; k < RB; ++k) sum += sh[a * RM + k * M + m];
             }
             partial[((int64_t)(l0 + a0 + a) * M + m) * G + blockIdx.x] = sum;

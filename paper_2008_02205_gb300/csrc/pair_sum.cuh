@@ -44,4 +44,17 @@ struct Sum<float> {
     MLPG_HD double value() const { return (double)hi + (double)lo; }
 };
 
+// The same with three floats: the errors of lo's additions go on into a third, so that a sum of floats
+// is held in more than the 53 bits of an FP64 sum.
+struct TripleSum {
+    float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+    MLPG_HD static float two_sum(float &s, float x) {   // s += x; returns the rounding error
+        const float a = s, b = add_rn(add_rn(a, x), -a);
+        s = add_rn(a, x);
+        return add_rn(add_rn(a, -add_rn(s, -b)), add_rn(x, -b));
+    }
+    MLPG_HD void add(float x) { lo = add_rn(lo, two_sum(mid, two_sum(hi, x))); }
+    MLPG_HD double value() const { return (double)hi + ((double)mid + (double)lo); }
+};
+
 }  // namespace mlpg

@@ -3,7 +3,8 @@ chains of products and a tree of chains, as the Arnoldi step forms them, against
 rounded products.
 
 Each addition's error goes into lo exactly and is rounded there to 24 bits of lo, which holds at most
-2^-24 count of the magnitudes' sum: count^2 2^-48 of it bounds the error, against 2^-24 for a sum of floats."""
+2^-24 count of the magnitudes' sum: count^2 2^-48 of it bounds the error, against 2^-24 for a sum of floats.
+Three floats carry the errors on once more: count^3 2^-72, below an FP64 sum's 2^-53 per addition."""
 import math
 import os
 import shutil
@@ -27,8 +28,10 @@ int main() {
         }
         for (int o = 16; o > 0; o /= 2)
             for (int l = 0; l < o; ++l) s[l].add(s[l + o]);
-        const double v = s[0].value();
-        fwrite(&v, 8, 1, stdout);
+        mlpg::TripleSum t;   // one chain over the same products
+        for (int k = 0; k < 256; ++k) t.add(x[2 * k] * x[2 * k + 1]);
+        const double v[2] = {s[0].value(), t.value()};
+        fwrite(v, 8, 2, stdout);
     }
 }
 '''
@@ -47,6 +50,9 @@ def test_pair_sums_hold_more_than_forty_bits(tmp_path):
     x[50:100, 128:] = x[50:100, :128] * [-1.0, 1.0]                  # sums that cancel
     x = x.astype(np.float32)
     out = np.frombuffer(subprocess.run([str(exe)], input=x.tobytes(), capture_output=True, check=True).stdout, np.float64)
-    for v, row in zip(out, x):
+    for (v, t), row in zip(out.reshape(-1, 2), x):
         p = (row[:, 0] * row[:, 1]).astype(np.float64)
-        assert abs(v - math.fsum(p)) <= 13**2 * 2.0**-48 * math.fsum(np.abs(p))
+        exact, size = math.fsum(p), math.fsum(np.abs(p))
+        assert abs(v - exact) <= 13**2 * 2.0**-48 * size
+        # the two roundings of the final sum, and 256 additions' errors 2^-24 three times over
+        assert abs(t - exact) <= 2.0**-52 * abs(exact) + 256**3 * 2.0**-72 * size
