@@ -814,19 +814,38 @@ __global__ void k_axpy1(int64_t N, const T *__restrict__ u, T *__restrict__ x) {
     if (e < N) x[e] += u[e];
 }
 
+// FP64 value of a sum; FP32 by integer moves (widen.cuh)
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+    uint32_t hi, lo;
+    widen_words(__float_as_uint(x), hi, lo);
+    return __hiloint2double((int)hi, (int)lo);
+}
+
 // out[i] = sum_m w[m] x[i][m]  (angular reduction D, Sec. 4.2), eight lanes per point: three FP64
 // additions of the lanes' parts per four points (a warp per point took five for each: 34 us at 256^2 S8,
-// all of it in the FP64 units)
+// all of it in the FP64 units).  FP32 products are added in FP32 over every 32nd direction only, four sums
+// per lane, and in FP64 from there.
 template <typename T>
 __global__ void k_Dreduce(int64_t n, int M, const double *__restrict__ w, const T *__restrict__ x,
                           double *__restrict__ out) {
     using A = typename Arith<T>::type;
+    constexpr int NS = sizeof(T) == 4 ? 4 : 1;   // sums per lane
     const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3;
     const int lane = threadIdx.x & 7;
-    A sl = 0;
+    A sl[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) sl[k] = 0;
     if (i < n)
-        for (int m = lane; m < M; m += 8) sl += (A)w[m] * (A)x[i * M + m];
-    double s = (double)sl;
+        for (int m0 = lane; m0 < M; m0 += 8 * NS)
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const int m = m0 + 8 * k;
+                if (m < M) sl[k] += (A)w[m] * (A)x[i * M + m];
+            }
+    double s = widen(sl[0]);
+#pragma unroll
+    for (int k = 1; k < NS; ++k) s += widen(sl[k]);
     for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (i < n && lane == 0) out[i] = s;
 }
