@@ -23,6 +23,7 @@
 
 #include <cuda_fp16.h>
 
+#include "four_pi.cuh"
 #include "internal.h"
 #include "pdl.cuh"
 #include "widen.cuh"
@@ -30,7 +31,6 @@
 namespace mlpg {
 
 namespace {
-constexpr double kFourPi = 12.566370614359172953850573533118;
 
 __global__ void k_rowidx(int64_t n, const int32_t *__restrict__ rowptr, int32_t *__restrict__ rowidx) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -990,12 +990,14 @@ __global__ void k_ms_spmv(int64_t n, int64_t nnz, const int32_t *__restrict__ ro
 #pragma unroll
     for (int a = 0; a < NT<D>(); ++a)
         for (int o = 4; o > 0; o >>= 1) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], o);
-    if (i < n && lane == 0)
+    double v = acc[0];   // lane a takes array a
 #pragma unroll
-        for (int a = 0; a < NT<D>(); ++a) {
-            abc[a * n + i] = acc[a];
-            if (abc32) abc32[a * n + i] = (float)(acc[a] * (1.0 / kFourPi));
-        }
+    for (int a = 1; a < NT<D>(); ++a)
+        if (lane == a) v = acc[a];
+    if (i < n && lane < NT<D>()) {
+        abc[lane * n + i] = v;
+        if (abc32) abc32[lane * n + i] = div_four_pi_f(v);
+    }
 }
 
 // thread per (point, direction)
@@ -1009,7 +1011,7 @@ __global__ void k_ms_expand(int64_t total, int m, int64_t n, const double *__res
     double v = abc[i];
 #pragma unroll
     for (int a = 0; a < D; ++a) v = v + coef[kCS * k + 1 + a] * abc[(1 + a) * n + i];
-    out[e] = (T)(v * (1.0 / kFourPi));
+    out[e] = (T)div_four_pi(v);
 }
 
 // FP32 variant: the per-point products arrive pre-scaled by 1/(4 pi) in float
