@@ -209,6 +209,10 @@ mlpg_status mlpg_step(mlpg_ctx *ctx, double dt);
  * problems, run concurrently: the caller's thread steps ctxs[0] and one host
  * thread per further context steps the others, each on its own context
  * stream, so their kernels overlap on the device.  dt[i] is problem i's step.
+ * The kernels are chosen for the problems together (a batch that fills the
+ * device takes another Gram-Schmidt form than a small problem alone), so a
+ * state may differ in rounding from that of the same step taken by mlpg_step
+ * or in another batch; the same call on the same states gives the same bits.
  * The contexts must be distinct and must not share a stream (contexts created
  * with a NULL stream own one): otherwise MLPG_ERR_ARG before any step.
  * Returns MLPG_OK when every step succeeded, else the first failing status in
