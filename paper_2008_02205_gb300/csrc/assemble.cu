@@ -521,8 +521,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_assemble_2d(AsmArgs A) {
 //   2. RK functions, two lanes per point over the point's own list (about 13 of the
 //      35 functions that reach the cell); the derivative moments are the third-order
 //      moments of the kernel's radial derivative (9 sums instead of 12);
-//   3. the table sqrt(w) (U, U_x, U_y) in fixed point, 54 bits below the chunk's
-//      largest U and largest derivative;
+//   3. the table sqrt(w) (U, U_x, U_y) in fixed point, 54 bits below each function's
+//      largest U and largest derivative in the chunk;
 //   4. every unordered pair a <= b sums the nine products over the points both
 //      support, in 64-bit integers (fixed_sum.cuh), and adds them to the pattern's
 //      upper entry; G(b, a) goes to six buffers of its own, and k_mirror_2d fills the lower
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
     __shared__ uint8_t plist[kLinPts][kMaxS];
     __shared__ int wcnt[kLinThreads / 32];
     __shared__ int S_sh;
-    __shared__ unsigned top[2];
+    __shared__ int16_t xu[kMaxS], xd[kMaxS];   // exponents of each function's largest values in the chunk
     extern __shared__ __align__(16) double lin_tab[];
     const int64_t i = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -672,7 +672,6 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
             qsw[tid] = sqrt(wq);
             qfs[tid] = fs;
         }
-        if (tid == 0) top[0] = top[1] = 0;
         for (int k = tid; k < P * S; k += kLinThreads) {
             tabu[k] = 0.0;
             tabd[k] = make_double2(0.0, 0.0);
@@ -710,7 +709,6 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
         }
         __syncthreads();
         // 2. RK functions: two lanes per point, 16 points per warp
-        unsigned mx0 = 0, mx1 = 0;   // high words of the largest |sqrt(w) u|, |sqrt(w) du|
         for (int p0 = warp * 16; p0 < P; p0 += kLinThreads / 2) {
             const int p = min(p0 + (lane >> 1), P - 1), l2 = lane & 1;   // spare lanes repeat the last point
             const bool mine = p0 + (lane >> 1) < P;
@@ -775,20 +773,11 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
                 const double ux = W * (gx + X * Cx[1] + Y * Cx[2]) + h * dx, uy = W * (gy + X * Cy[1] + Y * Cy[2]) + h * dy;
                 tabu[p * S + a] = ok ? u : 0.0;
                 tabd[p * S + a] = ok ? make_double2(ux, uy) : make_double2(0.0, 0.0);
-                if (ok) {
-                    mx0 = max(mx0, (unsigned)__double2hiint(u) & 0x7fffffffu);
-                    mx1 = max(mx1, max((unsigned)__double2hiint(ux) & 0x7fffffffu, (unsigned)__double2hiint(uy) & 0x7fffffffu));
-                }
             }
         }
-        mx0 = __reduce_max_sync(0xffffffffu, mx0);
-        mx1 = __reduce_max_sync(0xffffffffu, mx1);
-        if (lane == 0) {
-            atomicMax(&top[0], mx0);
-            atomicMax(&top[1], mx1);
-        }
         __syncthreads();
-        if (tid < S)   // vectors, before the table changes to fixed point
+        if (tid < S) {   // vectors and scales, before the table changes to fixed point
+            unsigned mx0 = 0, mx1 = 0;   // high words of the largest |sqrt(w) u|, |sqrt(w) du|
             for (uint64_t bits = fmask[tid]; bits; bits &= bits - 1) {
                 const int p = __ffsll((long long)bits) - 1;
                 const double sw = qsw[p], u = sw * tabu[p * S + tid];
@@ -797,24 +786,28 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
                     vq0 += u;
                     vqx += sw * d.x;
                     vqy += sw * d.y;
+                    mx0 = max(mx0, abs_hiword(tabu[p * S + tid]));
+                    mx1 = max(mx1, max(abs_hiword(d.x), abs_hiword(d.y)));
                 } else if (qfs[p] == 0) {
                     vb0 += u;
                 } else {
                     vb1 += u;
                 }
             }
+            xu[tid] = (int16_t)top_exp(mx0);
+            xd[tid] = (int16_t)top_exp(mx1);
+        }
         // 3. fixed point, in place
-        const int x0 = top_exp(top[0]), x1 = top_exp(top[1]);
         int2 *iu = reinterpret_cast<int2 *>(tabu);
         int4 *id = reinterpret_cast<int4 *>(tabd);
         if (vol) {
             __syncthreads();
-            const double sc0 = ldexp(1.0, 54 - x0), sc1 = ldexp(1.0, 54 - x1);   // 64 products of 2^108 fit 64 bits
             for (int k = tid; k < P * S; k += kLinThreads) {
                 const int p = k / S, a = k - p * S;
                 if (!((fmask[a] >> p) & 1)) continue;   // zero already
                 const double u = tabu[k];
                 const double2 d = tabd[k];
+                const double sc0 = pow2(54 - xu[a]), sc1 = pow2(54 - xd[a]);   // 64 products of 2^108 fit 64 bits
                 iu[k] = fixed_parts(u, sc0);
                 const int2 ix = fixed_parts(d.x, sc1), iy = fixed_parts(d.y, sc1);
                 id[k] = make_int4(ix.x, ix.y, iy.x, iy.y);
@@ -822,7 +815,6 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
             __syncthreads();
         }
         // 4. pairs.  value = 2^(e_a + e_b) 2^-108 (A 2^56 + B 2^28) = 2^(e_a + e_b - 56) (16 A + B / 2^24)
-        const double f00 = ldexp(1.0, 2 * x0 - 56), f01 = ldexp(1.0, x0 + x1 - 56), f11 = ldexp(1.0, 2 * x1 - 56);
         for (int pb = warp * 32; pb < nP; pb += kLinThreads) {   // whole warps: the reductions name every lane
             const int pr = pb + lane;
             int a = 0, b = 0;
@@ -876,9 +868,12 @@ __global__ void __launch_bounds__(kLinThreads, 4) k_assemble_2d_lin(AsmArgs A, d
             }
             if (pos < 0) continue;
             double v[9];
+            const double f00 = pow2(xu[a] + xu[b] - 56), f01 = pow2(xu[a] + xd[b] - 56), f10 = pow2(xd[a] + xu[b] - 56),
+                         f11 = pow2(xd[a] + xd[b] - 56);
 #pragma unroll
             for (int k = 0; k < 9; ++k)
-                v[k] = (double)(hh[k] * 16 + (hl[k] >> 24)) * (k == 0 ? f00 : (k < 3 || k % 3 == 0 ? f01 : f11));
+                v[k] = (double)(hh[k] * 16 + ((hl[k] + (1 << 23)) >> 24)) *
+                       (k == 0 ? f00 : (k < 3 ? f01 : (k % 3 == 0 ? f10 : f11)));
             atomicAdd(&A.mats[pos], v[0]);
             atomicAdd(&A.mats[nnz + pos], st * v[0]);
             atomicAdd(&A.mats[2 * nnz + pos], ss * v[0]);

@@ -425,11 +425,11 @@ __global__ void __launch_bounds__(kThreads3) k_assemble_3d(Asm3Args A) {
 //      list of functions; the derivative moments are the third-order moments of
 //      the kernel's radial derivative (19 sums instead of 30), M's Cholesky factor
 //      once per point;
-//   3. the table sqrt(w) (U, dU) is turned into fixed point, 56 bits below the
-//      group's largest U and dU, as two signed 28-bit parts;
+//   3. the table sqrt(w) (U, dU) is turned into fixed point, 55 bits below each
+//      function's largest U and dU in the group, as two signed 28-bit parts;
 //   4. every unordered pair a <= b sums the 16 products (u, u_x, u_y, u_z)_a x (u,
 //      u_x, u_y, u_z)_b over the group's points in 64-bit integers, exactly but for
-//      the products of two low parts (2^-56 of the largest product each);
+//      the products of two low parts (2^-56 of the two functions' largest each);
 //   5. the sums are added to the pattern's upper entries (FP64 atomics), the forms
 //      G(b, a) to three buffers of their own; k_mirror_3d fills the lower entries
 //      (M0 and K are each other's transposes) and applies the trial volumes V_b.
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(kThreads3) k_assemble_3d(Asm3Args A) {
 // tetrahedron the old kernel spent about 350k clocks (pairs twice, 17 operations each;
 // 40 warp sums of FP64 values and a Cholesky factor in all 32 lanes per point; 33k
 // atomics); now the RK functions bound it.
-// Accuracy: fixed point 2^-55 below the largest value in place of FP64's relative
-// 2^-53 per product and per sum.
+// Accuracy: fixed point 2^-55 below the function's largest value in the group in place of
+// FP64's relative 2^-53 per product and per sum.
 // Measured: the kernel at 15^3 (267,000 tetrahedra) 296 -> 51 ms.
 // A group with more functions than the table holds goes to k_assemble_3d, element by
 // element.
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
     __shared__ uint64_t fmask[kMaxS3];                 // points at which a function is supported
     __shared__ uint8_t plist[kGrpPts][kMaxS3];         // functions of each point
     __shared__ int pcnt[kGrpPts], wcnt[kGrpThreads / 32];
-    __shared__ unsigned top[2];
+    __shared__ int16_t xu[kMaxS3], xd[kMaxS3];         // exponents of each function's largest values
     __shared__ int S_sh, over;
     extern __shared__ __align__(16) unsigned char smem_tab[];
     double2 *tab = reinterpret_cast<double2 *>(smem_tab);   // [point][2][S]: (u, u_x), (u_y, u_z)
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
     const int nt = gr.y, P = 8 * nt;
     const int32_t o = A.owner[e0];
     const double *g = A.x + 3 * (int64_t)o;
-    if (tid == 0) { S_sh = 0; over = 0; top[0] = top[1] = 0; }
+    if (tid == 0) { S_sh = 0; over = 0; }
     if (tid < P) {
         const double *v = A.ev + 9 * (e0 + (tid >> 3));
         const int q = tid & 7;
@@ -607,7 +607,6 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
     __syncthreads();
     // 2. RK functions: four lanes per point
     const double s = 0.5 * A.R[o], is = 1.0 / s;
-    unsigned mx0 = 0, mx1 = 0;   // high words of the largest |sqrt(w) u|, |sqrt(w) du|
     for (int p0 = warp * 8; p0 < P; p0 += kGrpThreads / 4) {   // 8 points per warp (P is a multiple of 8)
         const int p = p0 + (lane >> 2), l4 = lane & 3, cnt = pcnt[p];
         const double px = qx[3 * p], py = qx[3 * p + 1], pz = qx[3 * p + 2];
@@ -721,25 +720,17 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
             if (ok) {
                 tp[a] = make_double2(u, ud[0]);
                 tp[S + a] = make_double2(ud[1], ud[2]);
-                mx0 = max(mx0, (unsigned)__double2hiint(u) & 0x7fffffffu);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) mx1 = max(mx1, (unsigned)__double2hiint(ud[c]) & 0x7fffffffu);
             } else {
                 tp[a] = make_double2(0.0, 0.0);
             }
         }
     }
-    mx0 = __reduce_max_sync(0xffffffffu, mx0);
-    mx1 = __reduce_max_sync(0xffffffffu, mx1);
-    if (lane == 0) {
-        atomicMax(&top[0], mx0);
-        atomicMax(&top[1], mx1);
-    }
     __syncthreads();
     const double st = A.sig_t[o], ss = A.sig_s[o];
     const int64_t nnz = A.nnz, n = A.n;
-    // vectors: Q0, Q (before the table changes to fixed point)
+    // vectors Q0, Q and the scales (before the table changes to fixed point)
     if (tid < S) {
+        unsigned mx0 = 0, mx1 = 0;   // high words of the largest |sqrt(w) u|, |sqrt(w) du|
         const double qv = A.q[o];
         double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
         for (uint64_t bits = fmask[tid]; bits; bits &= bits - 1) {
@@ -750,7 +741,11 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
             v1 += sw * u.y;
             v2 += sw * w.x;
             v3 += sw * w.y;
+            mx0 = max(mx0, abs_hiword(u.x));
+            mx1 = max(mx1, max(abs_hiword(u.y), max(abs_hiword(w.x), abs_hiword(w.y))));
         }
+        xu[tid] = (int16_t)top_exp(mx0);
+        xd[tid] = (int16_t)top_exp(mx1);
         const int32_t i = fidx[tid];
         if (v0 != 0.0) atomicAdd(&A.vecs[i], qv * v0);
         if (v1 != 0.0) atomicAdd(&A.vecs[n + i], qv * v1);
@@ -759,21 +754,19 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
     }
     __syncthreads();
     // 3. fixed point, in place: (hi, lo) of u, u_x | u_y, u_z
-    const int x0 = top_exp(top[0]), x1 = top_exp(top[1]);
-    const double sc0 = ldexp(1.0, 55 - x0), sc1 = ldexp(1.0, 55 - x1);   // 48 products of 2^110 fit 64 bits
     int4 *itab = reinterpret_cast<int4 *>(smem_tab);
     for (int k = tid; k < P * S; k += kGrpThreads) {
         const int p = k / S, a = k - p * S;
         if (!((fmask[a] >> p) & 1)) continue;   // zero already
         const int at = p * 2 * S + a;
         const double2 u = tab[at], w = tab[at + S];
+        const double sc0 = pow2(55 - xu[a]), sc1 = pow2(55 - xd[a]);   // 48 products of 2^110 fit 64 bits
         const int2 i0 = fixed_parts(u.x, sc0), i1 = fixed_parts(u.y, sc1), i2 = fixed_parts(w.x, sc1), i3 = fixed_parts(w.y, sc1);
         itab[at] = make_int4(i0.x, i0.y, i1.x, i1.y);
         itab[at + S] = make_int4(i2.x, i2.y, i3.x, i3.y);
     }
     __syncthreads();
     // 4. pairs.  value = 2^(e_a + e_b) 2^-110 (A 2^56 + B 2^28) = 2^(e_a + e_b - 57) (8 A + B / 2^25)
-    const double f00 = ldexp(1.0, 2 * x0 - 57), f01 = ldexp(1.0, x0 + x1 - 57), f11 = ldexp(1.0, 2 * x1 - 57);
     const int nP = S * (S + 1) / 2;
     for (int base = warp * 32; base < nP; base += kGrpThreads) {   // whole warps: the reductions name every lane
         const int pr = base + lane;
@@ -813,9 +806,12 @@ __global__ void __launch_bounds__(kGrpThreads, 2) k_assemble_3d_grp(Asm3Args A, 
         const int pos = find_col3(A.col, A.rowptr[fidx[a]], A.rowptr[fidx[a] + 1], fidx[b]);
         if (pos < 0) { atomicOr(A.flag, 8); continue; }
         double v[16];
+        const double f00 = pow2(xu[a] + xu[b] - 57), f01 = pow2(xu[a] + xd[b] - 57), f10 = pow2(xd[a] + xu[b] - 57),
+                     f11 = pow2(xd[a] + xd[b] - 57);
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-            v[k] = (double)(hh[k] * 8 + (hl[k] >> 25)) * (k == 0 ? f00 : (k < 4 || (k & 3) == 0 ? f01 : f11));
+            v[k] = (double)(hh[k] * 8 + ((hl[k] + (1 << 24)) >> 25)) *
+                   (k == 0 ? f00 : (k < 4 ? f01 : ((k & 3) == 0 ? f10 : f11)));
         atomicAdd(&A.mats[pos], v[0]);
         atomicAdd(&A.mats[nnz + pos], st * v[0]);
         atomicAdd(&A.mats[2 * nnz + pos], ss * v[0]);

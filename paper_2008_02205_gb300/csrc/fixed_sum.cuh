@@ -1,7 +1,8 @@
 // Sums of products in fixed point, for the pair sums of the integration: the FP64
 // units do 1.6 operations per clock and SM, the integer multiplier some 30 wide
 // products, and three of those (high x high, and the two mixed ones) stand for one
-// FP64 multiply-add.
+// FP64 multiply-add.  Each function has its own scale, so that a pair's error is 2^-53 of the two
+// functions' own largest values, whatever other functions share their points.
 #pragma once
 
 #include <stdint.h>
@@ -19,8 +20,14 @@ __device__ __forceinline__ int2 fixed_parts(double v, double scale) {
     const int lo = (int)((unsigned)x << 4) >> 4;
     return make_int2((int)((x - lo) >> 28), lo);
 }
-// e with |v| < 2^e for every value, from the largest high word (sign bit off); 0 for all zeros
-__device__ __forceinline__ int top_exp(unsigned hiword) { return hiword ? (int)(hiword >> 20) - 1022 : 0; }
+// e with |v| < 2^e for every value, from the largest high word (sign bit off); 0 for all zeros.  At least
+// -900, so that the scale 2^(bits - e) is finite.
+__device__ __forceinline__ int top_exp(unsigned hiword) { return hiword ? max((int)(hiword >> 20) - 1022, -900) : 0; }
+__device__ __forceinline__ unsigned abs_hiword(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __noinline__ double pow2_subnormal(int k) { return ldexp(1.0, k); }
+__device__ __forceinline__ double pow2(int k) {
+    return (unsigned)(k + 1022) < 2046u ? __hiloint2double((k + 1023) << 20, 0) : pow2_subnormal(k);
+}
 
 }  // namespace
 }  // namespace mlpg
