@@ -1065,25 +1065,16 @@ mlpg_status run_assemble(mlpg_ctx *ctx) {
     } else if (ctx->opt.rk_order == 2) {
         MLPG_TRY(run(k_assemble_2d<2, 48, 32>, 48, 32));
     } else {
-        struct Scratch {   // G of the lower entries, freed on every return (cudaFree waits for the device)
-            double *p = nullptr;
-            ~Scratch() {
-                if (p) cudaFree(p);
-            }
-        } gt;
-        if (cudaMalloc(&gt.p, sizeof(double) * 6 * std::max<int64_t>(ctx->nnz, 1)) != cudaSuccess) {
-            cudaGetLastError();
-            gt.p = nullptr;
-            return set_err(ctx, MLPG_ERR_OOM, "cudaMalloc failed: assembly buffers");
-        }
-        CU(ctx, cudaMemsetAsync(gt.p, 0, sizeof(double) * 6 * ctx->nnz, ctx->stream));
+        double *gt = nullptr;   // G of the lower entries
+        MLPG_TRY(assembly_scratch(ctx, &gt));
+        CU(ctx, cudaMemsetAsync(gt, 0, sizeof(double) * 6 * ctx->nnz, ctx->stream));
         // u and (u_x, u_y) of kLinEntries entries, the first rounded to a 16-byte boundary
         const size_t smem = sizeof(double) * (3 * (size_t)kLinEntries + 2);
         CU(ctx, cudaFuncSetAttribute(k_assemble_2d_lin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_assemble_2d_lin<<<(unsigned)ctx->n, kLinThreads, smem, ctx->stream>>>(a, gt.p);
+        k_assemble_2d_lin<<<(unsigned)ctx->n, kLinThreads, smem, ctx->stream>>>(a, gt);
         CU_LAUNCH(ctx);
         k_mirror_2d<<<(unsigned)((ctx->n * 8 + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->nnz, ctx->rowptr, ctx->col,
-                                                                                   ctx->V, gt.p, ctx->mats, ctx->d_flag);
+                                                                                   ctx->V, gt, ctx->mats, ctx->d_flag);
         CU_LAUNCH(ctx);
         return check_flag(ctx, "assembly");
     }

@@ -925,23 +925,6 @@ __global__ void __launch_bounds__(128) k_interp_3d(int64_t n, const double *__re
 
 }  // namespace
 
-// device scratch of one call, freed when it goes out of scope (the caller has synchronised its stream,
-// or an error ends the call: cudaFree waits for the device)
-template <typename T>
-struct ScratchBuf {
-    T *p = nullptr;
-    mlpg_status get(mlpg_ctx *ctx, size_t count) {
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&p), std::max<size_t>(count, 1) * sizeof(T));
-        if (e == cudaSuccess) return MLPG_OK;
-        cudaGetLastError();
-        p = nullptr;
-        return set_err(ctx, MLPG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
-    }
-    ~ScratchBuf() {
-        if (p) cudaFree(p);
-    }
-};
-
 static mlpg_status check_flag3(mlpg_ctx *ctx, const char *stage) {
     int flag = 0;
     CU(ctx, cudaMemcpyAsync(&flag, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1000,42 +983,41 @@ mlpg_status run_assemble_3d(mlpg_ctx *ctx) {
     cudaStream_t s = ctx->stream;
     size_t smem = sizeof(double) * (size_t)a.nq * 4 * kMaxS3;
     if (a.nelem > 0) {
-        // scratch of this call: group list, list of skipped elements, two counters, G of the lower entries
-        ScratchBuf<int2> grp;
-        ScratchBuf<int32_t> skip;
-        ScratchBuf<int> cnt;
-        ScratchBuf<double> gt;
-        MLPG_TRY(grp.get(ctx, a.nelem));
-        MLPG_TRY(skip.get(ctx, a.nelem));
-        MLPG_TRY(cnt.get(ctx, 2));
-        MLPG_TRY(gt.get(ctx, 9 * ctx->nnz));
-        CU(ctx, cudaMemsetAsync(cnt.p, 0, 2 * sizeof(int), s));
-        CU(ctx, cudaMemsetAsync(gt.p, 0, sizeof(double) * 9 * ctx->nnz, s));
-        k_tet_groups<<<(unsigned)((a.nelem + 127) / 128), 128, 0, s>>>(a.nelem, a.owner, a.ev, grp.p, cnt.p);
+        // group list, list of skipped elements, two counters; G of the lower entries
+        int2 *grp = nullptr;
+        int32_t *skip = nullptr;
+        int *cnt = nullptr;
+        double *gt = nullptr;
+        MLPG_TRY(dalloc(ctx, &grp, a.nelem));
+        MLPG_TRY(dalloc(ctx, &skip, a.nelem));
+        MLPG_TRY(dalloc(ctx, &cnt, 2));
+        MLPG_TRY(assembly_scratch(ctx, &gt));
+        CU(ctx, cudaMemsetAsync(cnt, 0, 2 * sizeof(int), s));
+        CU(ctx, cudaMemsetAsync(gt, 0, sizeof(double) * 9 * ctx->nnz, s));
+        k_tet_groups<<<(unsigned)((a.nelem + 127) / 128), 128, 0, s>>>(a.nelem, a.owner, a.ev, grp, cnt);
         CU_LAUNCH(ctx);
         int ngrp = 0, nskip = 0;
-        CU(ctx, cudaMemcpyAsync(&ngrp, cnt.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CU(ctx, cudaMemcpyAsync(&ngrp, cnt, sizeof(int), cudaMemcpyDeviceToHost, s));
         CU(ctx, cudaStreamSynchronize(s));
         const int gsmem = kGrpEntries * 32;
         if (ctx->opt.rk_order == 0) {
             CU(ctx, cudaFuncSetAttribute(k_assemble_3d_grp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, gsmem));
-            k_assemble_3d_grp<1><<<(unsigned)ngrp, kGrpThreads, gsmem, s>>>(a, grp.p, gt.p, cnt.p + 1, skip.p);
+            k_assemble_3d_grp<1><<<(unsigned)ngrp, kGrpThreads, gsmem, s>>>(a, grp, gt, cnt + 1, skip);
         } else {
             CU(ctx, cudaFuncSetAttribute(k_assemble_3d_grp<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, gsmem));
-            k_assemble_3d_grp<4><<<(unsigned)ngrp, kGrpThreads, gsmem, s>>>(a, grp.p, gt.p, cnt.p + 1, skip.p);
+            k_assemble_3d_grp<4><<<(unsigned)ngrp, kGrpThreads, gsmem, s>>>(a, grp, gt, cnt + 1, skip);
         }
         CU_LAUNCH(ctx);
         k_mirror_3d<<<(unsigned)((ctx->n * 32 + 255) / 256), 256, 0, s>>>(ctx->n, ctx->nnz, ctx->rowptr, ctx->col, ctx->V,
-                                                                        gt.p, ctx->mats, ctx->d_flag);
+                                                                        gt, ctx->mats, ctx->d_flag);
         CU_LAUNCH(ctx);
-        CU(ctx, cudaMemcpyAsync(&nskip, cnt.p + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CU(ctx, cudaMemcpyAsync(&nskip, cnt + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
         CU(ctx, cudaStreamSynchronize(s));
         if (nskip > 0) {
-            a.list = skip.p;
+            a.list = skip;
             if (ctx->opt.rk_order == 0) k_assemble_3d<false, 1><<<(unsigned)nskip, kThreads3, smem, s>>>(a);
             else k_assemble_3d<false, 4><<<(unsigned)nskip, kThreads3, smem, s>>>(a);
             CU_LAUNCH(ctx);
-            CU(ctx, cudaStreamSynchronize(s));   // the list is freed below
             a.list = nullptr;
         }
     }

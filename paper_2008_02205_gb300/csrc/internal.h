@@ -167,7 +167,8 @@ struct mlpg_ctx {
 
     // operators for the current 1/(c dt)
     double kappa = -1.0;
-    double *A64 = nullptr;      // [6][nnz] direction-independent LHS arrays
+    double *A64 = nullptr;      // [6 or 10][nnz] direction-independent LHS arrays; the assembly's scratch before
+    bool ops_ready = false;     // the operator arrays are allocated
     double *L64 = nullptr;      // [nnz][m] materialised per-direction L_m (FP64 path)
     float *A32 = nullptr;       // [6][nnz]
     int64_t nb = 0;             // boundary-segment entries
@@ -280,6 +281,9 @@ mlpg_status run_assemble(mlpg_ctx *ctx);
 mlpg_status run_interp_3d(mlpg_ctx *ctx);
 mlpg_status run_assemble_3d(mlpg_ctx *ctx);
 mlpg_status form_operators(mlpg_ctx *ctx, double kappa);
+// nnz-long FP64 arrays for the assembly, 6 in 2D and 10 in 3D: the place of the operators' A64, so that a
+// problem's peak and its device_bytes hold no more for them and nothing is freed (which waits for the device)
+mlpg_status assembly_scratch(mlpg_ctx *ctx, double **p);
 mlpg_status apply_L64(mlpg_ctx *ctx, const double *X, double *Y);
 mlpg_status apply_L32(mlpg_ctx *ctx, const float *X, float *Y);
 mlpg_status step_fp64(mlpg_ctx *ctx, double dt);

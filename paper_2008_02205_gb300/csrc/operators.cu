@@ -1963,7 +1963,7 @@ static mlpg_status init_operator_storage_d(mlpg_ctx *ctx) {
     MLPG_TRY(dalloc(ctx, &ctx->rowidx, nnz));
     k_rowidx<<<(n + 255) / 256, 256, 0, s>>>(n, ctx->rowptr, ctx->rowidx);
     CU_LAUNCH(ctx);
-    MLPG_TRY(dalloc(ctx, &ctx->A64, NA<D>() * nnz));
+    if (!ctx->A64) MLPG_TRY(dalloc(ctx, &ctx->A64, NA<D>() * nnz));
     MLPG_TRY(dalloc(ctx, &ctx->A32, NA<D>() * nnz));
     MLPG_TRY(dalloc(ctx, &ctx->T64, NT<D>() * nnz));
     MLPG_TRY(dalloc(ctx, &ctx->S64, NT<D>() * nnz));
@@ -2017,6 +2017,12 @@ static mlpg_status init_operator_storage_d(mlpg_ctx *ctx) {
     return MLPG_OK;
 }
 
+mlpg_status assembly_scratch(mlpg_ctx *ctx, double **p) {
+    if (!ctx->A64) MLPG_TRY(dalloc(ctx, &ctx->A64, (ctx->dim == 3 ? NA<3>() : NA<2>()) * ctx->nnz));
+    *p = ctx->A64;
+    return MLPG_OK;
+}
+
 static mlpg_status init_operator_storage(mlpg_ctx *ctx) {
     return ctx->dim == 3 ? init_operator_storage_d<3>(ctx) : init_operator_storage_d<2>(ctx);
 }
@@ -2026,7 +2032,10 @@ static mlpg_status form_operators_d(mlpg_ctx *ctx, double kappa) {
     const int64_t n = ctx->n, nnz = ctx->nnz;
     const int m = ctx->m;
     cudaStream_t s = ctx->stream;
-    if (!ctx->A64) MLPG_TRY(init_operator_storage(ctx));
+    if (!ctx->ops_ready) {
+        MLPG_TRY(init_operator_storage(ctx));
+        ctx->ops_ready = true;
+    }
     const double *Sf = ctx->mats + mat_S<D>() * nnz;
     k_form_arrays<D><<<(nnz + 255) / 256, 256, 0, s>>>(nnz, kappa, ctx->rowidx, ctx->tau, ctx->mats,
                                                     ctx->A64, ctx->A32, ctx->T64, ctx->S64);
