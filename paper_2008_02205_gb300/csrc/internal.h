@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <utility>
 #include <vector>
@@ -124,6 +125,7 @@ struct Gmres {
     T *Zf = nullptr;           // R * n * M: preconditioned basis vectors (flexible GMRES), or null
 };
 
+struct TilePlan;   // operators.cu
 }  // namespace mlpg
 
 struct mlpg_ctx {
@@ -215,7 +217,7 @@ struct mlpg_ctx {
     int64_t nblk = 0;
     int32_t *bmember = nullptr; // [nblk * kBlockPts] point of each block slot (-1: empty)
     int32_t *bof = nullptr;     // [n] block * kBlockPts + slot of each point
-    std::vector<int32_t> h_order;  // [n] points in the spatial order of the row tiles (host)
+    std::shared_ptr<const mlpg::TilePlan> tile_plan;  // host plan of the row tiles, from the assembly to the first apply
 
     // row tiles of the FP32 L-apply (tiles.cpp)
     int tile_rows = 0, tile_chunk = 0, tile_dpt = 0, tile_xs = 0;  // rows per tile, directions per CTA, per thread, smem row stride
@@ -284,6 +286,8 @@ mlpg_status form_operators(mlpg_ctx *ctx, double kappa);
 // nnz-long FP64 arrays for the assembly, 6 in 2D and 10 in 3D: the place of the operators' A64, so that a
 // problem's peak and its device_bytes hold no more for them and nothing is freed (which waits for the device)
 mlpg_status assembly_scratch(mlpg_ctx *ctx, double **p);
+// the row tiles of the FP32 apply (host work; reads only what integrate left on the host)
+std::shared_ptr<const TilePlan> plan_tiles(const mlpg_ctx *ctx);
 mlpg_status apply_L64(mlpg_ctx *ctx, const double *X, double *Y);
 mlpg_status apply_L32(mlpg_ctx *ctx, const float *X, float *Y);
 mlpg_status step_fp64(mlpg_ctx *ctx, double dt);

@@ -19,6 +19,8 @@
 // per boundary row.
 #include <algorithm>
 #include <cmath>
+#include <memory>
+#include <string>
 #include <type_traits>
 
 #include <cuda_fp16.h>
@@ -1755,8 +1757,9 @@ static mlpg_status pair_attr(mlpg_ctx *ctx) {
 
 // One tile layout: rows per tile, directions per thread and per CTA (chunk),
 // staged halo or gather mode, the host-side tiles (row pairs, or single rows for
-// the tensor cores).  chunk == 0: no layout.
+// the tensor cores).  chunk == 0: no layout.  err: an explicit request that cannot be met.
 struct TilePlan {
+    std::string err;
     int tr = 0, dpt = 0, chunk = 0, ks = 1;
     bool gather = false, mma = false;
     size_t rec_smem = 0;
@@ -1766,18 +1769,20 @@ struct TilePlan {
 };
 
 // Plans the tiles of one mode; an explicit request that cannot be met is an
-// error, the automatic choice only finds no layout (chunk 0).
+// error, the automatic choice only finds no layout (chunk 0).  Reads the points, the pattern and the
+// options only: it runs beside the assembly.
 template <int D>
-static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P) {
+static void plan_mode(const mlpg_ctx *ctx, const std::vector<int32_t> &order, bool gather, bool mma, TilePlan &P) {
     const int m = ctx->m;
     const bool ask = ctx->opt.apply_kernel != 0;
     P = TilePlan();
+    auto refuse = [&P](const char *why) { P.err = why; };
     P.gather = gather;
     P.mma = mma;
     // m no multiple of four: staged value by value.  The automatic choice takes four directions per thread:
     // eight measured slower at every size (256^2 S8: 69.3 against 60.8 us; more registers, fewer warps)
     const int dpt = (m & 3) != 0 ? 4 : (ctx->opt.tile_dpt ? ctx->opt.tile_dpt : ((m & 7) == 0 && !gather && (ask || mma) ? 8 : 4));
-    if ((m & 3) == 0 && m % dpt != 0) return set_err(ctx, MLPG_ERR_ARG, "tile_dpt must divide the number of directions");
+    if ((m & 3) == 0 && m % dpt != 0) return refuse("tile_dpt must divide the number of directions");
     int tr = ctx->opt.tile_rows;
     if (tr == 0 && !ask) {
         // gather: the most rows per tile (X rows shared through the L1) that keep a CTA at or below
@@ -1798,31 +1803,31 @@ static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P)
     }
     if (tr == 0) tr = 64;
     if (gather && tr == 64)
-        return ask ? set_err(ctx, MLPG_ERR_ARG, "apply_kernel 4 takes 4, 8, 16 or 32 rows per tile") : MLPG_OK;
+        return ask ? refuse("apply_kernel 4 takes 4, 8, 16 or 32 rows per tile") : void();
     if (gather && (int64_t)ctx->n * m >= (int64_t(1) << 31))
-        return ask ? set_err(ctx, MLPG_ERR_ARG, "apply_kernel 4 needs n x m < 2^31 (32-bit record offsets)") : MLPG_OK;
+        return ask ? refuse("apply_kernel 4 needs n x m < 2^31 (32-bit record offsets)") : void();
     if (mma) {
-        P.nslot = build_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), ctx->h_order.data(), tr, kRecK, P.tl);
+        P.nslot = build_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), order.data(), tr, kRecK, P.tl);
         P.max_halo = P.tl.max_halo;
         if (P.nslot * (int64_t)(rec_words<D>() / 4) >= (int64_t(1) << 31) || P.tl.hptr.back() >= (int64_t(1) << 31))
-            return MLPG_OK;   // beyond 32-bit slot indices: the row-team kernel serves
+            return;   // beyond 32-bit slot indices: the row-team kernel serves
         P.rec_smem = (size_t)kRecStages * kRecK * tr * (rec_words<D>() / 4) * sizeof(float4);
     } else {
-        P.nslot = build_pair_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), ctx->h_order.data(), tr, 4, !gather,
+        P.nslot = build_pair_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), order.data(), tr, 4, !gather,
                                    P.pl);
         P.max_halo = P.pl.max_halo;
-        if (P.nslot >= (int64_t(1) << 31) || P.pl.hptr.back() >= (int64_t(1) << 31)) return MLPG_OK;
+        if (P.nslot >= (int64_t(1) << 31) || P.pl.hptr.back() >= (int64_t(1) << 31)) return;
     }
     int chunk = 0;
     if (mma) {
         // tensor-core tiles: chunks of 8 NT directions (NT <= 6) dividing m; shared-memory row stride
         // 16 mod 32 words (two rows read by one 8-lane phase then fall on disjoint banks half the time)
-        if ((m & 7) != 0) return set_err(ctx, MLPG_ERR_ARG, "apply_kernel 3 needs a multiple of 8 directions");
+        if ((m & 7) != 0) return refuse("apply_kernel 3 needs a multiple of 8 directions");
         for (int nt = 6; nt >= 2 && !chunk; --nt) {
             const int mc = 8 * nt, xs = mc + (16 - mc % 32 + 32) % 32;
             if (m % mc == 0 && (size_t)P.max_halo * xs * sizeof(float) + P.rec_smem <= kTileSmem) chunk = mc;
         }
-        if (!chunk) return set_err(ctx, MLPG_ERR_ARG, "apply_kernel 3: no direction chunk fits shared memory");
+        if (!chunk) return refuse("apply_kernel 3: no direction chunk fits shared memory");
     }
     for (int nchunk = 1; nchunk <= (m + 3) / 4 && !mma; ++nchunk) {
         const int G = (m + dpt * nchunk - 1) / (dpt * nchunk);
@@ -1840,7 +1845,34 @@ static mlpg_status plan_tiles(mlpg_ctx *ctx, bool gather, bool mma, TilePlan &P)
     P.tr = tr;
     P.dpt = dpt;
     P.chunk = chunk;
-    return MLPG_OK;
+}
+
+template <int D>
+static void plan_apply(const mlpg_ctx *ctx, TilePlan &P) {
+    const int m = ctx->m, kind = ctx->opt.apply_kernel;
+    std::vector<int32_t> order(ctx->n);
+    spatial_order(ctx->n, D, ctx->h_x.data(), order.data());
+    // automatic choice: 3D halos (some 700 rows for 32) leave room for few directions per chunk, and
+    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit.  A
+    // request for 64 rows, which gather mode does not take, still goes to the staged tiles.
+    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->opt.tile_rows != 64 && ctx->n * m < (int64_t(1) << 31);
+    if (kind != 4 && !skip) {
+        plan_mode<D>(ctx, order, false, kind == 3, P);
+        if (!P.err.empty()) return;
+        // staged halos pay while the records are read by few chunks; past two chunks the gather
+        // mode reads them once
+        if (kind == 0 && P.chunk && (m + P.chunk - 1) / P.chunk > 2) P.chunk = 0;
+    }
+    if (kind == 4 || (kind == 0 && P.chunk == 0 && (m & 3) == 0)) plan_mode<D>(ctx, order, true, false, P);
+}
+
+std::shared_ptr<const TilePlan> plan_tiles(const mlpg_ctx *ctx) {
+    auto P = std::make_shared<TilePlan>();
+    if (ctx->opt.precision == MLPG_MIXED && ctx->opt.apply_kernel != 1) {
+        if (ctx->dim == 3) plan_apply<3>(ctx, *P);
+        else plan_apply<2>(ctx, *P);
+    }
+    return P;
 }
 
 template <typename T>
@@ -1852,22 +1884,9 @@ static mlpg_status to_device(mlpg_ctx *ctx, T **d, const std::vector<T> &h) {
 
 template <int D>
 static mlpg_status init_tiles(mlpg_ctx *ctx) {
-    const int m = ctx->m, kind = ctx->opt.apply_kernel;
-    if (kind == 1) return MLPG_OK;
-    ctx->h_order.resize(ctx->n);
-    spatial_order(ctx->n, D, ctx->h_x.data(), ctx->h_order.data());
-    TilePlan P;
-    // automatic choice: 3D halos (some 700 rows for 32) leave room for few directions per chunk, and
-    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit.  A
-    // request for 64 rows, which gather mode does not take, still goes to the staged tiles.
-    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->opt.tile_rows != 64 && ctx->n * m < (int64_t(1) << 31);
-    if (kind != 4 && !skip) {
-        MLPG_TRY(plan_tiles<D>(ctx, false, kind == 3, P));
-        // staged halos pay while the records are read by few chunks; past two chunks the gather
-        // mode reads them once
-        if (kind == 0 && P.chunk && (m + P.chunk - 1) / P.chunk > 2) P.chunk = 0;
-    }
-    if (kind == 4 || (kind == 0 && P.chunk == 0 && (m & 3) == 0)) MLPG_TRY(plan_tiles<D>(ctx, true, false, P));
+    const int m = ctx->m;
+    const std::shared_ptr<const TilePlan> plan = std::move(ctx->tile_plan);   // not needed after this
+    const TilePlan &P = *plan;
     if (P.chunk == 0) return MLPG_OK;
     const int tr = P.tr, chunk = P.chunk;
     const bool gather = P.gather, mma = P.mma;
@@ -2024,6 +2043,10 @@ mlpg_status assembly_scratch(mlpg_ctx *ctx, double **p) {
 }
 
 static mlpg_status init_operator_storage(mlpg_ctx *ctx) {
+    if (ctx->opt.precision == MLPG_MIXED) {   // planned beside the assembly, or now where no thread could be had
+        if (!ctx->tile_plan) ctx->tile_plan = plan_tiles(ctx);
+        if (!ctx->tile_plan->err.empty()) return set_err(ctx, MLPG_ERR_ARG, ctx->tile_plan->err);
+    }
     return ctx->dim == 3 ? init_operator_storage_d<3>(ctx) : init_operator_storage_d<2>(ctx);
 }
 

@@ -25,14 +25,16 @@ namespace mlpg {
 
 namespace {
 // threads for the per-tile passes: the host cores, fewer when their n-sized
-// scratch (12 bytes a point each) would pass 256 MB
-int tile_threads(int64_t n, int64_t ntile) {
+// scratch (12 bytes a point each) would pass 256 MB, and one per 64k pattern entries (some
+// 0.5 ms of work; starting and joining a thread takes 30 to 60 us on either pass)
+int tile_threads(int64_t n, int64_t ntile, int64_t entries) {
     int64_t T = std::max(1u, std::thread::hardware_concurrency());
     T = std::min<int64_t>(T, std::max<int64_t>(1, (int64_t(256) << 20) / std::max<int64_t>(1, 12 * n)));
+    T = std::min<int64_t>(T, entries >> 16);
     return (int)std::max<int64_t>(1, std::min<int64_t>(T, ntile / 8));
 }
-// f(first tile, end tile, worker) over T workers; an exception thrown by a worker (an
-// allocation that fails) is rethrown here, on the calling thread, after every worker ended
+// f(first tile, end tile, worker) over T workers, the calling thread among them; an exception thrown by a
+// worker (an allocation that fails) is rethrown here, on the calling thread, after every worker ended
 template <typename F>
 void over_tiles(int64_t ntile, int T, F &&f) {
     if (T <= 1) {
@@ -41,14 +43,21 @@ void over_tiles(int64_t ntile, int T, F &&f) {
     }
     std::vector<std::exception_ptr> errs(T);
     std::vector<std::thread> th;
-    for (int w = 0; w < T; ++w)
-        th.emplace_back([&, w]() {
-            try {
-                f(ntile * w / T, ntile * (w + 1) / T, w);
-            } catch (...) {
-                errs[w] = std::current_exception();
-            }
-        });
+    th.reserve(T - 1);
+    auto work = [&](int w) {
+        try {
+            f(ntile * w / T, ntile * (w + 1) / T, w);
+        } catch (...) {
+            errs[w] = std::current_exception();
+        }
+    };
+    int started = 1;
+    try {
+        for (; started < T; ++started) th.emplace_back(work, started);
+    } catch (...) {   // no thread: the rest here
+    }
+    work(0);
+    for (int w = started; w < T; ++w) work(w);
     for (auto &x : th) x.join();
     for (auto &e : errs)
         if (e) std::rethrow_exception(e);
@@ -66,7 +75,7 @@ int64_t build_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, const 
     out.width.assign(ntile, 0);
     out.row.assign(ntile * TR, -1);
     out.hptr.assign(ntile + 1, 0);
-    const int T = tile_threads(n, ntile);
+    const int T = tile_threads(n, ntile, rowptr[n]);
     // 1. per tile: rows, width and halo.  The halo is collected with a stamp per column
     //    (stamp[c] == t: already in it), then sorted; linear in the pattern entries.
     std::vector<std::vector<int32_t>> halo(ntile);
@@ -144,7 +153,7 @@ int64_t build_pair_tiles(int64_t n, const int32_t *rowptr, const int32_t *col, c
     out.row.assign(ntile * TR, -1);
     out.plen.assign(ntile * TP, 0);
     out.hptr.assign(ntile + 1, 0);
-    const int T = tile_threads(n, ntile);
+    const int T = tile_threads(n, ntile, rowptr[n]);
     auto merge = [rowptr, col](int32_t i, int32_t j, auto &&f) {   // f(entry of i or -1, entry of j or -1, column)
         int32_t a = i >= 0 ? rowptr[i] : 0, b = j >= 0 ? rowptr[j] : 0;
         const int32_t ae = i >= 0 ? rowptr[i + 1] : 0, be = j >= 0 ? rowptr[j + 1] : 0;

@@ -117,3 +117,13 @@ def test_non_finite_values_stay_in_their_rows(dim, side, sn, m, kernel, value):
             # a sum taken again adds in another order: one row's rounding
             assert torch.isfinite(got[~hit]).all()
             assert _rel(got[~hit].numpy(), clean[~hit].numpy()) < 1e-6
+
+
+def test_a_refused_shape_stays_refused():
+    prob = _problem(2, 13, 4, 12)
+    with _open(prob, apply_kernel=2, tile_dpt=8) as tp:   # eight directions per thread do not divide twelve
+        X = torch.rand(prob.n, 12, device="cuda")
+        for _ in range(2):
+            with pytest.raises(pkg.MlpgError) as e:
+                _apply(tp, prob, X, torch.empty_like(X))
+            assert e.value.status == pkg.MLPG_ERR_ARG
