@@ -3,11 +3,15 @@
 The tiled L-apply (Sec. 4.2, operator L for all directions at once) has two
 shape parameters: rows per tile (32 or 64) and directions per thread (4 or 8,
 dividing m); its tensor-core variant (m % 8 == 0) has the rows per tile; the
-row-team kernel is the alternative for any m.  Which is
-fastest depends on the dimension (stencil size, halo) and on the number of
-directions m, so this module times every candidate on the problem's own
+row-team kernel is the alternative for any m.  The library's automatic choice
+fits the tiles to the problem's size and alone uses staged tiles of 8 and 16 rows
+and for an m that is no multiple of four.  Which is
+fastest depends on the dimension (stencil size, halo), on the number of
+directions m and on the size, so this module times the automatic choice and every
+explicit one on the problem's own
 operators (CUDA events on the library stream, inputs resident, after warm-up)
-and keeps the fastest per (dim, m) in a JSON cache:
+and keeps the fastest per (dim, m, size) in a JSON cache, with the version of the
+kernels that it timed:
 
     choice = tuned_options(prob)          # {"apply_kernel": ..., "tile_rows": ..., "tile_dpt": ...}
     TransportProblem.from_problem(prob, precision=MLPG_MIXED, **choice)
@@ -18,7 +22,9 @@ computes the operator.
 """
 from __future__ import annotations
 
+import hashlib
 import json
+import math
 import os
 import statistics
 
@@ -30,8 +36,23 @@ def cache_path() -> str:
                                                             "apply_tiles.json")
 
 
+AUTOMATIC = {"apply_kernel": 0, "tile_rows": 0, "tile_dpt": 0}
+
+
+def kernel_version() -> str:
+    """Changes with the apply's kernels and tile builders: times taken on others say nothing."""
+    h = hashlib.sha256()
+    for name in ("operators.cu", "tiles.cpp", "order.cpp"):
+        try:
+            with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", name), "rb") as f:
+                h.update(f.read())
+        except OSError:
+            h.update(name.encode())
+    return h.hexdigest()[:16]
+
+
 def candidates(m: int):
-    """Every apply configuration the library accepts for m directions."""
+    """Every explicit apply configuration the library accepts for m directions."""
     out = [{"apply_kernel": 1, "tile_rows": 0, "tile_dpt": 0}]
     if m % 8 == 0:
         for rows in (64, 32):
@@ -51,6 +72,10 @@ def _key(dim: int, m: int) -> str:
     return f"dim{dim}-m{m}"
 
 
+def _size_key(dim: int, m: int, n: int) -> str:
+    return f"{_key(dim, m)}-n{round(math.log2(n))}"   # points to the nearest power of two
+
+
 def load_cache() -> dict:
     try:
         with open(cache_path()) as f:
@@ -59,9 +84,9 @@ def load_cache() -> dict:
         return {}
 
 
-def _store(key: str, entry: dict) -> None:
+def _store(keys, entry: dict) -> None:
     c = load_cache()
-    c[key] = entry
+    c.update({k: entry for k in keys})
     path = cache_path()
     os.makedirs(os.path.dirname(path), exist_ok=True)
     tmp = path + f".{os.getpid()}.tmp"
@@ -98,7 +123,7 @@ def time_apply(prob, options: dict, reps: int = 20, warmup: int = 5, stream=None
 
 
 def tune(prob, reps: int = 20, warmup: int = 5, stream=None, store: bool = True, cands=None):
-    """Time every candidate on `prob`; returns (best options, table of
+    """Time every candidate on `prob` (default: the explicit ones); returns (best options, table of
     {config, us, apply_kernel used, chunk, max halo}).  A candidate the
     library turns down is skipped: a tile shape whose context falls back to
     the row-team kernel, or one the apply refuses with MLPG_ERR_ARG (no
@@ -117,16 +142,18 @@ def tune(prob, reps: int = 20, warmup: int = 5, stream=None, store: bool = True,
     best = min(table, key=lambda r: r["us"])
     choice = {k: best[k] for k in ("apply_kernel", "tile_rows", "tile_dpt")}
     if store:
-        _store(_key(prob.dim, prob.m), {"choice": choice, "n": int(prob.n), "table": table})
+        _store((_key(prob.dim, prob.m), _size_key(prob.dim, prob.m, prob.n)),
+               {"choice": choice, "n": int(prob.n), "table": table, "kernels": kernel_version()})
     return choice, table
 
 
 def tuned_options(prob, **kw) -> dict:
-    """The cached choice for (prob.dim, prob.m); tunes on `prob` first when
-    the cache has none."""
-    hit = load_cache().get(_key(prob.dim, prob.m))
-    if hit:
+    """The cached choice for (prob.dim, prob.m) and prob's size; tunes on `prob` first, the automatic choice
+    included, when the cache has none that was timed on the present kernels."""
+    hit = load_cache().get(_size_key(prob.dim, prob.m, prob.n))
+    if hit and hit.get("kernels") == kernel_version():
         return dict(hit["choice"])
+    kw.setdefault("cands", [AUTOMATIC] + candidates(prob.m))
     return tune(prob, **kw)[0]
 
 
@@ -134,4 +161,4 @@ def problem_key(prob) -> str:
     return _key(prob.dim, prob.m)
 
 
-__all__ = ["candidates", "tune", "tuned_options", "time_apply", "cache_path", "load_cache", "problem_key"]
+__all__ = ["AUTOMATIC", "candidates", "kernel_version", "tune", "tuned_options", "time_apply", "cache_path", "load_cache", "problem_key"]
