@@ -93,11 +93,10 @@ typedef struct {
                               e.g. 3D, whose halos leave room for few directions per chunk);
                               default 0 */
     int tile_rows;         /* row tiles: rows per tile, 32 or 64 (apply_kernel 2, 3), 4, 8, 16 or
-                              32 (apply_kernel 4); 0 = by the problem's size (automatic choice), 64, or
-                              in gather mode the most rows that keep a CTA at or below 320 (row,
-                              direction group) tasks */
-    int tile_dpt;          /* row tiles: directions per thread, 4 or 8 (must divide m); 0 = 4, with an
-                              explicit apply_kernel 2 or 3 8 when m % 8 == 0 */
+                              32 (apply_kernel 4); 0 = by the problem's size (automatic choice and
+                              gather mode), else 64.  With the automatic choice in 3D a number given
+                              here asks for staged tiles where their halo takes at most two chunks */
+    int tile_dpt;          /* row tiles: directions per thread, 4 or 8 (must divide m); 0 = 4 */
     int outer_precond;     /* outer GMRES on Phi: 0 = none (the paper's), 1 = DSA-like diffusion
                               correction, right preconditioner I + C^-1 Ms with the P1-diffusion
                               operator C = diag(1/(3 sigma_t,i)) sum_a K_aa + kappa M0 + Mt - Ms

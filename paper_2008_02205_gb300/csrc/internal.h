@@ -224,6 +224,7 @@ struct mlpg_ctx {
     int tile_ks = 1;            // warp groups that share a tile's slots
     bool tile_mma = false;      // the tensor-core variant of the tiled apply (apply_kernel 3)
     bool tile_gather = false;   // tiles with X read from global memory, no staged halo (apply_kernel 4)
+    bool tile_single = false;   // gather mode with single rows instead of row pairs
     int64_t ntile = 0, nslot = 0;
     size_t tile_smem = 0;       // dynamic shared memory of the tiled kernel: halo rows + record stages
     int tile_xs_f4 = 0;         // float4 words of the staged halo (the record stages follow)

@@ -655,10 +655,18 @@ __device__ __forceinline__ f32x2 pair_combine(const f32x2 *a, const f32x2 *o) {
 
 constexpr int kPairStages = 3;
 constexpr int kPairMaxThreads = 320;
-constexpr int kPairMaxWarps = kPairMaxThreads / 32;
+constexpr int kPairMaxThreads3 = 640;  // 3D gather with four directions per thread: the slots' split may double it
+constexpr int kPairMaxWarps = kPairMaxThreads3 / 32;
 constexpr int kPairMinTiles = 304;     // tiles wanted: two per SM
 constexpr int kPairWarpsPerSm = 12;    // warps per SM below which warps share the slots of a tile
 __host__ __device__ constexpr int pair_min_blocks(int d, int dpt) { return dpt == 8 ? 1 : (d == 2 ? 3 : 2); }
+// the launch bound: the same registers a thread for all four-direction kernels of a dimension
+__host__ __device__ constexpr int pair_threads(int d, int dpt, bool gx) {
+    return d == 3 && gx && dpt == 4 ? kPairMaxThreads3 : kPairMaxThreads;
+}
+__host__ __device__ constexpr int pair_blocks(int d, int dpt, bool gx) {
+    return pair_min_blocks(d, dpt) * kPairMaxThreads / pair_threads(d, dpt, gx);
+}
 // the most pairs that the 32 lanes of one warp of a tile belong to
 static int pairs_per_warp(int TP, int G) {
     int most = 1;
@@ -682,7 +690,7 @@ __device__ __noinline__ float own_row_sum(const int32_t *rowptr, const int32_t *
 
 // tile header: first slot, slots per pair (unused here), halo range
 template <int D, int DPT, bool GX, bool UA>
-__global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_spmm32_pair(
+__global__ void __launch_bounds__(pair_threads(D, DPT, GX), pair_blocks(D, DPT, GX)) k_spmm32_pair(
     int m, int mc, int G, int TP, int KS, int xs, int hx_f4, int ppw, const int4 *__restrict__ head,
     const int32_t *__restrict__ plen, const int2 *__restrict__ trow, const int32_t *__restrict__ hcol,
     const float4 *__restrict__ rec, const float *__restrict__ coef32, const int32_t *__restrict__ bptr,
@@ -917,6 +925,125 @@ __global__ void __launch_bounds__(kPairMaxThreads, pair_min_blocks(D, DPT)) k_sp
             }
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// Gather mode with single rows, 3D, at most 40 directions: one CTA per 32 rows, thread (s, g) owns row s and
+// the directions 4g .. 4g + 3.  The tile's records (a row's ten values and its column's offset, single-row
+// sliced-ELL slots) stream through kRecStages stages of kRowK entries, moved by bulk copies that thread 0
+// issues; two directions share a packed FMA.
+//
+// Why beside the row pairs: few directions leave these a handful of warps per SM (24^3 x 24: ten), whose
+// chains of entries then decide, and a row per thread has twice the threads.  Single rows against row pairs (us):
+// 20^3 x 24 70 against 97, 24^3 x 24 89 against 118, 20^3 x 40 91 against 110, 20^3 x 8 73 against 87; but 24^3 x 40
+// 153 against 134, 10^3 x 24 47 against 39, 16^3 x 8 51 against 43.  So single rows from kRowMinPoints points (kRowMinFew
+// for fewer than 24 directions) up to kRowMaxValues values of X.
+// ---------------------------------------------------------------------------
+constexpr int kRowTile = 32, kRowK = 8, kRowMaxDirs = 40;
+constexpr int64_t kRowMinPoints = 1536, kRowMinFew = 5000, kRowMaxValues = 360000;   // kRowMinFew: fewer than 24 directions
+template <int D>
+__global__ void __launch_bounds__(kRowTile * kRowMaxDirs / 4, 2) k_spmm32_row(
+    int m, const int32_t *__restrict__ base, const int32_t *__restrict__ width, const int32_t *__restrict__ trow,
+    const float4 *__restrict__ rec, const float *__restrict__ coef32, const int32_t *__restrict__ bptr,
+    const int32_t *__restrict__ boff, const float *__restrict__ bval, int64_t nb, const int32_t *rowptr,
+    const int32_t *col, const float *A32, int64_t nnz, const float *__restrict__ X, const float *__restrict__ B,
+    float *__restrict__ Y, int *__restrict__ err) {
+    constexpr int K = NA<D>(), RW4 = rec_words<D>() / 4, NS = kRecStages, SF4 = kRowK * kRowTile * RW4;
+    constexpr uint32_t SBYTES = SF4 * 16u;
+    extern __shared__ float4 smem_x4[];   // [NS][kRowK][kRowTile][RW4]
+    __shared__ __align__(8) uint64_t bars[NS];
+    const int t = blockIdx.x, G = m / 4, s = threadIdx.x / G, d = 4 * (threadIdx.x - s * G);
+    const int nst = width[t] / kRowK;
+    const float4 *rg = rec + (int64_t)base[t] * RW4;
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < NS; ++b) mbar_init(&bars[b], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        fence_proxy_async();
+        for (int st = 0; st < NS && st < nst; ++st) {
+            mbar_expect(&bars[st], SBYTES);
+            bulk_g2s(smem_x4 + st * SF4, rg + (int64_t)st * SF4, SBYTES, &bars[st]);
+        }
+    }
+    f32x2 c[K][2], acc[2];   // coefficients and sums of two directions each; c[0] is 1
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int k = 1; k < K; ++k) c[k][h] = pack2(coef32[16 * (d + 2 * h) + k], coef32[16 * (d + 2 * h + 1) + k]);
+        acc[h] = pack2(0.0f, 0.0f);
+    }
+    __syncthreads();
+    const float *Xd = X + d;
+    bool ok = true;
+    int st = 0;
+    for (; st < nst; ++st) {
+        const int b = st % NS;
+        ok = __syncthreads_and(mbar_wait(&bars[b], (st / NS) & 1));
+        if (!ok) break;
+        const float4 *rb = smem_x4 + b * SF4 + s * RW4;
+#pragma unroll
+        for (int kk = 0; kk < kRowK; ++kk) {
+            float a[4 * RW4];
+#pragma unroll
+            for (int q = 0; q < RW4; ++q) {
+                const float4 v = rb[kk * kRowTile * RW4 + q];
+                a[4 * q] = v.x; a[4 * q + 1] = v.y; a[4 * q + 2] = v.z; a[4 * q + 3] = v.w;
+            }
+            const float4 x = __ldg(reinterpret_cast<const float4 *>(Xd + __float_as_int(a[K])));
+            f32x2 v0 = pack2(a[0], a[0]), v1 = v0;
+#pragma unroll
+            for (int k = 1; k < K; ++k) {
+                const f32x2 ak = pack2(a[k], a[k]);
+                v0 = fma2(c[k][0], ak, v0);
+                v1 = fma2(c[k][1], ak, v1);
+            }
+            acc[0] = fma2(v0, pack2(x.x, x.y), acc[0]);
+            acc[1] = fma2(v1, pack2(x.z, x.w), acc[1]);
+        }
+        // the stage's reads (generic proxy) before the bulk copy that refills it (async proxy)
+        fence_proxy_async();
+        __syncthreads();
+        if (threadIdx.x == 0 && st + NS < nst) {
+            mbar_expect(&bars[b], SBYTES);
+            bulk_g2s(smem_x4 + b * SF4, rg + (int64_t)(st + NS) * SF4, SBYTES, &bars[b]);
+        }
+    }
+    if (!ok) {   // (block-uniform) report, let the copies in flight land, leave
+        if (threadIdx.x == 0) {
+            atomicOr(err, 1);
+            for (int k = st; k < nst && k < st + NS; ++k) mbar_wait(&bars[k % NS], (k / NS) & 1);
+        }
+        __syncthreads();
+        return;
+    }
+    const int32_t row = trow[(int64_t)t * kRowTile + s];
+    if (row < 0) return;
+    float res[4];
+    unpack2(acc[0], res[0], res[1]);
+    unpack2(acc[1], res[2], res[3]);
+    // padding slots add a zero times X of point 0: a sum that is not finite is taken again without them
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (!isfinite(res[j])) res[j] = own_row_sum<D>(rowptr, col, A32, nnz, coef32, X, m, row, d + j);
+    // outflow-face terms of a boundary row: sum_f max(Omega . n_f, 0) (S_f X)_i
+    const int32_t q1 = bptr[row + 1];
+    for (int32_t q = bptr[row]; q < q1; ++q) {
+        const float4 x = *reinterpret_cast<const float4 *>(Xd + boff[q]);
+        const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float v = 0.0f;
+#pragma unroll
+            for (int f = 0; f < NF<D>(); ++f) v = fmaf(coef32[16 * (d + j) + face_slot<D>() + f], bval[f * nb + q], v);
+            res[j] = fmaf(v, xv[j], res[j]);
+        }
+    }
+    const int64_t e = (int64_t)row * m + d;
+    float4 o = make_float4(res[0], res[1], res[2], res[3]);
+    if (B) {
+        const float4 bv = *reinterpret_cast<const float4 *>(B + e);
+        o = make_float4(bv.x - o.x, bv.y - o.y, bv.z - o.z, bv.w - o.w);
+    }
+    *reinterpret_cast<float4 *>(Y + e) = o;
 }
 
 __global__ void k_brows(int64_t n, const int32_t *__restrict__ bptr, int32_t *__restrict__ brow,
@@ -1703,6 +1830,19 @@ static int pair_split(int64_t ctas, int TP, int G, int width) {
         ks *= 2;
     return ks;
 }
+// The same in 3D with four directions per thread, whose warps are few and bound by their chains of entries: the
+// largest split whose CTAs, at 96 registers a thread, are all resident at once (10^3 x 168: three groups 64 us, the
+// four that need a second wave 74; 12^3 x 80 70 -> 57 with three, 8^3 x 168 57 -> 35 with six)
+static int wave_split(int64_t ctas, int TP, int G, int width) {
+    const int w1 = (TP * G + 31) / 32, sms = 152;
+    int best = 1;
+    for (int ks : {2, 3, 4, 6, 8, 12}) {
+        const int threads = ks * w1 * 32;
+        if (threads > kPairMaxThreads3 || width / (4 * ks) < 3 || (ctas + sms - 1) / sms > kPairMaxThreads3 / threads) break;
+        best = ks;
+    }
+    return best;
+}
 // shared memory of the warps' rings, or of the partial sums of the split, which reuse it
 template <int D>
 static size_t ring_bytes(int TP, int G, int dpt, int ks) {
@@ -1737,7 +1877,18 @@ static mlpg_status mma_attr(mlpg_ctx *ctx) {
 }
 
 template <int D>
+static mlpg_status launch_row(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
+    k_spmm32_row<D><<<(unsigned)ctx->ntile, kRowTile * (ctx->m / 4), ctx->tile_smem, ctx->stream>>>(
+        ctx->m, ctx->t_base, ctx->t_width, ctx->t_row, reinterpret_cast<const float4 *>(ctx->t_rec), ctx->coef32, ctx->bptr,
+        ctx->t_bhalo, ctx->bval32, ctx->nb, ctx->rowptr, ctx->col, ctx->A32, ctx->nnz, X, B, Y, ctx->d_tile_err);
+    CU_LAUNCH(ctx);
+    return MLPG_OK;
+}
+
+template <int D>
 static mlpg_status run_tile(mlpg_ctx *ctx, const float *X, const float *B, float *Y) {
+    if constexpr (D == 3)
+        if (ctx->tile_single) return launch_row<D>(ctx, X, B, Y);
     if (ctx->tile_mma) {
         if (ctx->tile_rows == 32) { MMA_NT_SWITCH(D, 32, launch_mma, ctx, X, B, Y) }
         MMA_NT_SWITCH(D, 64, launch_mma, ctx, X, B, Y)
@@ -1762,9 +1913,10 @@ struct TilePlan {
     std::string err;
     int tr = 0, dpt = 0, chunk = 0, ks = 1;
     bool gather = false, mma = false;
+    bool single = false;   // k_spmm32_row
     size_t rec_smem = 0;
-    TileLayout tl;
-    PairTileLayout pl;
+    TileLayout tl;         // single rows (mma, single)
+    PairTileLayout pl;     // row pairs
     int64_t nslot = 0, max_halo = 0;
 };
 
@@ -1779,26 +1931,25 @@ static void plan_mode(const mlpg_ctx *ctx, const std::vector<int32_t> &order, bo
     auto refuse = [&P](const char *why) { P.err = why; };
     P.gather = gather;
     P.mma = mma;
-    // m no multiple of four: staged value by value.  The automatic choice takes four directions per thread:
-    // eight measured slower at every size (256^2 S8: 69.3 against 60.8 us; more registers, fewer warps)
-    const int dpt = (m & 3) != 0 ? 4 : (ctx->opt.tile_dpt ? ctx->opt.tile_dpt : ((m & 7) == 0 && !gather && (ask || mma) ? 8 : 4));
+    // m no multiple of four: staged value by value.  Four directions per thread unless the caller names eight,
+    // which measured slower at every size (more registers, fewer warps)
+    const int dpt = (m & 3) != 0 ? 4 : (ctx->opt.tile_dpt ? ctx->opt.tile_dpt : ((m & 7) == 0 && mma ? 8 : 4));
     if ((m & 3) == 0 && m % dpt != 0) return refuse("tile_dpt must divide the number of directions");
     int tr = ctx->opt.tile_rows;
-    if (tr == 0 && !ask) {
+    if (tr == 0 && (!ask || gather)) {
         // gather: the most rows per tile (X rows shared through the L1) that keep a CTA at or below
         // kPairMaxThreads; staged: 64 rows (the smallest halo per row), fewer while that leaves SMs without a tile
         const int G = (m + dpt - 1) / dpt;
         tr = gather ? 32 : 64;
         while (tr > 4 && gather && tr / 2 * G > kPairMaxThreads) tr /= 2;
         while (tr > (gather ? 4 : 8) && (ctx->n + tr - 1) / tr < kPairMinTiles) tr /= 2;
-    }
-    if (gather && tr == 0) {   // the most rows per tile with at most 320 (row, direction group) tasks
-        const int G = (m + dpt - 1) / dpt;
-        tr = 4;
-        for (int c : {32, 16, 8})
-            if (c * G <= 320) {
-                tr = c;
-                break;
+        if (D == 3 && gather)   // better one CTA on most SMs, its slots split over many warps (13^3 x 80: 70 -> 54 us)
+            for (int c : {16, 8}) {
+                const int64_t tiles = (ctx->n + c - 1) / c;
+                if (c > tr && tiles >= 96 && tiles <= 152 && c / 2 * G <= kPairMaxThreads) {
+                    tr = c;
+                    break;
+                }
             }
     }
     if (tr == 0) tr = 64;
@@ -1833,9 +1984,10 @@ static void plan_mode(const mlpg_ctx *ctx, const std::vector<int32_t> &order, bo
         const int G = (m + dpt * nchunk - 1) / (dpt * nchunk);
         if (ask ? G > tile_max_groups(tr, dpt, gather) : tr / 2 * G > kPairMaxThreads) continue;
         const int64_t nch = (m + G * dpt - 1) / (G * dpt);
-        P.ks = pair_split(P.pl.ntile * nch, tr / 2, G, P.pl.max_width);
+        P.ks = D == 3 && gather && dpt == 4 ? wave_split(P.pl.ntile * nch, tr / 2, G, P.pl.max_width)
+                                            : pair_split(P.pl.ntile * nch, tr / 2, G, P.pl.max_width);
         const size_t halo = gather ? 0 : (size_t)P.max_halo * (G * dpt + 4) * sizeof(float);
-        while (P.ks > 1 && halo + ring_bytes<D>(tr / 2, G, dpt, P.ks) > kTileSmem) P.ks /= 2;
+        while (P.ks > 1 && halo + ring_bytes<D>(tr / 2, G, dpt, P.ks) > kTileSmem) P.ks = (P.ks + 1) / 2;
         P.rec_smem = ring_bytes<D>(tr / 2, G, dpt, P.ks);
         if (halo + P.rec_smem <= kTileSmem) {
             chunk = G * dpt;
@@ -1853,9 +2005,21 @@ static void plan_apply(const mlpg_ctx *ctx, TilePlan &P) {
     std::vector<int32_t> order(ctx->n);
     spatial_order(ctx->n, D, ctx->h_x.data(), order.data());
     // automatic choice: 3D halos (some 700 rows for 32) leave room for few directions per chunk, and
-    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit.  A
-    // request for 64 rows, which gather mode does not take, still goes to the staged tiles.
-    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->opt.tile_rows != 64 && ctx->n * m < (int64_t(1) << 31);
+    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit.  Rows
+    // per tile that the caller names go to the staged tiles first.
+    const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->opt.tile_rows == 0 && ctx->n * m < (int64_t(1) << 31);
+    if (skip && ctx->opt.tile_dpt != 8 && m <= kRowMaxDirs && ctx->n >= (m < 24 ? kRowMinFew : kRowMinPoints) &&
+        ctx->n * m <= kRowMaxValues) {
+        P.gather = P.single = true;
+        P.tr = kRowTile;
+        P.dpt = 4;
+        P.nslot = build_tiles(ctx->n, ctx->h_rowptr.data(), ctx->h_col.data(), order.data(), P.tr, kRowK, P.tl);
+        P.max_halo = P.tl.max_halo;
+        for (int64_t e = 0; e < P.nslot; ++e) P.tl.lcol[e] = P.tl.perm[e] >= 0 ? ctx->h_col[P.tl.perm[e]] : 0;   // not the halo's index
+        P.rec_smem = (size_t)kRecStages * kRowK * kRowTile * (rec_words<D>() / 4) * sizeof(float4);
+        if (P.nslot * (int64_t)(rec_words<D>() / 4) < (int64_t(1) << 31)) P.chunk = m;
+        return;
+    }
     if (kind != 4 && !skip) {
         plan_mode<D>(ctx, order, false, kind == 3, P);
         if (!P.err.empty()) return;
@@ -1889,7 +2053,7 @@ static mlpg_status init_tiles(mlpg_ctx *ctx) {
     const TilePlan &P = *plan;
     if (P.chunk == 0) return MLPG_OK;
     const int tr = P.tr, chunk = P.chunk;
-    const bool gather = P.gather, mma = P.mma;
+    const bool gather = P.gather, mma = P.mma, rows = P.mma || P.single;   // rows: single-row slots
     const int64_t nslot = P.nslot;
     ctx->tile_rows = tr;
     ctx->tile_dpt = P.dpt;
@@ -1897,17 +2061,18 @@ static mlpg_status init_tiles(mlpg_ctx *ctx) {
     ctx->tile_chunk = chunk;
     ctx->tile_mma = mma;
     ctx->tile_gather = gather;
+    ctx->tile_single = P.single;
     // gather: the record index is the column's global offset col x m; otherwise the column's
     // staged row in shared memory, a padded row that spreads halo rows over the banks
     ctx->tile_xs = gather ? m : (mma ? chunk + (16 - chunk % 32 + 32) % 32 : chunk + 4);
     cudaStream_t s = ctx->stream;
-    const int64_t ntile = mma ? P.tl.ntile : P.pl.ntile;
-    const std::vector<int64_t> &base = mma ? P.tl.base : P.pl.base, &hptr = mma ? P.tl.hptr : P.pl.hptr;
-    const std::vector<int32_t> &row = mma ? P.tl.row : P.pl.row, &hcol = mma ? P.tl.hcol : P.pl.hcol;
+    const int64_t ntile = rows ? P.tl.ntile : P.pl.ntile;
+    const std::vector<int64_t> &base = rows ? P.tl.base : P.pl.base, &hptr = rows ? P.tl.hptr : P.pl.hptr;
+    const std::vector<int32_t> &row = rows ? P.tl.row : P.pl.row, &hcol = rows ? P.tl.hcol : P.pl.hcol;
     ctx->ntile = ntile;
     ctx->nslot = nslot;
     std::vector<int32_t> base32(base.begin(), base.end()), hptr32(hptr.begin(), hptr.end()), head(4 * ntile);
-    if (mma) {
+    if (rows) {
         MLPG_TRY(to_device(ctx, &ctx->t_base, base32));
         MLPG_TRY(to_device(ctx, &ctx->t_hptr, hptr32));
         MLPG_TRY(to_device(ctx, &ctx->t_width, P.tl.width));
@@ -1922,13 +2087,13 @@ static mlpg_status init_tiles(mlpg_ctx *ctx) {
     }
     MLPG_TRY(to_device(ctx, &ctx->t_hcol, hcol));
     MLPG_TRY(to_device(ctx, &ctx->t_row, row));
-    MLPG_TRY(to_device(ctx, &ctx->t_lcol, mma ? P.tl.lcol : P.pl.lcol));
-    MLPG_TRY(to_device(ctx, &ctx->t_perm, mma ? P.tl.perm : P.pl.perm0));
-    if (!mma) {
+    MLPG_TRY(to_device(ctx, &ctx->t_lcol, rows ? P.tl.lcol : P.pl.lcol));
+    MLPG_TRY(to_device(ctx, &ctx->t_perm, rows ? P.tl.perm : P.pl.perm0));
+    if (!rows) {
         MLPG_TRY(to_device(ctx, &ctx->t_perm1, P.pl.perm1));
         MLPG_TRY(to_device(ctx, &ctx->t_plen, P.pl.plen));
     }
-    MLPG_TRY(dalloc(ctx, &ctx->t_rec, nslot * (mma ? rec_words<D>() : group_f4<D>())));   // a group: group_f4 float4 for four slots
+    MLPG_TRY(dalloc(ctx, &ctx->t_rec, nslot * (rows ? rec_words<D>() : group_f4<D>())));   // a group: group_f4 float4 for four slots
     // halo offset (index x shared-memory row stride) of every boundary-segment entry's column
     std::vector<int32_t> bptr(ctx->n + 1), bcol(std::max<int64_t>(ctx->nb, 1)), bhalo(std::max<int64_t>(ctx->nb, 1), 0);
     CU(ctx, cudaMemcpyAsync(bptr.data(), ctx->bptr, (ctx->n + 1) * 4, cudaMemcpyDeviceToHost, s));
@@ -1957,6 +2122,8 @@ static mlpg_status init_tiles(mlpg_ctx *ctx) {
             MMA_NT_SWITCH(D, 64, mma_attr, ctx)
         };
         MLPG_TRY(set());
+    } else if (P.single) {
+        CU(ctx, cudaFuncSetAttribute(k_spmm32_row<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem));
     } else {
         MLPG_TRY((pair_attr<D, 8, true, false>(ctx)));
         MLPG_TRY((pair_attr<D, 4, true, false>(ctx)));
@@ -2065,7 +2232,7 @@ static mlpg_status form_operators_d(mlpg_ctx *ctx, double kappa) {
     CU_LAUNCH(ctx);
     if (ctx->t_rec) {
         const int64_t gr = (ctx->nslot + 255) / 256;
-        if (ctx->tile_mma)
+        if (ctx->tile_mma || ctx->tile_single)
             k_tile_records<D><<<gr, 256, 0, s>>>(ctx->nslot, nnz, ctx->tile_xs, ctx->t_perm, ctx->t_lcol, ctx->A32,
                                                  reinterpret_cast<float4 *>(ctx->t_rec));
         else

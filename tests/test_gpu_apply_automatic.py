@@ -46,8 +46,9 @@ CASES = [
     (2, 30, 12, 80, 64, 2, True),   # two equal chunks
     (3, 5, 8, 27, 0, 2, False),     # staged tiles in 3D
     (3, 6, 4, 23, 0, 2, False),
-    (3, 6, 4, 24, 0, 4, False),     # gather mode
-    (3, 6, 4, 24, 32, 4, False),
+    (3, 6, 4, 24, 0, 4, False),     # gather mode, row pairs
+    (3, 12, 4, 24, 0, 4, False),    # gather mode, single rows
+    (3, 6, 4, 24, 32, 2, False),
     (3, 6, 4, 24, 64, 2, False),    # gather mode takes at most 32 rows: staged tiles
 ]
 
@@ -94,7 +95,7 @@ def test_applies_back_to_back_read_each_others_output(dim, side, sn, m):
 
 
 @pytest.mark.parametrize("kernel", [0, 2, 4])
-@pytest.mark.parametrize("dim,side,sn,m", [(2, 13, 4, 12), (2, 13, 4, 11), (2, 30, 8, 40), (3, 6, 4, 24), (3, 6, 4, 23)])
+@pytest.mark.parametrize("dim,side,sn,m", [(2, 13, 4, 12), (2, 13, 4, 11), (2, 30, 8, 40), (3, 6, 4, 24), (3, 6, 4, 23), (3, 12, 4, 24)])
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 def test_non_finite_values_stay_in_their_rows(dim, side, sn, m, kernel, value):
     """A NaN or an infinity at one point and direction reaches the rows whose pattern holds the point, in that
