@@ -242,7 +242,7 @@ __global__ void k_scan1(int64_t n, const int *__restrict__ in, int32_t *__restri
 // memory.  Lanes that split a row's entries and add their parts by shuffles spent
 // a seventh of that time on the additions (54.7 us); here every lane's operation is
 // a product of the sum.  SPLIT > 1: that many lanes share a row's entries, for problems
-// too small to fill the chip, where the chain of loads decides.
+// too small to fill the chip, where the chain of loads decides (spmm64_split).
 template <int SPLIT>
 __global__ void __launch_bounds__(256) k_spmm64(int64_t total, int m, const int32_t *__restrict__ rowptr,
                                                 const int32_t *__restrict__ col, const double *__restrict__ L64,
@@ -2336,17 +2336,32 @@ static void timing_end(mlpg_ctx *ctx) {
     ctx->ev_used++;
 }
 
-// values below which four lanes share a row: one thread per value leaves fewer than 16 warps per SM
-constexpr int64_t kSpmm64Split = 152 * 512;
-mlpg_status apply_L64_res(mlpg_ctx *ctx, const double *X, const double *B, double *Y) {
+// Lanes that share a (row, direction) of the FP64 apply: with one thread for each the chain of a row's loads
+// decides when there are few of them, and the longer the rows (200 entries in 3D, 45 in 2D) the more of them it
+// takes.  At least eight entries a lane; eight and more lanes only for the smallest problems.  us with
+// 1 / 2 / 4 / 8 lanes: 2D 64^2 x 13 12.9 / 10.3 / 12.3 / 14.4, 32^2 x 12 12.3 / 8.3 / 6.2 / 6.2, 64^2 x 40
+// 21.9 / 21.6 / 24.6 / 32.1; 3D 16^3 x 24 95.7 / 67.5 / 56.3 / 58.0, 20^3 x 24 103 / 108 / 94 / 102, 10^3 x 27
+// 39.0 / 26.7 / 18.5 / 18.5, 16^3 x 80 146 / 138 / 141 / 166; 10^3 x 1 43 / 27 / 16 / 11, 8 with sixteen.
+static int spmm64_split(int64_t total, int64_t len) {
+    for (int s : {16, 8, 4, 2})
+        if (len >= 8 * s && total * s <= (s == 16 ? 100000 : (s == 8 ? 250000 : 3700 * len))) return s;
+    return 1;
+}
+template <int SPLIT>
+static void launch_spmm64(mlpg_ctx *ctx, const double *X, const double *B, double *Y) {
     const int64_t total = ctx->n * ctx->m;
+    k_spmm64<SPLIT><<<(unsigned)((total * SPLIT + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col,
+                                                                                     ctx->L64, X, B, Y);
+}
+mlpg_status apply_L64_res(mlpg_ctx *ctx, const double *X, const double *B, double *Y) {
     timing_begin(ctx);
-    if (total < kSpmm64Split)
-        k_spmm64<4><<<(unsigned)((total * 4 + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col,
-                                                                                 ctx->L64, X, B, Y);
-    else
-        k_spmm64<1><<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(total, ctx->m, ctx->rowptr, ctx->col,
-                                                                             ctx->L64, X, B, Y);
+    switch (spmm64_split(ctx->n * ctx->m, ctx->nnz / ctx->n)) {
+        case 16: launch_spmm64<16>(ctx, X, B, Y); break;
+        case 8: launch_spmm64<8>(ctx, X, B, Y); break;
+        case 4: launch_spmm64<4>(ctx, X, B, Y); break;
+        case 2: launch_spmm64<2>(ctx, X, B, Y); break;
+        default: launch_spmm64<1>(ctx, X, B, Y);
+    }
     timing_end(ctx);
     CU_LAUNCH(ctx);
     return MLPG_OK;
