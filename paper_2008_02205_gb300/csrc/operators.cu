@@ -658,6 +658,7 @@ constexpr int kPairMaxThreads = 320;
 constexpr int kPairMaxThreads3 = 640;  // 3D gather with four directions per thread: the slots' split may double it
 constexpr int kPairMaxWarps = kPairMaxThreads3 / 32;
 constexpr int kPairMinTiles = 304;     // tiles wanted: two per SM
+constexpr int64_t kOddMaxPoints = 6500, kOddMinLarge = 10000, kOddMaxChunked = 150000;   // 3D, m no multiple of four (plan_apply)
 constexpr int kPairWarpsPerSm = 12;    // warps per SM below which warps share the slots of a tile
 __host__ __device__ constexpr int pair_min_blocks(int d, int dpt) { return dpt == 8 ? 1 : (d == 2 ? 3 : 2); }
 // the launch bound: the same registers a thread for all four-direction kernels of a dimension
@@ -2026,6 +2027,14 @@ static void plan_apply(const mlpg_ctx *ctx, TilePlan &P) {
         // staged halos pay while the records are read by few chunks; past two chunks the gather
         // mode reads them once
         if (kind == 0 && P.chunk && (m + P.chunk - 1) / P.chunk > 2) P.chunk = 0;
+        // 3D and m no multiple of four, where there is no gather mode: the row teams (us) are ahead on large sets
+        // (20^3 x 27 136 against 158, 24^3 x 27 221 against 269, 20^3 x 6 74 against 92) and with two chunks on
+        // middling ones (16^3 x 78 195 against 221), the tiles before (18^3 x 27 103 against 98, 16^3 x 27 77 against
+        // 64, 15^3 x 42 118 against 99, 8^3 x 78 111 against 41) and for few directions beyond (24^3 x 13 192 against 169)
+        if (kind == 0 && D == 3 && (m & 3) != 0 &&
+            ((P.chunk < m && ctx->n * m > kOddMaxChunked) ||
+             (ctx->n > kOddMaxPoints && !(m <= 16 && ctx->n >= kOddMinLarge))))
+            P.chunk = 0;
     }
     if (kind == 4 || (kind == 0 && P.chunk == 0 && (m & 3) == 0)) plan_mode<D>(ctx, order, true, false, P);
 }
