@@ -141,7 +141,7 @@ class ClockSampler:
 PROFILE = os.path.join(ROOT, "profiles", "k_spmm32_pair.md")
 APPLY_KERNELS = {1: "k_spmm32 (row teams)", 2: "k_spmm32_pair (row-pair tiles, TMA-staged)",
                  3: "k_spmm32_mma (row tiles, tensor cores)",
-                 4: "k_spmm32_pair (row-pair tiles, gather mode)"}
+                 4: "k_spmm32_pair / k_spmm32_row (row tiles, gather mode)"}
 KERNEL_SRC = os.path.join(ROOT, "paper_2008_02205_gb300", "csrc", "operators.cu")
 # FP32 FMA peak of the GB300 (TFMA/s): 152 SMs x 128 FP32 lanes x 2.07 GHz maximum SM clock
 FP32_FMA_PEAK_T = 152 * 128 * 2.07e9 / 1e12

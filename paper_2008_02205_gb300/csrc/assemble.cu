@@ -136,7 +136,8 @@ template <int ORD>
 __device__ uint64_t rk_point_gen(double px, double py, double s, int S, const double *fx, const double *fy,
                                  const double *fR2, const double *finvh, const double *fV, double *U, double *Ux,
                                  double *Uy, int stride) {
-    constexpr int NP = ORD == 0 ? 1 : (ORD == 1 ? 3 : 6);
+    static_assert(ORD == 0 || ORD == 2, "the linear functions have kernels of their own");
+    constexpr int NP = ORD == 0 ? 1 : 6;
     double M[NP][NP], Dx[NP][NP], Dy[NP][NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i)
@@ -147,11 +148,9 @@ __device__ uint64_t rk_point_gen(double px, double py, double s, int S, const do
     auto basis = [&](double dx, double dy, double *P, double *Px, double *Py) {
         const double ex = dx * is, ey = dy * is;
         P[0] = 1.0; Px[0] = 0.0; Py[0] = 0.0;
-        if (ORD >= 1) {
+        if constexpr (ORD == 2) {
             P[1] = ex; Px[1] = is; Py[1] = 0.0;
             P[2] = ey; Px[2] = 0.0; Py[2] = is;
-        }
-        if (ORD >= 2) {
             P[3] = ex * ex; Px[3] = 2.0 * ex * is; Py[3] = 0.0;
             P[4] = ex * ey; Px[4] = ey * is; Py[4] = ex * is;
             P[5] = ey * ey; Px[5] = 0.0; Py[5] = 2.0 * ey * is;

@@ -230,7 +230,7 @@ struct mlpg_ctx {
     int tile_xs_f4 = 0;         // float4 words of the staged halo (the record stages follow)
     int64_t tile_max_halo = 0;  // largest halo of a tile
     int *d_tile_err = nullptr;  // set by a tile-kernel wait that gave up (bounded waits)
-    int32_t *t_head = nullptr;   // [ntile][4]: first slot, slots per pair, halo range (row pairs)
+    int32_t *t_head = nullptr;   // [ntile][4]: first slot, (unused), halo range (row pairs)
     int32_t *t_base = nullptr, *t_width = nullptr, *t_row = nullptr, *t_hptr = nullptr, *t_hcol = nullptr;
     int32_t *t_perm = nullptr, *t_perm1 = nullptr, *t_lcol = nullptr, *t_plen = nullptr;   // t_perm1, t_plen: row pairs
     int32_t *t_bhalo = nullptr;  // [nb]: halo offset (index x tile_xs) of each boundary-segment entry's column

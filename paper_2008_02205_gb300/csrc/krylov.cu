@@ -513,10 +513,9 @@ __global__ void k_givens(int M, int R, int j, int G, const double *__restrict__ 
 // and move 32-byte sectors of whole rows.  The line: points (times the problems that
 // mlpg_step_batch runs at once, which fill the chip themselves) up to kGsRows32 in FP32,
 // kGsRows64 in FP64, whose sums keep the few FP64 units of a cluster's SMs busy.  Whole
-// steps, separate -> one launch (ms): FP32 32^2 S4 11.4 -> 7.9, 75^2 S6 22.9 -> 18.4,
-// 128^2 S8 25.7 -> 21.8, 180^2 S8 37.7 -> 38.5; 3D 20^3 S8 92.5 -> 86.9; FP64 32^2 S4
-// 28.8 -> 21.2, 64^2 S8 172 -> 167, 96^2 S8 324 -> 362.  Eight problems of 1k to 16k points
-// at once: 57.0 with separate passes, 60.8 in one launch.
+// steps, separate -> one launch (ms): FP32 32^2 S4 9.6 -> 7.6, 75^2 S6 20.7 -> 18.8, 128^2 S8 22.8 -> 21.8,
+// 180^2 S8 34.2 -> 38.1; 3D 20^3 S8 87.8 -> 86.6; FP64 32^2 S4 28.8 -> 21.2, 64^2 S8 168 -> 156,
+// 96^2 S8 320 -> 329.  Eight problems of 1k to 16k points at once: 49 with separate passes, 60 in one launch.
 // ---------------------------------------------------------------------------
 constexpr int64_t kGsRows32 = 16384, kGsRows64 = 4096;
 constexpr int kGsGroup = 8;   // basis vectors per accumulator group

@@ -434,15 +434,10 @@ __global__ void __launch_bounds__(256) k_faces32(int64_t nbr, int m, int tm_log2
 }
 
 // ---------------------------------------------------------------------------
-// Row tiles (m % 4 == 0), shared by the CUDA-core and tensor-core tile
-// kernels.  A tile is TR rows in the spatial order; its halo is the sorted union
-// of their columns.  One CTA per (row tile, direction chunk) stages the halo
-// rows of X (mc of the m directions) in shared memory once, so a neighbour
-// row shared by several rows of the tile is read from HBM once per tile.  The
-// tile's entries are sliced-ELL records, entry k of row slot s at
-// [k][s] (width padded to a multiple of kRecK with zero records): the K
-// base-array values of the entry and the offset of its column's staged row,
-// padded to whole float4 words.
+// Single-row records, for the tensor-core tiles and the single-row gather kernel.  A tile is TR
+// rows in the spatial order; its entries are sliced-ELL records, entry k of row slot s at
+// [k][s] (width padded with zero records): the K base-array values of the entry and the offset
+// of its column's row (in the staged halo, or in X), padded to whole float4 words.
 // ---------------------------------------------------------------------------
 template <int D>
 __host__ __device__ constexpr int rec_words() { return (NA<D>() + 4) / 4 * 4; }   // K values + halo index, padded to float4
@@ -575,10 +570,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 // return path (a 16-byte load costs a warp 4 clocks, 2 when the lanes of each
 // even-odd pair share their address; 26 us); about 60 % of the issue slots are taken.
 // 3D: X through the L1 (272 directions: half of the 2 GB that 24^3 reads come from L2).
-// Before (one row per thread, CTA-wide record stages) and after, warm, back to back:
-//   2D  32^2 S4 14.4 -> 10.3 us, 100^2 S8 24.6 -> 20.6, 256^2 S8 80.5 -> 60.8,
-//       128^2 S12 63.8 -> 45.1, 181^2 with 14 directions (row teams before) 47.1 -> 23.9
-//   3D  8^3 S4 65.6 -> 28.8 us, 20^3 S8 154.6 -> 138.6, 24^3 x 272 759 -> 579
+// Before (one row per thread, CTA-wide record stages; row teams for 14 directions) and after, warm, back to
+// back:
+//   2D  32^2 S4 5.5 -> 3.0 us, 256^2 S8 60.8 -> 47.4, 181^2 with 14 directions 38.7 -> 13.9
+//   3D  8^3 S4 65 -> 26 us, 20^3 S8 155 -> 144, 24^3 x 272 758 -> 586; few directions: k_spmm32_row
 // Tried and not kept: the combination on mma.sync (FP16 parts) with the union of
 // 8 rows, whose legacy tensor path issues one m16n8k16 in about 64 clocks here (93 us at
 // 256^2 S8, 1.5 ms at 24^3 x 272); a producer warp with CTA-wide stages (66 us).
@@ -689,7 +684,7 @@ __device__ __noinline__ float own_row_sum(const int32_t *rowptr, const int32_t *
     return sum;
 }
 
-// tile header: first slot, slots per pair (unused here), halo range
+// tile header: first slot, (unused), halo range
 template <int D, int DPT, bool GX, bool UA>
 __global__ void __launch_bounds__(pair_threads(D, DPT, GX), pair_blocks(D, DPT, GX)) k_spmm32_pair(
     int m, int mc, int G, int TP, int KS, int xs, int hx_f4, int ppw, const int4 *__restrict__ head,
@@ -1444,8 +1439,8 @@ __global__ void __launch_bounds__(256) k_bjacobi_scalar(int64_t nblk, int m, con
 }
 
 // ---------------------------------------------------------------------------
-// Tiled FP32 L-apply on tensor cores (m % 8 == 0).  The same tiles, halo
-// staging and record pipeline as k_spmm32_tile; one warp per 16 row slots of
+// Tiled FP32 L-apply on tensor cores (m % 8 == 0).  The tile's halo rows of X and its records are staged in
+// shared memory by 16-byte cp.async, the records in a pipeline of kRecStages stages; one warp per 16 row slots of
 // the tile.  For each entry step k, the combination of the K base arrays with
 // the direction coefficients,
 //     V[s][d] = sum_k a_k(s, k) c_k(d)      (16 rows x 8 directions per n-tile),
@@ -2085,10 +2080,9 @@ static mlpg_status init_tiles(mlpg_ctx *ctx) {
         MLPG_TRY(to_device(ctx, &ctx->t_base, base32));
         MLPG_TRY(to_device(ctx, &ctx->t_hptr, hptr32));
         MLPG_TRY(to_device(ctx, &ctx->t_width, P.tl.width));
-    } else {   // tile headers: first slot, slots per pair, halo range
+    } else {   // tile headers: first slot, (unused), halo range
         for (int64_t t = 0; t < ntile; ++t) {
             head[4 * t] = base32[t];
-            head[4 * t + 1] = P.pl.width[t];
             head[4 * t + 2] = hptr32[t];
             head[4 * t + 3] = hptr32[t + 1];
         }
