@@ -573,7 +573,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 // Before (one row per thread, CTA-wide record stages; row teams for 14 directions) and after, warm, back to
 // back:
 //   2D  32^2 S4 5.5 -> 3.0 us, 256^2 S8 60.8 -> 47.4, 181^2 with 14 directions 38.7 -> 13.9
-//   3D  8^3 S4 65 -> 26 us, 20^3 S8 155 -> 144, 24^3 x 272 758 -> 586; few directions: k_spmm32_row
+//   3D  8^3 S4 65 -> 26 us, 20^3 S8 155 -> 144, 24^3 x 272 723 -> 533; few directions: k_spmm32_row
 // Tried and not kept: the combination on mma.sync (FP16 parts) with the union of
 // 8 rows, whose legacy tensor path issues one m16n8k16 in about 64 clocks here (93 us at
 // 256^2 S8, 1.5 ms at 24^3 x 272); a producer warp with CTA-wide stages (66 us).
