@@ -573,7 +573,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 // Before (one row per thread, CTA-wide record stages; row teams for 14 directions) and after, warm, back to
 // back:
 //   2D  32^2 S4 5.5 -> 3.0 us, 256^2 S8 60.8 -> 47.4, 181^2 with 14 directions 38.7 -> 13.9
-//   3D  8^3 S4 65 -> 26 us, 20^3 S8 155 -> 144, 24^3 x 272 723 -> 533; few directions: k_spmm32_row
+//   3D  8^3 S4 23 -> 15 us, 20^3 S8 115 -> 85, 24^3 x 272 721 -> 532; few directions: k_spmm32_row
 // Tried and not kept: the combination on mma.sync (FP16 parts) with the union of
 // 8 rows, whose legacy tensor path issues one m16n8k16 in about 64 clocks here (93 us at
 // 256^2 S8, 1.5 ms at 24^3 x 272); a producer warp with CTA-wide stages (66 us).
@@ -653,7 +653,7 @@ constexpr int kPairMaxThreads = 320;
 constexpr int kPairMaxThreads3 = 640;  // 3D gather with four directions per thread: the slots' split may double it
 constexpr int kPairMaxWarps = kPairMaxThreads3 / 32;
 constexpr int kPairMinTiles = 304;     // tiles wanted: two per SM
-constexpr int64_t kOddMaxPoints = 6500, kOddMinLarge = 10000, kOddMaxChunked = 150000;   // 3D, m no multiple of four (plan_apply)
+constexpr int64_t kOddMaxPoints = 2000, kOddMaxFew = 6500, kOddMinLarge = 10000, kOddMaxChunked = 150000;   // 3D, m no multiple of four (plan_apply)
 constexpr int kPairWarpsPerSm = 12;    // warps per SM below which warps share the slots of a tile
 __host__ __device__ constexpr int pair_min_blocks(int d, int dpt) { return dpt == 8 ? 1 : (d == 2 ? 3 : 2); }
 // the launch bound: the same registers a thread for all four-direction kernels of a dimension
@@ -930,10 +930,10 @@ __global__ void __launch_bounds__(pair_threads(D, DPT, GX), pair_blocks(D, DPT, 
 // issues; two directions share a packed FMA.
 //
 // Why beside the row pairs: few directions leave these a handful of warps per SM (24^3 x 24: ten), whose
-// chains of entries then decide, and a row per thread has twice the threads.  Single rows against row pairs (us):
-// 20^3 x 24 70 against 97, 24^3 x 24 89 against 118, 20^3 x 40 91 against 110, 20^3 x 8 73 against 87; but 24^3 x 40
-// 153 against 134, 10^3 x 24 47 against 39, 16^3 x 8 51 against 43.  So single rows from kRowMinPoints points (kRowMinFew
-// for fewer than 24 directions) up to kRowMaxValues values of X.
+// chains of entries then decide, and a row per thread has twice the threads.  Single rows against row pairs (us, warm,
+// back to back): 18^3 x 24 31 against 59, 20^3 x 24 35 against 45, 24^3 x 24 58 against 69, 15^3 x 40 32 against 38, 18^3 x 8
+// 36 against 59; but 24^3 x 40 98 against 79, 11^3 x 24 and below pairs, 13^3 x 8 23 against 22.  So single rows from
+// kRowMinPoints points (kRowMinFew for fewer than 24 directions) up to kRowMaxValues values of X.
 // ---------------------------------------------------------------------------
 constexpr int kRowTile = 32, kRowK = 8, kRowMaxDirs = 40;
 constexpr int64_t kRowMinPoints = 1536, kRowMinFew = 5000, kRowMaxValues = 360000;   // kRowMinFew: fewer than 24 directions
@@ -1818,26 +1818,15 @@ static mlpg_status launch_pair(mlpg_ctx *ctx, const float *X, const float *B, fl
     return MLPG_OK;
 }
 // Warp groups that share the slots of a tile: enough of them to give every SM kPairWarpsPerSm warps,
-// while a group keeps at least two groups of four slots and the CTA its thread limit
-static int pair_split(int64_t ctas, int TP, int G, int width) {
+// while a group keeps at least two groups of four slots and the CTA its thread limit.  Larger CTAs only where half
+// the SMs have none: they would keep the next apply's CTAs, launched early, off the SM (8^3 x 24, 128 CTAs: 14 us with
+// eight groups, 24 with twelve; 6^3 x 272, 54 CTAs: 20 with two, 16 with four)
+static int pair_split(int64_t ctas, int TP, int G, int width, int max_threads) {
     const int w1 = (TP * G + 31) / 32;
     int ks = 1;
-    while (2 * ks * w1 * 32 <= kPairMaxThreads && ctas * w1 * ks < (int64_t)kPairWarpsPerSm * 152 && width / (8 * ks) >= 2)
+    while (2 * ks * w1 * 32 <= max_threads && ctas * w1 * ks < (int64_t)kPairWarpsPerSm * 152 && width / (8 * ks) >= 2)
         ks *= 2;
     return ks;
-}
-// The same in 3D with four directions per thread, whose warps are few and bound by their chains of entries: the
-// largest split whose CTAs, at 96 registers a thread, are all resident at once (10^3 x 168: three groups 64 us, the
-// four that need a second wave 74; 12^3 x 80 70 -> 57 with three, 8^3 x 168 57 -> 35 with six)
-static int wave_split(int64_t ctas, int TP, int G, int width) {
-    const int w1 = (TP * G + 31) / 32, sms = 152;
-    int best = 1;
-    for (int ks : {2, 3, 4, 6, 8, 12}) {
-        const int threads = ks * w1 * 32;
-        if (threads > kPairMaxThreads3 || width / (4 * ks) < 3 || (ctas + sms - 1) / sms > kPairMaxThreads3 / threads) break;
-        best = ks;
-    }
-    return best;
 }
 // shared memory of the warps' rings, or of the partial sums of the split, which reuse it
 template <int D>
@@ -1939,14 +1928,6 @@ static void plan_mode(const mlpg_ctx *ctx, const std::vector<int32_t> &order, bo
         tr = gather ? 32 : 64;
         while (tr > 4 && gather && tr / 2 * G > kPairMaxThreads) tr /= 2;
         while (tr > (gather ? 4 : 8) && (ctx->n + tr - 1) / tr < kPairMinTiles) tr /= 2;
-        if (D == 3 && gather)   // better one CTA on most SMs, its slots split over many warps (13^3 x 80: 70 -> 54 us)
-            for (int c : {16, 8}) {
-                const int64_t tiles = (ctx->n + c - 1) / c;
-                if (c > tr && tiles >= 96 && tiles <= 152 && c / 2 * G <= kPairMaxThreads) {
-                    tr = c;
-                    break;
-                }
-            }
     }
     if (tr == 0) tr = 64;
     if (gather && tr == 64)
@@ -1980,8 +1961,12 @@ static void plan_mode(const mlpg_ctx *ctx, const std::vector<int32_t> &order, bo
         const int G = (m + dpt * nchunk - 1) / (dpt * nchunk);
         if (ask ? G > tile_max_groups(tr, dpt, gather) : tr / 2 * G > kPairMaxThreads) continue;
         const int64_t nch = (m + G * dpt - 1) / (G * dpt);
-        P.ks = D == 3 && gather && dpt == 4 ? wave_split(P.pl.ntile * nch, tr / 2, G, P.pl.max_width)
-                                            : pair_split(P.pl.ntile * nch, tr / 2, G, P.pl.max_width);
+        const int64_t ctas = P.pl.ntile * nch;
+        const bool wide = D == 3 && gather && dpt == 4;
+        P.ks = pair_split(ctas, tr / 2, G, P.pl.max_width, wide && 2 * ctas <= 152 && tr / 2 * G > 64 ? kPairMaxThreads3 : kPairMaxThreads);
+        // 3D gather: no second wave for the split's sake (96 registers a thread; 11^3 x 272 61 -> 49 us, 13^3 x 168
+        // 60 -> 51, 16^3 x 80 56 -> 50)
+        while (wide && P.ks > 1 && (ctas + 151) / 152 > kPairMaxThreads3 / (P.ks * ((tr / 2 * G + 31) / 32) * 32)) P.ks /= 2;
         const size_t halo = gather ? 0 : (size_t)P.max_halo * (G * dpt + 4) * sizeof(float);
         while (P.ks > 1 && halo + ring_bytes<D>(tr / 2, G, dpt, P.ks) > kTileSmem) P.ks = (P.ks + 1) / 2;
         P.rec_smem = ring_bytes<D>(tr / 2, G, dpt, P.ks);
@@ -2001,7 +1986,7 @@ static void plan_apply(const mlpg_ctx *ctx, TilePlan &P) {
     std::vector<int32_t> order(ctx->n);
     spatial_order(ctx->n, D, ctx->h_x.data(), order.data());
     // automatic choice: 3D halos (some 700 rows for 32) leave room for few directions per chunk, and
-    // gathering measured faster at every size (20^3 S8: 137 against 182 us); row teams past its limit.  Rows
+    // gathering measured faster at every size; row teams past its limit.  Rows
     // per tile that the caller names go to the staged tiles first.
     const bool skip = kind == 0 && D == 3 && (m & 3) == 0 && ctx->opt.tile_rows == 0 && ctx->n * m < (int64_t(1) << 31);
     if (skip && ctx->opt.tile_dpt != 8 && m <= kRowMaxDirs && ctx->n >= (m < 24 ? kRowMinFew : kRowMinPoints) &&
@@ -2023,12 +2008,12 @@ static void plan_apply(const mlpg_ctx *ctx, TilePlan &P) {
         // mode reads them once
         if (kind == 0 && P.chunk && (m + P.chunk - 1) / P.chunk > 2) P.chunk = 0;
         // 3D and m no multiple of four, where there is no gather mode: the row teams (us) are ahead on large sets
-        // (20^3 x 27 136 against 158, 24^3 x 27 221 against 269, 20^3 x 6 74 against 92) and with two chunks on
-        // middling ones (16^3 x 78 195 against 221), the tiles before (18^3 x 27 103 against 98, 16^3 x 27 77 against
-        // 64, 15^3 x 42 118 against 99, 8^3 x 78 111 against 41) and for few directions beyond (24^3 x 13 192 against 169)
+        // (15^3 x 27 44 against 61, 18^3 x 27 76 against 97, 24^3 x 27 187 against 210) and with two chunks on
+        // middling ones, the tiles before (9^3 x 27 21 against 15, 8^3 x 27 20 against 14; 13^3 x 27 30 against 34) and, for
+        // few directions, which waste the teams' lanes, up to 18^3 and from 22^3
+        const int64_t most = m <= 16 ? kOddMaxFew : kOddMaxPoints;
         if (kind == 0 && D == 3 && (m & 3) != 0 &&
-            ((P.chunk < m && ctx->n * m > kOddMaxChunked) ||
-             (ctx->n > kOddMaxPoints && !(m <= 16 && ctx->n >= kOddMinLarge))))
+            ((P.chunk < m && ctx->n * m > kOddMaxChunked) || (ctx->n > most && !(m <= 16 && ctx->n >= kOddMinLarge))))
             P.chunk = 0;
     }
     if (kind == 4 || (kind == 0 && P.chunk == 0 && (m & 3) == 0)) plan_mode<D>(ctx, order, true, false, P);
@@ -2340,15 +2325,15 @@ static void timing_end(mlpg_ctx *ctx) {
 }
 
 // Lanes that share a (row, direction) of the FP64 apply: with one thread for each the chain of a row's loads
-// decides when there are few of them, and the longer the rows (200 entries in 3D, 45 in 2D) the more of them it
-// takes.  At least eight entries a lane; eight and more lanes only for the smallest problems.  us with
-// 1 / 2 / 4 / 8 lanes: 2D 64^2 x 13 12.9 / 10.3 / 12.3 / 14.4, 32^2 x 12 12.3 / 8.3 / 6.2 / 6.2, 64^2 x 40
-// 21.9 / 21.6 / 24.6 / 32.1; 3D 16^3 x 24 95.7 / 67.5 / 56.3 / 58.0, 20^3 x 24 103 / 108 / 94 / 102, 10^3 x 27
-// 39.0 / 26.7 / 18.5 / 18.5, 16^3 x 80 146 / 138 / 141 / 166; 10^3 x 1 43 / 27 / 16 / 11, 8 with sixteen.
+// decides while they leave fewer than 16 warps per SM; beyond that the lanes' sums only cost.  us with 1 / 2 / 4 /
+// 8 lanes: 3D 8^3 x 80 31.2 / 22.1 / 15.4 / 14.8, 12^3 x 24 31.7 / 22.7 / 15.5 / 17.3, 12^3 x 40 32.9 / 25.4 / 24.1 /
+// 28.9, 18^3 x 24 50.5 / 52.5 / 54.7 / 64.5, 15^3 x 80 86.5 / 93.9 / 103 / 124; 2D 64^2 x 14 7.3 / 6.6 / 6.7 / 9.4.
+// Long rows and next to no threads take more (10^3 x 1: 16 us with four lanes, 8 with sixteen).
+constexpr int64_t kSpmm64Split = 152 * 512;
 static int spmm64_split(int64_t total, int64_t len) {
-    for (int s : {16, 8, 4, 2})
-        if (len >= 8 * s && total * s <= (s == 16 ? 100000 : (s == 8 ? 250000 : 3700 * len))) return s;
-    return 1;
+    if (total <= 2000 && len >= 128) return 16;
+    if (total <= 6000 && len >= 64) return 8;
+    return total < kSpmm64Split ? 4 : 1;
 }
 template <int SPLIT>
 static void launch_spmm64(mlpg_ctx *ctx, const double *X, const double *B, double *Y) {
@@ -2362,7 +2347,6 @@ mlpg_status apply_L64_res(mlpg_ctx *ctx, const double *X, const double *B, doubl
         case 16: launch_spmm64<16>(ctx, X, B, Y); break;
         case 8: launch_spmm64<8>(ctx, X, B, Y); break;
         case 4: launch_spmm64<4>(ctx, X, B, Y); break;
-        case 2: launch_spmm64<2>(ctx, X, B, Y); break;
         default: launch_spmm64<1>(ctx, X, B, Y);
     }
     timing_end(ctx);

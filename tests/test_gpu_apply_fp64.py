@@ -1,4 +1,4 @@
-"""The FP64 transport-operator apply with 1, 2, 4, 8 and 16 lanes per (row, direction), at the sizes that each
+"""The FP64 transport-operator apply with 1, 4, 8 and 16 lanes per (row, direction), at the sizes that each
 serves, against the oracle's L_m.  The operators' forms agree to 1e-11 of their largest entry (the form tests)."""
 import numpy as np
 import pytest
